@@ -373,6 +373,7 @@ constexpr size_t kGeoSmem = (size_t)7 * 7 * 128 * 8;
 struct DevInfo {
     int sms = 0;
     int geo_blocks[3] = {0, 0, 0};  // per SM, indexed by precision: [fp64, mixed, fast]
+    int geo64_wide = 0;             // FP64 form, the shape for fewer rays
     int tr_occ[2][8] = {};          // transfer variants: [double, float][feature bits]
     int tr_mlp_occ[2] = {0, 0};     // learned-coefficient transfer: [fast light, slow light]
     int mi_occ[2] = {0, 0};         // learned-coefficient model inputs: [fast, slow light]
@@ -426,13 +427,17 @@ int dev_info(DevInfo& out) {
     if (di.sms == 0) {
         BL_CUDA(cudaDeviceGetAttribute(&di.sms, cudaDevAttrMultiProcessorCount, dev));
         // the stage derivatives exceed the default 48 KB of shared memory
-        BL_CUDA(cudaFuncSetAttribute(bl::geodesic_kernel<float, double>,
+        BL_CUDA(cudaFuncSetAttribute(bl::geodesic64_kernel<double>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGeoSmem));
+        BL_CUDA(cudaFuncSetAttribute(bl::geodesic64_kernel<float>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGeoSmem));
         BL_CUDA(cudaFuncSetAttribute(bl::geodesic_kernel<float, bl::df64>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGeoSmem));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo_blocks[0], bl::geodesic_kernel_fp64, 128, 0));
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo_blocks[1], bl::geodesic_kernel<float, double>, 128, kGeoSmem));
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo_blocks[1], bl::geodesic64_kernel<float>, 128, kGeoSmem));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo_blocks[2], bl::geodesic_kernel<float, bl::df64>, 128, kGeoSmem));
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo64_wide, bl::geodesic64_kernel<double>, 128, kGeoSmem));
+        if (di.geo64_wide < 1) di.geo64_wide = 1;
         for (int i = 0; i < 3; ++i)
             if (di.geo_blocks[i] < 1) di.geo_blocks[i] = 1;
         int rc = occ_transfer_all<double, double>(di.tr_occ[0]);
@@ -591,6 +596,8 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
     auto pick = [](int want, int occ) { return want > 0 && want < occ ? want : occ; };
     const unsigned geo_grid = (unsigned)(di.sms * pick(cfg.geo_ctas, di.geo_blocks[pidx]));
     const unsigned tr_grid = (unsigned)(di.sms * pick(cfg.tr_ctas, di.transfer(precision, mlp, cfg.feat)));
+    // a hand-set or tuned number of geodesic CTAs an SM (otherwise the kernels' own rules apply)
+    const bool geo_set = cfg.geo_ctas > 0 && cfg.geo_ctas < di.geo_blocks[pidx];
     const int record = transfer ? 1 : 0;
     const bool slow = (cfg.feat & bl::kFSlow) != 0;
     for (int64_t w = 0; w < n_waves; ++w) {
@@ -622,13 +629,18 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
             }
             if (precision == BL_PREC_FP64) {
                 bl::RecordSink<double> sink{(double*)(ws + L.pool), chunks, (unsigned long long)L.pool_chunks, ctr};
-                bl::geodesic_kernel_fp64<<<geo_grid, 128, 0, st>>>(
-                    d_desc, n_images, b, e, hdr, sink, record, cfg.bs, init);
+                if (!geo_set && e - b <= bl::kGeo64DeepRays * di.sms)
+                    bl::geodesic64_kernel<double><<<(unsigned)(di.sms * di.geo64_wide), 128, kGeoSmem, st>>>(
+                        d_desc, n_images, b, e, hdr, sink, record, cfg.bs, di.sms);
+                else
+                    bl::geodesic_kernel_fp64<<<geo_grid, 128, 0, st>>>(
+                        d_desc, n_images, b, e, hdr, sink, record, cfg.bs);
             } else {
                 bl::RecordSink<float> sink{(float*)(ws + L.pool), chunks, (unsigned long long)L.pool_chunks, ctr};
                 if (precision == BL_PREC_MIXED)
-                    bl::geodesic_kernel<float, double><<<geo_grid, 128, kGeoSmem, st>>>(
-                        d_desc, n_images, b, e, hdr, sink, record, cfg.bs, init);
+                    bl::geodesic64_kernel<float><<<geo_grid, 128, kGeoSmem, st>>>(
+                        d_desc, n_images, b, e, hdr, sink, record, cfg.bs,
+                        geo_set ? 0 : di.sms);
                 else
                     bl::geodesic_kernel<float, bl::df64><<<geo_grid, 128, kGeoSmem, st>>>(
                         d_desc, n_images, b, e, hdr, sink, record, cfg.bs, init);

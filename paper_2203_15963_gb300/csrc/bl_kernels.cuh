@@ -831,6 +831,18 @@ __device__ __forceinline__ double inv_fifth_root(double e) {
     return y;
 }
 
+// x is neither NaN nor infinite (exponent field not all ones)
+__device__ __forceinline__ bool finite_bits(float x) {
+    return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u;
+}
+__device__ __forceinline__ bool finite_bits(double x) {
+    return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
+
+}  // namespace bl
+#include "bl_geo64.cuh"
+namespace bl {
+
 template <class R, class G, bool kKsmem>
 __device__ __forceinline__ void geodesic_body(const ImageDesc* __restrict__ imgs,
                                               int n_images, int64_t ray_begin, int64_t ray_end,
@@ -1309,21 +1321,41 @@ __global__ void __launch_bounds__(128, BL_GEO_MIN_CTAS) geodesic_kernel(const Im
     geodesic_body<R, G, true>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs, init);
 }
 
-// Resident CTAs per SM the FP64-form geodesic kernel is compiled for: 16 (32 registers, the
-// SM's 64 warps; stage derivatives in local memory) measured 189.7 ms on the 9 x 256^2 step,
-// against 199.6 ms at 3 CTAs with them in shared memory (4: 203.9; in local memory 4: 201.7,
-// 6: 202.7, 8: 207.6). The mixed form (FP32 records, whose midpoints are formed in FP32)
-// stays in the shared-memory kernel at 3 CTAs: 148.8 ms there against 160.5 ms in this one.
+// The FP64-arithmetic geodesic kernels (bl_geo64.cuh). Two shapes:
+//   geodesic64_kernel      3 CTAs an SM (168 registers, no spills, stage derivatives in shared
+//                          memory): the mixed form, and the FP64 form up to kGeo64DeepRays rays
+//                          an SM;
+//   geodesic_kernel_fp64   16 CTAs an SM (32 registers, the SM's 64 warps, stage derivatives in
+//                          local memory): more FP64 rays than that, where resident warps keep
+//                          the FP64 pipe fed (9 x 256^2: 151 ms against 162; three images: 61
+//                          against 52).
+// Four warps an SM, one a scheduler, already hold the FP64 pipe at 84 % of its rate, and every
+// further warp slows the ones there: a launch of few rays ends with its longest rays, which then
+// run at the pace of the crowd. So up to kGeo64SparseRays rays an SM a single CTA an SM works
+// through the queue (FP64, one 256^2 image: 22.2 ms against 28.5 at 3 CTAs and 33.9 at 16; mixed
+// 17.9 against 27.7; three images, 1293 rays an SM: 61 against 52, so the line lies between). The
+// CTAs beyond the first of an SM decide that for themselves, as a device block list's length is
+// not known to the host.
 #ifndef BL_GEO64_MIN_CTAS
 #define BL_GEO64_MIN_CTAS 16
 #endif
-// The FP64 form (FP64 state, FP64 records) with its own register budget.
+#ifndef BL_GEO64_WIDE_CTAS
+#define BL_GEO64_WIDE_CTAS 3
+#endif
+constexpr int64_t kGeo64SparseRays = 4 * 128, kGeo64DeepRays = 20 * 128;   // rays an SM
 __global__ void __launch_bounds__(128, BL_GEO64_MIN_CTAS) geodesic_kernel_fp64(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
-        RayHdr* __restrict__ hdr, RecordSink<double> sink, int record, BlockSource bs,
-        const RayInit* __restrict__ init) {
-    geodesic_body<double, double, false>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs,
-                                         init);
+        RayHdr* __restrict__ hdr, RecordSink<double> sink, int record, BlockSource bs) {
+    geodesic64_body<double, false>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs);
+}
+// sms > 0: CTAs from number `sms` on leave at once when the wave is sparse.
+template <class R>
+__global__ void __launch_bounds__(128, BL_GEO64_WIDE_CTAS) geodesic64_kernel(
+        const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
+        RayHdr* __restrict__ hdr, RecordSink<R> sink, int record, BlockSource bs, int sms) {
+    if (sms > 0 && (int)blockIdx.x >= sms &&
+        wave_end(bs, ray_end) - ray_begin <= kGeo64SparseRays * sms) return;
+    geodesic64_body<R, true>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs);
 }
 
 // Per-image constant in the transfer arithmetic.
@@ -1562,13 +1594,6 @@ __device__ __forceinline__ T grid_val(float f) {
     }
 }
 
-// x is neither NaN nor infinite (exponent field not all ones)
-__device__ __forceinline__ bool finite_bits(float x) {
-    return (__float_as_uint(x) & 0x7f800000u) != 0x7f800000u;
-}
-__device__ __forceinline__ bool finite_bits(double x) {
-    return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
-}
 
 // Fused multiply-add in T, written out: the grid sums below fix their rounding in the source
 // (a sum of two products may otherwise be fused either way), so that both grid layouts and
