@@ -596,8 +596,9 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
     auto pick = [](int want, int occ) { return want > 0 && want < occ ? want : occ; };
     const unsigned geo_grid = (unsigned)(di.sms * pick(cfg.geo_ctas, di.geo_blocks[pidx]));
     const unsigned tr_grid = (unsigned)(di.sms * pick(cfg.tr_ctas, di.transfer(precision, mlp, cfg.feat)));
-    // a hand-set or tuned number of geodesic CTAs an SM (otherwise the kernels' own rules apply)
+    // a hand-set or tuned number of CTAs an SM (otherwise the kernels' own rules apply)
     const bool geo_set = cfg.geo_ctas > 0 && cfg.geo_ctas < di.geo_blocks[pidx];
+    const bool tr_set = cfg.tr_ctas > 0 && cfg.tr_ctas < di.transfer(precision, mlp, cfg.feat);
     const int record = transfer ? 1 : 0;
     const bool slow = (cfg.feat & bl::kFSlow) != 0;
     for (int64_t w = 0; w < n_waves; ++w) {
@@ -629,7 +630,7 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
             }
             if (precision == BL_PREC_FP64) {
                 bl::RecordSink<double> sink{(double*)(ws + L.pool), chunks, (unsigned long long)L.pool_chunks, ctr};
-                if (!geo_set && e - b <= bl::kGeo64DeepRays * di.sms)
+                if (!geo_set && e - b <= bl::kDeep64Rays * di.sms)
                     bl::geodesic64_kernel<double><<<(unsigned)(di.sms * di.geo64_wide), 128, kGeoSmem, st>>>(
                         d_desc, n_images, b, e, hdr, sink, record, cfg.bs, di.sms);
                 else
@@ -727,9 +728,14 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                 bl::work_scatter_kernel<bl::kTransportGroup><<<sgrid, 256, 0, st>>>(tkey, cfg.bs, b, e, thist, tperm);
                 g_launches += 4;
                 BL_CUDA(cudaGetLastError());
-                bl::transport_fp64_kernel<<<tr_grid, bl::kTransferFp64Threads, 0, st>>>(
-                    d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs,
-                    bl::SideIn{nullptr, nullptr, pre, pflag, tfirst}, tperm);
+                if (!tr_set && e - b <= bl::kDeep64Rays * di.sms)
+                    bl::transport64_wide_kernel<<<(unsigned)(di.sms * bl::kTransport64WideCtas), 128, 0, st>>>(
+                        d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs,
+                        bl::SideIn{nullptr, nullptr, pre, pflag, tfirst}, tperm, di.sms);
+                else
+                    bl::transport_fp64_kernel<<<tr_grid, bl::kTransferFp64Threads, 0, st>>>(
+                        d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs,
+                        bl::SideIn{nullptr, nullptr, pre, pflag, tfirst}, tperm);
             } else {
                 if (cfg.order_transfer && (rc = order_by_records())) return rc;
                 launch_transfer<double, double>(cfg.feat, tr_grid, st, d_desc, n_images, b, e,

@@ -1323,7 +1323,7 @@ __global__ void __launch_bounds__(128, BL_GEO_MIN_CTAS) geodesic_kernel(const Im
 
 // The FP64-arithmetic geodesic kernels (bl_geo64.cuh). Two shapes:
 //   geodesic64_kernel      3 CTAs an SM (168 registers, no spills, stage derivatives in shared
-//                          memory): the mixed form, and the FP64 form up to kGeo64DeepRays rays
+//                          memory): the mixed form, and the FP64 form up to kDeep64Rays rays
 //                          an SM;
 //   geodesic_kernel_fp64   16 CTAs an SM (32 registers, the SM's 64 warps, stage derivatives in
 //                          local memory): more FP64 rays than that, where resident warps keep
@@ -1331,7 +1331,7 @@ __global__ void __launch_bounds__(128, BL_GEO_MIN_CTAS) geodesic_kernel(const Im
 //                          against 52).
 // Four warps an SM, one a scheduler, already hold the FP64 pipe at 84 % of its rate, and every
 // further warp slows the ones there: a launch of few rays ends with its longest rays, which then
-// run at the pace of the crowd. So up to kGeo64SparseRays rays an SM a single CTA an SM works
+// run at the pace of the crowd. So up to kSparse64Rays rays an SM a single CTA an SM works
 // through the queue (FP64, one 256^2 image: 22.2 ms against 28.5 at 3 CTAs and 33.9 at 16; mixed
 // 17.9 against 27.7; three images, 1293 rays an SM: 61 against 52, so the line lies between). The
 // CTAs beyond the first of an SM decide that for themselves, as a device block list's length is
@@ -1342,7 +1342,12 @@ __global__ void __launch_bounds__(128, BL_GEO_MIN_CTAS) geodesic_kernel(const Im
 #ifndef BL_GEO64_WIDE_CTAS
 #define BL_GEO64_WIDE_CTAS 3
 #endif
-constexpr int64_t kGeo64SparseRays = 4 * 128, kGeo64DeepRays = 20 * 128;   // rays an SM
+constexpr int64_t kSparse64Rays = 4 * 128, kDeep64Rays = 20 * 128;   // rays an SM
+// Few enough rays in this wave for one CTA an SM.
+__device__ __forceinline__ bool sparse_wave(const BlockSource& bs, int64_t ray_begin,
+                                            int64_t ray_end, int sms) {
+    return wave_end(bs, ray_end) - ray_begin <= kSparse64Rays * sms;
+}
 __global__ void __launch_bounds__(128, BL_GEO64_MIN_CTAS) geodesic_kernel_fp64(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         RayHdr* __restrict__ hdr, RecordSink<double> sink, int record, BlockSource bs) {
@@ -1353,8 +1358,7 @@ template <class R>
 __global__ void __launch_bounds__(128, BL_GEO64_WIDE_CTAS) geodesic64_kernel(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         RayHdr* __restrict__ hdr, RecordSink<R> sink, int record, BlockSource bs, int sms) {
-    if (sms > 0 && (int)blockIdx.x >= sms &&
-        wave_end(bs, ray_end) - ray_begin <= kGeo64SparseRays * sms) return;
+    if (sms > 0 && (int)blockIdx.x >= sms && sparse_wave(bs, ray_begin, ray_end, sms)) return;
     geodesic64_body<R, true>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs);
 }
 
@@ -2223,12 +2227,10 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
         if (!kUnpol && started) {
             // merged N half-steps from the previous sample to this one (to the camera node on
             // the finishing iteration, where the far half is empty)
-            T A0[4][4], A1[4][4];
             const T kp[4] = {kt, prev[3], prev[4], prev[5]};
             const T kn[4] = {kt, prev[9], prev[10], prev[11]};
-            transport_matrix<T>(prev, kp, a, m, flat, A0);
-            transport_matrix<T>(prev + 6, kn, a, m, flat, A1);
-            coh_pc_step(N, A0, A1, T(0.5) * (prev[12] + (finishing ? T(0) : cur[12])));
+            coh_pc_step<T>(N, prev, kp, prev + 6, kn, a, m, flat,
+                           T(0.5) * (prev[12] + (finishing ? T(0) : cur[12])));
         }
         if (finishing) {
             const int64_t npix = im.n_rays;
@@ -2656,7 +2658,7 @@ __global__ void transport_key_kernel(const int32_t* __restrict__ tfirst,
 #ifndef BL_TRANSPORT64_MAXNREG
 #define BL_TRANSPORT64_MAXNREG 32
 #endif
-__global__ void __maxnreg__(BL_TRANSPORT64_MAXNREG) transport_fp64_kernel(
+__device__ __forceinline__ void transport_fp64_body(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         const RayHdr* __restrict__ hdr, const double* __restrict__ pool,
         const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side,
@@ -2725,22 +2727,11 @@ __global__ void __maxnreg__(BL_TRANSPORT64_MAXNREG) transport_fp64_kernel(
             const double* pr = pool + record_index(chunks, wray, idx + 1) * RecStride<double>::v;
             if (started) {
                 const T h = T(0.5) * (__ldg(pr + 12) + dl_cur);
-                T A[4][4];
-                Coh<T> nh;
-                {
-                    const T x0[3] = {__ldg(pr), __ldg(pr + 1), __ldg(pr + 2)};
-                    const T k0[4] = {kt, __ldg(pr + 3), __ldg(pr + 4), __ldg(pr + 5)};
-                    transport_matrix<T>(x0, k0, a, m, flat, A);
-                }
-                coh_axpy(N, N, A, T(0.5) * h, nh);
-                {
-                    const T x1[3] = {__ldg(pr + 6), __ldg(pr + 7), __ldg(pr + 8)};
-                    const T k1[4] = {kt, __ldg(pr + 9), __ldg(pr + 10), __ldg(pr + 11)};
-                    transport_matrix<T>(x1, k1, a, m, flat, A);
-                }
-                Coh<T> out;
-                coh_axpy(N, nh, A, h, out);
-                N = out;
+                const T x0[3] = {__ldg(pr), __ldg(pr + 1), __ldg(pr + 2)};
+                const T k0[4] = {kt, __ldg(pr + 3), __ldg(pr + 4), __ldg(pr + 5)};
+                const T x1[3] = {__ldg(pr + 6), __ldg(pr + 7), __ldg(pr + 8)};
+                const T k1[4] = {kt, __ldg(pr + 9), __ldg(pr + 10), __ldg(pr + 11)};
+                coh_pc_step<T>(N, x0, k0, x1, k1, a, m, flat, h);
             }
             if (finishing) {
                 // read out in the camera basis at the camera-side node of the last record
@@ -2774,6 +2765,28 @@ __global__ void __maxnreg__(BL_TRANSPORT64_MAXNREG) transport_fp64_kernel(
         }
         --idx;
     }
+}
+
+// Two shapes, as for the FP64 geodesics: 32 registers and the SM's 64 warps for dense waves, 3
+// CTAs of 128 threads an SM without spills up to kDeep64Rays rays an SM (three 256^2 images,
+// both transfer passes: 34.3 ms against 48.9), of which all but the first of an SM leave when the
+// wave is sparse (one 256^2 image: 14.3 ms against 22.0 with all and 24.0 in the dense shape; a
+// 32^2 image 5.4 against 7.0). Nine images: 105 ms dense, 109 in the other shape.
+__global__ void __maxnreg__(BL_TRANSPORT64_MAXNREG) transport_fp64_kernel(
+        const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
+        const RayHdr* __restrict__ hdr, const double* __restrict__ pool,
+        const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side,
+        const int32_t* __restrict__ perm) {
+    transport_fp64_body(imgs, n_images, ray_begin, ray_end, hdr, pool, chunks, ctr, bs, side, perm);
+}
+constexpr int kTransport64WideCtas = 3;
+__global__ void __launch_bounds__(128, kTransport64WideCtas) transport64_wide_kernel(
+        const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
+        const RayHdr* __restrict__ hdr, const double* __restrict__ pool,
+        const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side,
+        const int32_t* __restrict__ perm, int sms) {
+    if ((int)blockIdx.x >= sms && sparse_wave(bs, ray_begin, ray_end, sms)) return;
+    transport_fp64_body(imgs, n_images, ray_begin, ray_end, hdr, pool, chunks, ctr, bs, side, perm);
 }
 
 // ---------------------------------------------------------------------------------------

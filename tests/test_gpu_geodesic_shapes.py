@@ -1,4 +1,4 @@
-"""The FP64-arithmetic geodesic kernels: every launch shape integrates a ray with the same bits,
+"""The FP64-arithmetic kernels: every launch shape traces a ray with the same bits,
 and the FP32 decision into how many samples a step splits (FP64 where its error bound straddles
 a boundary) gives the FP64 decision, which a trace with auxiliary images always takes."""
 import math
@@ -36,13 +36,13 @@ def _image(n, spin, inc, precision, **metric):
     (48, 0.0, 17.0, native.BL_PREC_FP64), (37, 0.97, 80.0, native.BL_PREC_MIXED)])
 def test_launch_shapes_give_the_same_bits(torus, n, spin, inc, precision):
     """The default shape against a plan with a set number of CTAs an SM (FP64: the 64-warp
-    kernel)."""
+    kernels)."""
     gp, prims = torus
     cam, met = _image(n, spin, inc, precision)
     a, b = _outs(n, precision), _outs(n, precision)
     images.trace_images([cam], [met], [gp], [prims[spin]], [FREQ], outs=[a])
     plan = native.Plan([cam], [met], [gp], [prims[spin]], [FREQ], [b],
-                       config={"geo_ctas_per_sm": 2})
+                       config={"geo_ctas_per_sm": 2, "tr_ctas_per_sm": 2})
     plan.run()
     plan.check()
     plan.close()
