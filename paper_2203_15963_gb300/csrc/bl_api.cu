@@ -612,10 +612,10 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
             const unsigned rk_grid = (unsigned)(di.sms * pick(cfg.geo_ctas, di.rk_occ[ri]));
             if (precision == BL_PREC_FP64) {
                 bl::RecordSink<double> sink{(double*)(ws + L.pool), chunks, (unsigned long long)L.pool_chunks, ctr};
-                bl::geodesic_rk_kernel<double><<<rk_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, sink, record, cfg.bs);
+                bl::geodesic_rk_kernel<double><<<rk_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, sink, record, cfg.bs, geo_set ? 0 : di.sms);
             } else {
                 bl::RecordSink<float> sink{(float*)(ws + L.pool), chunks, (unsigned long long)L.pool_chunks, ctr};
-                bl::geodesic_rk_kernel<float><<<rk_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, sink, record, cfg.bs);
+                bl::geodesic_rk_kernel<float><<<rk_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, sink, record, cfg.bs, geo_set ? 0 : di.sms);
             }
         } else {
             // double-float form: the wave's pixel initial states first, then the integrator

@@ -189,28 +189,6 @@ __device__ __forceinline__ T dot4(const KSGeom<T>& G, const T u[4], const T v[4]
     return -u[0] * v[0] + u[1] * v[1] + u[2] * v[2] + u[3] * v[3] + G.f * lu * lv;
 }
 
-// Eq. (geodesic): dx^a/dl = g^ab k_b; dk_t/dl = 0; dk_c/dl = -1/2 d_c g^ab k_a k_b
-//   = L (1/2 d_c f L + f sum_b d_c l_b k_b),  L = l^a k_a.
-// Returns r at the evaluation point (used for the termination tests).
-__device__ __forceinline__ double geodesic_rhs(const double y[8], double a, double m, bool flat,
-                                               double dy[8]) {
-    KSGeom<double> G;
-    ks_geom<double>(y[1], y[2], y[3], a, m, flat, true, G);
-    const double* k = y + 4;
-    const double L = -k[0] + G.l[1] * k[1] + G.l[2] * k[2] + G.l[3] * k[3];
-    dy[0] = -k[0] + G.f * L;
-    dy[1] = k[1] - G.f * G.l[1] * L;
-    dy[2] = k[2] - G.f * G.l[2] * L;
-    dy[3] = k[3] - G.f * G.l[3] * L;
-    dy[4] = 0.0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const double S = G.dl[c][0] * k[1] + G.dl[c][1] * k[2] + G.dl[c][2] * k[3];
-        dy[5 + c] = L * (0.5 * G.df[c] * L + G.f * S);
-    }
-    return G.r;
-}
-
 // ---------------------------------------------------------------------------------------
 // Coordinate terms of Eq. (polarized_n), read as parallel transport of the coherency
 // tensor: dN/dl = A N + N A^T with A^a_d = -k^c Gamma^a_cd. For g = eta + f l l the
