@@ -1828,10 +1828,26 @@ int blacklight_mlp_normalise(int64_t n, const float* inputs, const float* target
     if (!rc) rc = device_pointer(targets, "targets");
     if (!rc) rc = device_pointer(params, "params");
     if (rc) return rc;
-    bl::mlp::normalise_kernel<<<1, 256, 0, (cudaStream_t)stream>>>(n, inputs, targets, params);
-    ++g_launches;
-    BL_CUDA(cudaGetLastError());
-    BL_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    cudaStream_t st = (cudaStream_t)stream;
+    DevInfo di;
+    if ((rc = dev_info(di))) return rc;
+    // block sums of either pass, then beta
+    const int64_t want = (n + bl::mlp::kNormThreads - 1) / bl::mlp::kNormThreads;
+    const int blocks = (int)(want < 4 * di.sms ? want : 4 * di.sms);
+    const size_t n_part = (size_t)blocks * bl::mlp::kNormSums;
+    double* buf = nullptr;
+    cudaError_t e = cudaMallocAsync((void**)&buf, sizeof(double) * (n_part + 28), st);
+    if (e != cudaSuccess) { cudaGetLastError(); return fail(BL_ENOMEM, "cudaMallocAsync: %s", cudaGetErrorString(e)); }
+    double* beta = buf + n_part;
+    bl::mlp::normalise_sums_kernel<<<blocks, bl::mlp::kNormThreads, 0, st>>>(n, inputs, targets, buf);
+    bl::mlp::normalise_solve_kernel<<<1, 64, 0, st>>>(blocks, buf, beta);
+    bl::mlp::normalise_residual_kernel<<<blocks, bl::mlp::kNormThreads, 0, st>>>(n, inputs, targets, beta, buf);
+    bl::mlp::normalise_store_kernel<<<1, 32, 0, st>>>(n, blocks, buf, beta, params);
+    g_launches += 4;
+    e = cudaGetLastError();
+    cudaFreeAsync(buf, st);
+    if (e != cudaSuccess) return cuda_fail(e, "normalise");
+    BL_CUDA(cudaStreamSynchronize(st));
     return 0;
 }
 

@@ -48,8 +48,17 @@ __device__ __forceinline__ uint64_t kdesc(const void* tile, int K, int s) {
     return sdesc(smem_addr(tile) + 256u * (uint32_t)s, 128u, (uint32_t)(K >> 3) * 128u);
 }
 
+// The same tile read MN-major (its rows along K, its columns along M or N): core matrices of 8 K
+// rows x 8 columns, adjacent column groups 128 bytes apart (stride byte offset), adjacent groups
+// of 8 K rows one row group of the tile, (pitch/8) 128, apart (leading byte offset); K-step s of
+// 16 rows starts two row groups further.
+__device__ __forceinline__ uint64_t mndesc(const void* tile, int pitch, int s) {
+    const uint32_t group = (uint32_t)(pitch >> 3) * 128u;
+    return sdesc(smem_addr(tile) + 2u * group * (uint32_t)s, group, 128u);
+}
+
 // Instruction descriptor, kind::f16: D FP32 (bits 4-5 = 1), A and B BF16 (bits 7-9, 10-12 =
-// 1), both K-major, N >> 3 at bits 17-22, M >> 4 at bits 24-28.
+// 1), both K-major (bits 15, 16: A, B MN-major), N >> 3 at bits 17-22, M >> 4 at bits 24-28.
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
            ((uint32_t)(M >> 4) << 24);
@@ -98,6 +107,24 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, long l
     return false;
 }
 
+// --- bulk copy (one thread): bytes (a multiple of 16, both addresses 16-byte aligned) from global
+// to this CTA's shared memory; bar's phase completes when they have arrived ---
+__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;"
+                 ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, "
+                 "[%3];" ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
+}
+
+// --- programmatic dependent launch: wait for the grids this one depends on (all their writes are
+// then visible); allow the next grid in the stream to start its own independent part ---
+__device__ __forceinline__ void grid_dependency_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void grid_launch_dependents() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // --- MMA (issued by one thread) ---
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
                                          uint32_t idesc, bool accumulate) {
@@ -110,6 +137,20 @@ __device__ __forceinline__ void gemm_bf16(uint32_t d_tmem, const void* A, const 
                                           int K) {
     const uint32_t id = idesc_bf16_f32(128, N);
     for (int s = 0; s < (K >> 4); ++s) mma_bf16(d_tmem, kdesc(A, K, s), kdesc(B, K, s), id, s > 0);
+}
+// The same with the tiles' row pitches (in columns) given.
+__device__ __forceinline__ void gemm_kmajor(uint32_t d_tmem, const void* A, int pitch_a,
+                                            const void* B, int pitch_b, int N, int K) {
+    const uint32_t id = idesc_bf16_f32(128, N);
+    for (int s = 0; s < (K >> 4); ++s)
+        mma_bf16(d_tmem, kdesc(A, pitch_a, s), kdesc(B, pitch_b, s), id, s > 0);
+}
+// D[M=128][N] = A^T B of tiles A [K][M], B [K][N] (both read MN-major).
+__device__ __forceinline__ void gemm_mnmajor(uint32_t d_tmem, const void* A, int pitch_a,
+                                             const void* B, int pitch_b, int N, int K) {
+    const uint32_t id = idesc_bf16_f32(128, N) | (1u << 15) | (1u << 16);
+    for (int s = 0; s < (K >> 4); ++s)
+        mma_bf16(d_tmem, mndesc(A, pitch_a, s), mndesc(B, pitch_b, s), id, s > 0);
 }
 // arrive on bar once every MMA issued so far by this thread has completed
 __device__ __forceinline__ void mma_commit(uint64_t* bar) {
@@ -135,6 +176,23 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float v[16]) {
                  :: "memory");
 #pragma unroll
     for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+}
+// The load and its wait apart: several loads in flight, then one tmem_ld16_wait for each before its
+// registers are used.
+__device__ __forceinline__ void tmem_ld16_issue(uint32_t taddr, uint32_t r[16]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,"
+                 "%12,%13,%14,%15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]),
+                   "=r"(r[6]), "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]),
+                   "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld16_wait(uint32_t r[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]),
+                   "+r"(r[6]), "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]),
+                   "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :: "memory");
 }
 // address of (this warp's first lane, column col)
 __device__ __forceinline__ uint32_t tmem_lane_addr(uint32_t base, int col) {
