@@ -1862,15 +1862,18 @@ int blacklight_mlp_grad(const float* params, int64_t n, const float* inputs, con
     if (!rc) rc = mlp_train_attr();
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    float* dloss = nullptr;
-    cudaError_t e = cudaMallocAsync((void**)&dloss, sizeof(float), st);
+    // the weight image, then the error sum
+    unsigned char* img = nullptr;
+    cudaError_t e = cudaMallocAsync((void**)&img, bl::mlp::kImgBytes + sizeof(float), st);
     if (e != cudaSuccess) { cudaGetLastError(); return fail(BL_ENOMEM, "cudaMallocAsync: %s", cudaGetErrorString(e)); }
+    float* dloss = (float*)(img + bl::mlp::kImgBytes);
     rc = with_tc_flag(st, [&](int* err) -> int {
         BL_CUDA(cudaMemsetAsync(grad, 0, sizeof(float) * BL_MLP_PARAMS, st));
-        BL_CUDA(cudaMemsetAsync(dloss, 0, sizeof(float), st));
+        BL_CUDA(cudaMemsetAsync(img, 0, bl::mlp::kImgBytes + sizeof(float), st));
+        bl::mlp::image_kernel<<<(BL_MLP_PARAMS + 127) / 128, 128, 0, st>>>(params, img, nullptr);
         bl::mlp::train_kernel<<<(unsigned)((n + 127) / 128), 128, bl::mlp::kTrainSmem, st>>>(
-            params, n, inputs, targets, 0, n, (double)n, grad, dloss, nullptr, nullptr, err);
-        ++g_launches;
+            img, n, inputs, targets, 0, n, (double)n, grad, dloss, nullptr, nullptr, err);
+        g_launches += 2;
         BL_CUDA(cudaGetLastError());
         float h = 0.0f;
         BL_CUDA(cudaMemcpyAsync(&h, dloss, sizeof(float), cudaMemcpyDeviceToHost, st));
@@ -1878,7 +1881,7 @@ int blacklight_mlp_grad(const float* params, int64_t n, const float* inputs, con
         *loss = (float)(h / (7.0 * (double)n));
         return 0;
     });
-    cudaFreeAsync(dloss, st);
+    cudaFreeAsync(img, st);
     return rc;
 }
 
@@ -1898,38 +1901,61 @@ int blacklight_mlp_train(const bl_mlp_train_t* cfg, float* params, float* loss_h
     if (!rc) rc = mlp_train_attr();
     if (rc) return rc;
     cudaStream_t st = (cudaStream_t)stream;
-    // m, v [BL_MLP_PARAMS] each, then per-tile gradient sums [tiles][trained parameters] and
-    // per-tile losses [tiles]: the tiles' sums are reduced in a fixed order, so a training run
-    // is reproducible bit for bit
+    // the weight image, then floats: weights, m, v [trained parameters] each in slot order,
+    // per-tile gradient sums [tiles][trained parameters] and per-tile losses [tiles]: the tiles'
+    // sums are reduced in a fixed order, so a training run is reproducible bit for bit
     const int64_t tiles = cfg->batch / 128;
-    const size_t n_part = (size_t)tiles * bl::mlp::kOffMean;
-    float* buf = nullptr;
-    const size_t bytes = sizeof(float) * (2 * (size_t)BL_MLP_PARAMS + n_part + (size_t)tiles);
+    const size_t n_tr = bl::mlp::kOffMean, n_part = (size_t)tiles * n_tr;
+    const size_t img_bytes = align_up(bl::mlp::kImgBytes);
+    char* buf = nullptr;
+    const size_t bytes = img_bytes + sizeof(float) * (3 * n_tr + n_part + (size_t)tiles);
     cudaError_t e = cudaMallocAsync((void**)&buf, bytes, st);
     if (e != cudaSuccess) { cudaGetLastError(); return fail(BL_ENOMEM, "cudaMallocAsync: %s", cudaGetErrorString(e)); }
-    float *m = buf, *v = buf + BL_MLP_PARAMS, *part = buf + 2 * BL_MLP_PARAMS,
+    unsigned char* img = (unsigned char*)buf;
+    float *w = (float*)(buf + img_bytes), *m = w + n_tr, *v = m + n_tr, *part = v + n_tr,
           *part_loss = part + n_part;
     rc = with_tc_flag(st, [&](int* err) -> int {
-        BL_CUDA(cudaMemsetAsync(buf, 0, bytes, st));
-        const unsigned blocks = (unsigned)tiles;
+        BL_CUDA(cudaMemsetAsync(buf, 0, img_bytes + sizeof(float) * 3 * n_tr, st));
+        bl::mlp::image_kernel<<<(BL_MLP_PARAMS + 127) / 128, 128, 0, st>>>(params, img, w);
+        ++g_launches;
+        BL_CUDA(cudaGetLastError());
+        // each kernel may start while the one before it ends: it waits for that one's results
+        // itself (griddepcontrol.wait)
+        cudaLaunchAttribute pdl{};
+        pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        pdl.val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t tc{}, ac{};
+        tc.gridDim = dim3((unsigned)tiles);
+        tc.blockDim = dim3(128);
+        tc.dynamicSmemBytes = bl::mlp::kTrainSmem;
+        ac.gridDim = dim3(bl::mlp::kAdamBlocks);
+        ac.blockDim = dim3(bl::mlp::kAdamThreads);
+        tc.stream = ac.stream = st;
+        tc.attrs = ac.attrs = &pdl;
+        tc.numAttrs = ac.numAttrs = 1;
         const double b1 = cfg->beta1, b2 = cfg->beta2;
         double p1 = 1.0, p2 = 1.0;
         for (int64_t t = 0; t < cfg->steps; ++t) {
             const int64_t first = (int64_t)((t * (int64_t)cfg->batch) % cfg->n);
-            bl::mlp::train_kernel<<<blocks, 128, bl::mlp::kTrainSmem, st>>>(
-                params, cfg->n, cfg->inputs, cfg->targets, first, cfg->batch, (double)cfg->batch,
-                nullptr, nullptr, part, part_loss, err);
+            BL_CUDA(cudaLaunchKernelEx(&tc, bl::mlp::train_kernel, (const unsigned char*)img,
+                                       (int64_t)cfg->n, cfg->inputs, cfg->targets, first,
+                                       (int64_t)cfg->batch, (double)cfg->batch, (float*)nullptr,
+                                       (float*)nullptr, part, part_loss, err));
             const double frac = cfg->steps > 1 ? (double)t / (double)(cfg->steps - 1) : 0.0;
             const double lr = cfg->lr_start * pow(cfg->lr_end / cfg->lr_start, frac);
             p1 *= b1;
             p2 *= b2;
-            bl::mlp::adam_kernel<<<(bl::mlp::kOffMean + 255) / 256, 256, 0, st>>>(
-                params, part, (int)tiles, m, v, (float)lr, (float)b1, (float)b2, (float)cfg->eps,
-                (float)(1.0 - p1), (float)(1.0 - p2), part_loss,
-                loss_history ? loss_history + t : nullptr, (float)(1.0 / (7.0 * cfg->batch)));
+            BL_CUDA(cudaLaunchKernelEx(&ac, bl::mlp::adam_kernel, w, img, (const float*)part,
+                                       (int)tiles, m, v, (float)lr, (float)b1, (float)b2,
+                                       (float)cfg->eps, (float)(1.0 - p1), (float)(1.0 - p2),
+                                       (const float*)part_loss,
+                                       loss_history ? loss_history + t : (float*)nullptr,
+                                       (float)(1.0 / (7.0 * cfg->batch))));
             g_launches += 2;
-            BL_CUDA(cudaGetLastError());
         }
+        bl::mlp::unslot_kernel<<<(unsigned)((n_tr + 127) / 128), 128, 0, st>>>(w, params);
+        ++g_launches;
+        BL_CUDA(cudaGetLastError());
         return 0;
     });
     cudaFreeAsync(buf, st);

@@ -474,43 +474,117 @@ __global__ void __launch_bounds__(128) coefficients_kernel(const float* __restri
 
 // ---------------------------------------------------------------------------------------
 // Training: forward and backward of one 128-sample tile per CTA, all nine products on the
-// tensor cores. Weight gradients contract over the samples (K = 128): their A operand is the
-// transposed error (rows = units; the rows beyond the layer's units read neighbouring
-// shared memory and produce accumulator rows that are never read), their B operand the
-// transposed activations with a row of ones appended, whose column yields the bias gradient.
+// tensor cores. Weight gradients contract over the samples (K = 128): the same shared-memory
+// tiles as the forward and backward operands are then read MN-major (samples along K), with a
+// column of ones appended to the activations, whose accumulator column yields the bias gradient;
+// accumulator rows beyond the layer's units come from whatever follows the tile in shared memory
+// and are never read.
+// A step is a chain of five dependent products, so it is bound by latency, and what is not the
+// chain is taken off it: the weights arrive as one bulk copy of an image in operand layout (bf16
+// tiles, then the FP32 biases and output map) that adam_kernel keeps up to date, everything a
+// thread stores to shared memory is 16 bytes wide, tile gradients go out in the order the
+// accumulators come (slots), coalesced, and the next kernel's launch and the loads that do not
+// depend on the weights overlap the step before (programmatic dependent launch). Batch 16384, a
+// step (this kernel and adam_kernel): 41 us with the transposed copies, scalar stores and one
+// weight staging a tile, 14.2 us so.
 // ---------------------------------------------------------------------------------------
-constexpr uint32_t kTdZ2T = 0;        // [64][128] dZ2^T  (A, 128-row window to 32768)
-constexpr uint32_t kTdZ1T = 16384;    // [64][128] dZ1^T  (A window to 49152)
-constexpr uint32_t kTdZ3T = 32768;    // [8][128]  dY^T   (A window to 65536)
-constexpr uint32_t kTH1T = 34816;     // [80][128] H1^T, ones row 64 (B)
-constexpr uint32_t kTH2T = 55296;     // [80][128] H2^T, ones row 64 (B)
-constexpr uint32_t kTXT = 75776;      // [16][128] X^T (B): inputs, ones row 3
-constexpr uint32_t kTX = 79872;       // [128][16] X (A)
-constexpr uint32_t kTH1 = 83968;      // [128][64] H1 (A)
-constexpr uint32_t kTH2 = 100352;     // [128][64] H2 (A)
-constexpr uint32_t kTdZ3 = 116736;    // [128][16] dY (A)
-constexpr uint32_t kTdZ2 = 120832;    // [128][64] dZ2 (A)
-constexpr uint32_t kTW1 = 137216;     // [64][16] W1 (B)
-constexpr uint32_t kTW2 = 139264;     // [64][64] W2 (B)
-constexpr uint32_t kTW3 = 147456;     // [16][64] W3 (B)
-constexpr uint32_t kTW3T = 149504;    // [64][16] W3^T (B)
-constexpr uint32_t kTW2T = 151552;    // [64][64] W2^T (B)
-constexpr uint32_t kTF32 = 159744;    // b2[64] b3[8] mean[8] scale[8] red[32] A[24]
-constexpr uint32_t kTBar = 161024;    // mbarrier, tensor-memory base
-constexpr uint32_t kTrainSmem = 161280;
+constexpr int kHPitch = 80;           // activation tiles: 64 units, the ones column, zeros
+constexpr uint32_t kTX = 0;           // [128][16] X: inputs, ones column 3
+constexpr uint32_t kTH1 = 4096;       // [128][80] H1
+constexpr uint32_t kTH2 = 24576;      // [128][80] H2
+constexpr uint32_t kTdZ3 = 45056;     // [128][16] dY
+constexpr uint32_t kTdZ2 = 49152;     // [128][64] dZ2
+constexpr uint32_t kTdZ1 = 65536;     // [128][64] dZ1
+constexpr uint32_t kTImg = 81920;     // the weight image
+constexpr uint32_t kTRed = 105472;    // float [32]
+constexpr uint32_t kTBar = 105600;    // two mbarriers, tensor-memory base
+constexpr uint32_t kTrainSmem = 105632;
+// the weight image: byte offsets of its parts
+constexpr uint32_t kIW1 = 0;          // [64][16] W1 (bias in column 3)
+constexpr uint32_t kIW2 = 2048;       // [64][64] W2
+constexpr uint32_t kIW3 = 10240;      // [16][64] W3 (rows 7-15 zero)
+constexpr uint32_t kIW3T = 12288;     // [64][16] W3^T
+constexpr uint32_t kIW2T = 14336;     // [64][64] W2^T
+constexpr uint32_t kIF32 = 22528;     // float b2[64] b3[8] mean[8] scale[8] A[24]
+constexpr uint32_t kImgBytes = kIF32 + 4 * 112;
+static_assert(kTImg + kImgBytes <= kTRed && kImgBytes % 16 == 0, "weight image");
 // tensor-memory columns (512 allocated)
 constexpr int kCZ1 = 0, kCZ2 = 64, kCZ3 = 128, kCdH2 = 160, kCdW3 = 224, kCdH1 = 304,
               kCdW2 = 368, kCdW1 = 448;
 constexpr uint32_t kTrainCols = 512;
 
+// Slot order of the trained parameters (tile gradients, Adam state): the accumulators' order, W2
+// and W3 by input unit first; the other parameters keep their places.
+__device__ __forceinline__ int slot_param(int s) {
+    if (s >= kOffW2 && s < kOffB2) {
+        const int q = s - kOffW2;
+        return kOffW2 + 64 * (q & 63) + (q >> 6);
+    }
+    if (s >= kOffW3 && s < kOffB3) {
+        const int q = s - kOffW3, c = q / kOut;
+        return kOffW3 + 64 * (q - kOut * c) + c;
+    }
+    return s;
+}
+
+// Parameter i (value w) in the weight image.
+__device__ __forceinline__ void image_store(unsigned char* __restrict__ img, int i, float w) {
+    float* fl = reinterpret_cast<float*>(img + kIF32);
+    if (i < kOffW2) {
+        tc::st_bf16(img + kIW1, i >> 2, i & 3, 16, w);
+    } else if (i < kOffB2) {
+        const int j = (i - kOffW2) >> 6, k = (i - kOffW2) & 63;
+        tc::st_bf16(img + kIW2, j, k, 64, w);
+        tc::st_bf16(img + kIW2T, k, j, 64, w);
+    } else if (i < kOffW3) {
+        fl[i - kOffB2] = w;
+    } else if (i < kOffB3) {
+        const int o = (i - kOffW3) >> 6, j = (i - kOffW3) & 63;
+        tc::st_bf16(img + kIW3, o, j, 64, w);
+        tc::st_bf16(img + kIW3T, j, o, 16, w);
+    } else if (i < kOffMean) {
+        fl[64 + i - kOffB3] = w;
+    } else if (i < kOffScale) {
+        fl[72 + i - kOffMean] = w;
+    } else if (i < kOffA) {
+        fl[80 + i - kOffScale] = w;
+    } else {
+        fl[88 + i - kOffA] = w;
+    }
+}
+
+// The image of P (img zeroed beforehand: padding rows and columns) and, where w is given, the
+// trained parameters in slot order.
+__global__ void image_kernel(const float* __restrict__ P, unsigned char* __restrict__ img,
+                             float* __restrict__ w) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= kParams) return;
+    image_store(img, i, P[i]);
+    if (w && i < kOffMean) w[i] = P[slot_param(i)];
+}
+// The trained parameters back into P.
+__global__ void unslot_kernel(const float* __restrict__ w, float* __restrict__ P) {
+    const int s = blockIdx.x * blockDim.x + threadIdx.x;
+    if (s < kOffMean) P[slot_param(s)] = w[s];
+}
+
+// Eight consecutive values of a row of a bf16 operand tile: one 16-byte store.
+__device__ __forceinline__ void st_row8(unsigned char* tile, int row, int col, int pitch,
+                                        const float v[8]) {
+    *reinterpret_cast<uint4*>(tile + tc::kmajor(row, col, pitch)) =
+        make_uint4(tc::pack_bf16x2(v[0], v[1]), tc::pack_bf16x2(v[2], v[3]),
+                   tc::pack_bf16x2(v[4], v[5]), tc::pack_bf16x2(v[6], v[7]));
+}
+
 // Gradients of the mean squared error over n_total samples x 7 outputs and the summed squared
 // error; block b takes the 128-sample tile b of the `count` samples starting at sample `first`
 // of the n-sample set (wrapping around). With part == nullptr the tiles add into grad[kParams]
 // and *loss atomically (summation order, and so the last bits, vary between runs). Otherwise
-// tile b stores its own sums, part[b][kOffMean] (every trained parameter) and part_loss[b], for
-// a reduction in a fixed order (adam_kernel), which makes training reproducible bit for bit.
-__global__ void __launch_bounds__(128, 1) train_kernel(const float* __restrict__ P, int64_t n,
-                                                       const float* __restrict__ in,
+// tile b stores its own sums, part[b][kOffMean] (every trained parameter, in slot order) and
+// part_loss[b], for a reduction in a fixed order (adam_kernel), which makes training
+// reproducible bit for bit.
+__global__ void __launch_bounds__(128, 1) train_kernel(const unsigned char* __restrict__ img,
+                                                       int64_t n, const float* __restrict__ in,
                                                        const float* __restrict__ tg,
                                                        int64_t first, int64_t count,
                                                        double n_total, float* __restrict__ grad,
@@ -518,60 +592,46 @@ __global__ void __launch_bounds__(128, 1) train_kernel(const float* __restrict__
                                                        float* __restrict__ part,
                                                        float* __restrict__ part_loss, int* err) {
     extern __shared__ __align__(1024) unsigned char sm[];
-    float* b2 = (float*)(sm + kTF32);
-    float* b3 = b2 + 64;
-    float* mean = b3 + 8;
-    float* scale = mean + 8;
-    float* red = scale + 8;
-    float* Atr = red + 32;
+    const float* b2 = (const float*)(sm + kTImg + kIF32);
+    const float* b3 = b2 + 64;
+    const float* mean = b3 + 8;
+    const float* scale = mean + 8;
+    const float* Atr = scale + 8;
+    float* red = (float*)(sm + kTRed);
     uint64_t* bar = (uint64_t*)(sm + kTBar);
-    uint32_t* tbase = (uint32_t*)(sm + kTBar + 8);
+    uint64_t* ibar = bar + 1;
+    uint32_t* tbase = (uint32_t*)(sm + kTBar + 16);
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
 
-    // ---- stage weights, constant rows and padding
-    for (int i = t; i < 64 * 16; i += 128) {
-        const int j = i >> 4, k = i & 15;
-        const float w = k < 4 ? P[kOffW1 + 4 * j + k] : 0.0f;
-        tc::st_bf16(sm + kTW1, j, k, 16, w);
-    }
-    for (int i = t; i < 64 * 64; i += 128) {
-        const int j = i >> 6, k = i & 63;
-        const float w = P[kOffW2 + i];
-        tc::st_bf16(sm + kTW2, j, k, 64, w);      // W2[j][k]: out j, in k
-        tc::st_bf16(sm + kTW2T, k, j, 64, w);     // W2^T[k][j]
-    }
-    for (int i = t; i < 16 * 64; i += 128) {
-        const int o = i >> 6, j = i & 63;
-        const float w = o < kOut ? P[kOffW3 + 64 * o + j] : 0.0f;
-        tc::st_bf16(sm + kTW3, o, j, 64, w);
-        tc::st_bf16(sm + kTW3T, j, o, 16, w);
-    }
-    for (int i = t; i < 16 * 128; i += 128) {     // X^T rows 3-15 and X columns 3-15
-        const int k = i >> 7, s = i & 127;
-        if (k >= 3) {
-            tc::st_bf16(sm + kTXT, k, s, 128, k == 3 ? 1.0f : 0.0f);
-            tc::st_bf16(sm + kTX, s, k, 16, k == 3 ? 1.0f : 0.0f);
-        }
-    }
-    for (int i = t; i < 16 * 128; i += 128) {     // ones row 64 and zero rows 65-79
-        const int r = 64 + (i >> 7), s = i & 127;
-        tc::st_bf16(sm + kTH1T, r, s, 128, r == 64 ? 1.0f : 0.0f);
-        tc::st_bf16(sm + kTH2T, r, s, 128, r == 64 ? 1.0f : 0.0f);
-    }
-    for (int i = t; i < 128 * 16; i += 128) {     // dY columns 7-15, dY^T row 7
-        const int s = i >> 4, k = i & 15;
-        if (k >= kOut) tc::st_bf16(sm + kTdZ3, s, k, 16, 0.0f);
-    }
-    tc::st_bf16(sm + kTdZ3T, 7, t, 128, 0.0f);
-    if (t < 64) b2[t] = P[kOffB2 + t];
-    if (t < 8) {
-        b3[t] = t < kOut ? P[kOffB3 + t] : 0.0f;
-        mean[t] = t < kOut ? P[kOffMean + t] : 0.0f;
-        scale[t] = t < kOut ? P[kOffScale + t] : 1.0f;
-    }
-    if (t < 24) Atr[t] = t < 3 * kOut ? P[kOffA + t] : 0.0f;
+    // ---- before the step's weights exist: tensor memory, barriers, this thread's sample (block
+    // b takes samples first + 128 b + t (mod n), t < count), constant columns
     if (warp == 0) tc::tmem_alloc(tbase, kTrainCols);
-    if (t == 0) tc::mbar_init(bar, 1);
+    if (t == 0) {
+        tc::mbar_init(bar, 1);
+        tc::mbar_init(ibar, 1);
+    }
+    const int64_t base = (int64_t)blockIdx.x * 128;
+    const bool valid = base + t < count;
+    const int64_t i = (first + base + t) % n;
+    float f[3] = {0.0f, 0.0f, 0.0f}, tn[7];
+    if (valid) {
+        f[0] = 2.0f * (in[3 * i] - kLxLo) / (kLxHi - kLxLo) - 1.0f;
+        f[1] = 2.0f * (in[3 * i + 1] - kLtLo) / (kLtHi - kLtLo) - 1.0f;
+        f[2] = 2.0f * fabsf(in[3 * i + 2]) - 1.0f;
+    }
+    for (int k = 0; k < kOut; ++k) tn[k] = valid ? tg[7 * i + k] : 0.0f;
+    {
+        const float zero[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        const float one[8] = {1.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        const float x[8] = {f[0], f[1], f[2], 1.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+        st_row8(sm + kTX, t, 0, 16, x);
+        st_row8(sm + kTX, t, 8, 16, zero);
+        st_row8(sm + kTH1, t, 64, kHPitch, one);
+        st_row8(sm + kTH1, t, 72, kHPitch, zero);
+        st_row8(sm + kTH2, t, 64, kHPitch, one);
+        st_row8(sm + kTH2, t, 72, kHPitch, zero);
+        st_row8(sm + kTdZ3, t, 8, 16, zero);
+    }
     tc::fence_smem_to_async();
     tc::fence_before_sync();
     __syncthreads();
@@ -591,169 +651,179 @@ __global__ void __launch_bounds__(128, 1) train_kernel(const float* __restrict__
         tc::fence_before_sync();
         __syncthreads();
     };
+    // the 64 accumulator columns from `col` of this thread's row
+    auto load64 = [&](int col, float v[64]) {
+        uint32_t r[4][16];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) tc::tmem_ld16_issue(tc::tmem_lane_addr(tm, col + 16 * c), r[c]);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            tc::tmem_ld16_wait(r[c]);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) v[16 * c + j] = __uint_as_float(r[c][j]);
+        }
+    };
 
-    // ---- this thread's sample: block b takes samples first + 128 b + t (mod n), t < count
-    const int64_t base = (int64_t)blockIdx.x * 128;
-    const bool valid = base + t < count;
-    const int64_t i = (first + base + t) % n;
-    float f[3] = {0.0f, 0.0f, 0.0f}, tn[7];
-    if (valid) {
-        f[0] = 2.0f * (in[3 * i] - kLxLo) / (kLxHi - kLxLo) - 1.0f;
-        f[1] = 2.0f * (in[3 * i + 1] - kLtLo) / (kLtHi - kLtLo) - 1.0f;
-        f[2] = 2.0f * fabsf(in[3 * i + 2]) - 1.0f;
-    }
-    __syncthreads();   // offset, scale and A staged
-    for (int k = 0; k < kOut; ++k)
-        tn[k] = valid ? (tg[7 * i + k] - mean[k] - Atr[3 * k] * f[0] - Atr[3 * k + 1] * f[1] -
-                         Atr[3 * k + 2] * f[2]) / scale[k]
-                      : 0.0f;
-    for (int k = 0; k < 3; ++k) {
-        tc::st_bf16(sm + kTX, t, k, 16, f[k]);
-        tc::st_bf16(sm + kTXT, k, t, 128, f[k]);
-    }
+    // ---- the weights of this step
+    tc::grid_dependency_wait();
+    tc::grid_launch_dependents();
+    if (t == 0) tc::bulk_load(sm + kTImg, img, kImgBytes, ibar);
+    const bool have = __syncthreads_and(tc::mbar_wait(ibar, 0u, kWaitCycles)) != 0;
 
     do {
+        if (!(ok = have)) break;
+        for (int k = 0; k < kOut; ++k)
+            tn[k] = valid ? (tn[k] - mean[k] - Atr[3 * k] * f[0] - Atr[3 * k + 1] * f[1] -
+                             Atr[3 * k + 2] * f[2]) / scale[k]
+                          : 0.0f;
         // ---- forward
-        barrier();
         if (t == 0) {
             tc::fence_after_sync();
-            tc::gemm_bf16(tm + kCZ1, sm + kTX, sm + kTW1, 64, 16);
+            tc::gemm_kmajor(tm + kCZ1, sm + kTX, 16, sm + kTImg + kIW1, 16, 64, 16);
             tc::mma_commit(bar);
         }
         if (!(ok = wait())) break;
-        for (int c = 0; c < 4; ++c) {
-            float v[16];
-            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCZ1 + 16 * c), v);
-            for (int j = 0; j < 16; ++j) {
-                const float h = silu(v[j]);
-                tc::st_bf16(sm + kTH1, t, 16 * c + j, 64, h);
-                tc::st_bf16(sm + kTH1T, 16 * c + j, t, 128, h);
-            }
+        {
+            float v[64];
+            load64(kCZ1, v);
+#pragma unroll
+            for (int j = 0; j < 64; ++j) v[j] = silu(v[j]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) st_row8(sm + kTH1, t, 8 * c, kHPitch, v + 8 * c);
         }
         barrier();
         if (t == 0) {
             tc::fence_after_sync();
-            tc::gemm_bf16(tm + kCZ2, sm + kTH1, sm + kTW2, 64, 64);
+            tc::gemm_kmajor(tm + kCZ2, sm + kTH1, kHPitch, sm + kTImg + kIW2, 64, 64, 64);
             tc::mma_commit(bar);
         }
         if (!(ok = wait())) break;
-        for (int c = 0; c < 4; ++c) {
-            float v[16];
-            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCZ2 + 16 * c), v);
-            for (int j = 0; j < 16; ++j) {
-                const float h = silu(v[j] + b2[16 * c + j]);
-                tc::st_bf16(sm + kTH2, t, 16 * c + j, 64, h);
-                tc::st_bf16(sm + kTH2T, 16 * c + j, t, 128, h);
-            }
+        {
+            float v[64];
+            load64(kCZ2, v);
+#pragma unroll
+            for (int j = 0; j < 64; ++j) v[j] = silu(v[j] + b2[j]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) st_row8(sm + kTH2, t, 8 * c, kHPitch, v + 8 * c);
         }
         barrier();
         if (t == 0) {
             tc::fence_after_sync();
-            tc::gemm_bf16(tm + kCZ3, sm + kTH2, sm + kTW3, 16, 64);
+            tc::gemm_kmajor(tm + kCZ3, sm + kTH2, kHPitch, sm + kTImg + kIW3, 64, 16, 64);
             tc::mma_commit(bar);
         }
         if (!(ok = wait())) break;
         // ---- loss and output error dY = 2 (y - t) / (n_total 7)
         float se = 0.0f;
         {
-            float v[16];
+            float v[16], dy[8];
             tc::tmem_ld16(tc::tmem_lane_addr(tm, kCZ3), v);
             const float sc = (float)(2.0 / (n_total * kOut));
+            dy[7] = 0.0f;
+#pragma unroll
             for (int k = 0; k < kOut; ++k) {
                 const float e = valid ? v[k] + b3[k] - tn[k] : 0.0f;
                 se += e * e;
-                const float dy = sc * e;
-                tc::st_bf16(sm + kTdZ3, t, k, 16, dy);
-                tc::st_bf16(sm + kTdZ3T, k, t, 128, dy);
+                dy[k] = sc * e;
             }
+            st_row8(sm + kTdZ3, t, 0, 16, dy);
         }
         for (int off = 16; off > 0; off >>= 1) se += __shfl_xor_sync(0xffffffffu, se, off);
         if (lane == 0) red[warp] = se;
-        // ---- dH2 = dY W3, dW3 (+ db3) = dY^T [H2, 1]
+        // ---- dH2 = dY W3 (waited for), dW3 (+ db3) = dY^T [H2, 1] (runs on)
         barrier();
         if (t == 0) {
             tc::fence_after_sync();
+            tc::gemm_kmajor(tm + kCdH2, sm + kTdZ3, 16, sm + kTImg + kIW3T, 16, 64, 16);
+            tc::mma_commit(bar);
+            tc::gemm_mnmajor(tm + kCdW3, sm + kTdZ3, 16, sm + kTH2, kHPitch, 80, 128);
             const float tile_loss = red[0] + red[1] + red[2] + red[3];
             if (part_loss) part_loss[blockIdx.x] = tile_loss;
             else atomicAdd(loss, tile_loss);
-            tc::gemm_bf16(tm + kCdH2, sm + kTdZ3, sm + kTW3T, 64, 16);
-            tc::gemm_bf16(tm + kCdW3, sm + kTdZ3T, sm + kTH2T, 80, 128);
-            tc::mma_commit(bar);
         }
         if (!(ok = wait())) break;
         // ---- dZ2 = dH2 * silu'(Z2)
-        for (int c = 0; c < 4; ++c) {
-            float dh[16], z[16];
-            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCdH2 + 16 * c), dh);
-            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCZ2 + 16 * c), z);
-            for (int j = 0; j < 16; ++j) {
-                const float d = dh[j] * silu_grad(z[j] + b2[16 * c + j]);
-                tc::st_bf16(sm + kTdZ2, t, 16 * c + j, 64, d);
-                tc::st_bf16(sm + kTdZ2T, 16 * c + j, t, 128, d);
-            }
+        {
+            float dh[64], z[64];
+            load64(kCdH2, dh);
+            load64(kCZ2, z);
+#pragma unroll
+            for (int j = 0; j < 64; ++j) dh[j] = dh[j] * silu_grad(z[j] + b2[j]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) st_row8(sm + kTdZ2, t, 8 * c, 64, dh + 8 * c);
         }
-        // ---- dH1 = dZ2 W2, dW2 (+ db2) = dZ2^T [H1, 1]
+        // ---- dH1 = dZ2 W2 (waited for), dW2 (+ db2) = dZ2^T [H1, 1] (runs on)
         barrier();
         if (t == 0) {
             tc::fence_after_sync();
-            tc::gemm_bf16(tm + kCdH1, sm + kTdZ2, sm + kTW2T, 64, 64);
-            tc::gemm_bf16(tm + kCdW2, sm + kTdZ2T, sm + kTH1T, 80, 128);
+            tc::gemm_kmajor(tm + kCdH1, sm + kTdZ2, 64, sm + kTImg + kIW2T, 64, 64, 64);
             tc::mma_commit(bar);
+            tc::gemm_mnmajor(tm + kCdW2, sm + kTdZ2, 64, sm + kTH1, kHPitch, 80, 128);
         }
         if (!(ok = wait())) break;
         // ---- dZ1 = dH1 * silu'(Z1)
-        for (int c = 0; c < 4; ++c) {
-            float dh[16], z[16];
-            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCdH1 + 16 * c), dh);
-            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCZ1 + 16 * c), z);
-            for (int j = 0; j < 16; ++j)
-                tc::st_bf16(sm + kTdZ1T, 16 * c + j, t, 128, dh[j] * silu_grad(z[j]));
+        {
+            float dh[64], z[64];
+            load64(kCdH1, dh);
+            load64(kCZ1, z);
+#pragma unroll
+            for (int j = 0; j < 64; ++j) dh[j] = dh[j] * silu_grad(z[j]);
+#pragma unroll
+            for (int c = 0; c < 8; ++c) st_row8(sm + kTdZ1, t, 8 * c, 64, dh + 8 * c);
         }
-        // ---- dW1 (+ db1 in column 3) = dZ1^T X
+        // ---- dW1 (+ db1 in column 3) = dZ1^T X; the commit covers every product so far
         barrier();
         if (t == 0) {
             tc::fence_after_sync();
-            tc::gemm_bf16(tm + kCdW1, sm + kTdZ1T, sm + kTXT, 16, 128);
+            tc::gemm_mnmajor(tm + kCdW1, sm + kTdZ1, 64, sm + kTX, 16, 16, 128);
             tc::mma_commit(bar);
         }
         if (!(ok = wait())) break;
-        // ---- accumulate this tile's weight gradients (rows = units: lanes 0-63)
+        // ---- this tile's weight gradients (rows = units: lanes 0-63)
         float* const own = part ? part + (size_t)blockIdx.x * kOffMean : nullptr;
-        auto put = [&](int idx, float val) {
-            if (own) own[idx] = val;
-            else atomicAdd(&grad[idx], val);
-        };
         if (warp < 2) {
             const int j = t;                    // unit of layers 1 and 2
-            for (int c = 0; c < 5; ++c) {       // dW2 columns 0-63, db2 in column 64
-                float v[16];
-                tc::tmem_ld16(tc::tmem_lane_addr(tm, kCdW2 + 16 * c), v);
-                for (int q = 0; q < 16; ++q) {
-                    const int col = 16 * c + q;
-                    if (col < 64) put(kOffW2 + 64 * j + col, v[q]);
-                    else if (col == 64) put(kOffB2 + j, v[q]);
-                }
+            float v[64], u[16], w1[16];
+            load64(kCdW2, v);                   // dW2 columns 0-63, db2 in column 64
+            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCdW2 + 64), u);
+            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCdW1), w1);
+            if (own) {
+#pragma unroll
+                for (int c = 0; c < 64; ++c) own[kOffW2 + 64 * c + j] = v[c];
+                own[kOffB2 + j] = u[0];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) own[kOffW1 + 4 * j + q] = w1[q];
+            } else {
+                for (int c = 0; c < 64; ++c) atomicAdd(&grad[kOffW2 + 64 * j + c], v[c]);
+                atomicAdd(&grad[kOffB2 + j], u[0]);
+                for (int q = 0; q < 4; ++q) atomicAdd(&grad[kOffW1 + 4 * j + q], w1[q]);
             }
-            float v[16];
-            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCdW1), v);
-            for (int q = 0; q < 4; ++q) put(kOffW1 + 4 * j + q, v[q]);
         }
-        if (warp == 0) {
-            for (int c = 0; c < 5; ++c) {       // dW3 rows 0-6, db3 in column 64
-                float v[16];
-                tc::tmem_ld16(tc::tmem_lane_addr(tm, kCdW3 + 16 * c), v);
-                if (lane < kOut)
-                    for (int q = 0; q < 16; ++q) {
-                        const int col = 16 * c + q;
-                        if (col < 64) put(kOffW3 + 64 * lane + col, v[q]);
-                        else if (col == 64) put(kOffB3 + lane, v[q]);
-                    }
+        if (warp == 0) {                        // dW3 rows 0-6, db3 in column 64
+            float v[64], u[16];
+            load64(kCdW3, v);
+            tc::tmem_ld16(tc::tmem_lane_addr(tm, kCdW3 + 64), u);
+            if (lane < kOut) {
+                if (own) {
+#pragma unroll
+                    for (int c = 0; c < 64; ++c) own[kOffW3 + kOut * c + lane] = v[c];
+                    own[kOffB3 + lane] = u[0];
+                } else {
+                    for (int c = 0; c < 64; ++c) atomicAdd(&grad[kOffW3 + 64 * lane + c], v[c]);
+                    atomicAdd(&grad[kOffB3 + lane], u[0]);
+                }
             }
         }
     } while (false);
     if (!ok) {
+        // no copy and no product of this CTA stays in flight (bounded)
         if (t == 0) atomicExch(err, 1);
-        tc::mbar_wait(bar, phase ^ 1u, kWaitCycles);
+        if (!have) tc::mbar_wait(ibar, 0u, kWaitCycles);
+        else {
+            if (t == 0) tc::mma_commit(bar);
+            tc::mbar_wait(bar, phase ^ 1u, kWaitCycles);
+            tc::mbar_wait(bar, phase, kWaitCycles);
+        }
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -761,29 +831,61 @@ __global__ void __launch_bounds__(128, 1) train_kernel(const float* __restrict__
     if (warp == 0) tc::tmem_dealloc(tm, kTrainCols);
 }
 
-// One Adam step (Kingma & Ba 2015) on every trained parameter; clears the gradient. c1, c2
-// are the bias corrections 1 - beta1^t, 1 - beta2^t. Also moves the step's summed squared
-// error into loss_hist (mean over n_total x 7) and clears it.
-__global__ void adam_kernel(float* __restrict__ P, const float* __restrict__ part, int n_tiles,
-                            float* __restrict__ m, float* __restrict__ v, float lr, float beta1,
-                            float beta2, float eps, float c1, float c2,
-                            const float* __restrict__ part_loss, float* loss_hist,
-                            float inv_count) {
-    // one Adam step from the tiles' gradient sums, added in tile order
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i == 0 && loss_hist) {
-        float l = 0.0f;
-        for (int b = 0; b < n_tiles; ++b) l += part_loss[b];
-        *loss_hist = l * inv_count;
+// One Adam step (Kingma & Ba 2015) on every trained parameter (slot order) from the tiles'
+// gradient sums, added in tile order: a block takes 32 slots, its eight warps bring their columns
+// of 128 tiles into shared memory at once (16 loads in flight a thread; one thread a slot walking
+// the tiles in device memory took twice the time), one warp adds them. c1, c2 are the bias
+// corrections 1 - beta1^t, 1 - beta2^t. Writes the new weight into the next step's image. The
+// last block adds the tiles' squared errors into loss_hist (mean over n_total x 7).
+constexpr int kAdamThreads = 256, kAdamTiles = 128;
+constexpr int kAdamBlocks = (kOffMean + 31) / 32 + 1;
+__global__ void __launch_bounds__(kAdamThreads) adam_kernel(
+        float* __restrict__ w, unsigned char* __restrict__ img, const float* __restrict__ part,
+        int n_tiles, float* __restrict__ m, float* __restrict__ v, float lr, float beta1,
+        float beta2, float eps, float c1, float c2, const float* __restrict__ part_loss,
+        float* loss_hist, float inv_count) {
+    __shared__ float col[kAdamTiles][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    tc::grid_dependency_wait();
+    tc::grid_launch_dependents();
+    const bool is_loss = blockIdx.x == kAdamBlocks - 1;
+    const int s = blockIdx.x * 32 + lane;
+    const bool on = is_loss ? lane == 0 && loss_hist != nullptr : s < kOffMean;
+    const float* src = is_loss ? part_loss : part + s;
+    const size_t stride = is_loss ? 1 : kOffMean;
+    float mo = 0.0f, vo = 0.0f, wo = 0.0f, g = 0.0f;
+    if (warp == 0 && on && !is_loss) {
+        mo = m[s];
+        vo = v[s];
+        wo = w[s];
     }
-    if (i >= kOffMean) return;
-    float g = 0.0f;
-    for (int b = 0; b < n_tiles; ++b) g += part[(size_t)b * kOffMean + i];
-    const float mi = beta1 * m[i] + (1.0f - beta1) * g;
-    const float vi = beta2 * v[i] + (1.0f - beta2) * g * g;
-    m[i] = mi;
-    v[i] = vi;
-    P[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    for (int b0 = 0; b0 < n_tiles; b0 += kAdamTiles) {
+        const int nb = n_tiles - b0 < kAdamTiles ? n_tiles - b0 : kAdamTiles;
+#pragma unroll
+        for (int k = 0; k < kAdamTiles / 8; ++k) {
+            const int b = warp + 8 * k;
+            if (on && b < nb) col[b][lane] = src[(size_t)(b0 + b) * stride];
+        }
+        __syncthreads();
+        if (warp == 0 && on) {
+#pragma unroll 8
+            for (int b = 0; b < nb; ++b) g += col[b][lane];
+        }
+        __syncthreads();
+    }
+    if (warp != 0 || !on) return;
+    if (is_loss) {
+        *loss_hist = g * inv_count;
+        return;
+    }
+    // (roundings written out: a run's bits do not hang on the compiler's choice of products)
+    const float mi = __fmaf_rn(1.0f - beta1, g, __fmul_rn(beta1, mo));
+    const float vi = __fmaf_rn(__fmul_rn(1.0f - beta2, g), g, __fmul_rn(beta2, vo));
+    m[s] = mi;
+    v[s] = vi;
+    const float wn = wo - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+    w[s] = wn;
+    image_store(img, slot_param(s), wn);
 }
 
 // n uniform samples of the input box (SplitMix64 stream `seed`: draws 3i, 3i+1, 3i+2) and

@@ -1,5 +1,5 @@
-"""Training kernels at the edges of their work split: the normalisation adds block sums of the
-whole device."""
+"""Training kernels at the edges of their work split: the Adam kernel brings 128 tiles' gradient
+sums into shared memory at a time, the normalisation adds block sums of the whole device."""
 import numpy as np
 import pytest
 import torch
@@ -22,6 +22,31 @@ def _data(n, seed):
     tg = torch.empty((n, 7), dtype=torch.float32, device=DEV)
     native.blacklight_mlp_dataset(n, seed, inp, tg)
     return inp, tg
+
+
+@pytest.mark.parametrize("tiles", [1, 127, 128, 129, 300])
+def test_adam_step_over_tile_counts(tiles):
+    """From zero moments the first step moves each parameter by lr g / (|g| + eps) against its
+    gradient; the loss is the gradient entry point's, summed in another order
+    (FP32: n 2^-24 relative at most, and 1e-5 for n <= 300 tiles of sums)."""
+    n = 128 * tiles
+    inp, tg = _data(n, 11 + tiles)
+    p = torch.empty(M.N_PARAMS, dtype=torch.float32, device=DEV)
+    native.blacklight_mlp_init(p, 3)
+    native.blacklight_mlp_normalise(inp, tg, p)
+    g = torch.empty_like(p)
+    loss = native.blacklight_mlp_grad(p, inp, tg, g)
+    q = p.clone()
+    hist = torch.zeros(1, dtype=torch.float32, device=DEV)
+    native.blacklight_mlp_train(q, inp, tg, n, 1, 1e-3, 1e-3, loss_history=hist)
+    gg = g[:M.OFF_MEAN].double().cpu().numpy()
+    step = (q - p).double().cpu().numpy()
+    big = np.abs(gg) > 1e-3 * np.abs(gg).max()
+    # the first step is lr g / (|g| + eps), eps = 1e-8; q - p carries the rounding of q (2^-24 |q|)
+    want = -1e-3 * gg[big] / (np.abs(gg[big]) + 1e-8)
+    np.testing.assert_allclose(step[:M.OFF_MEAN][big], want, rtol=1e-3)
+    assert np.all(step[M.OFF_MEAN:] == 0.0)
+    assert float(hist[0]) == pytest.approx(loss, rel=1e-5)
 
 
 @pytest.mark.parametrize("n", [64, 127, 129, 77825, 300001])
