@@ -374,7 +374,7 @@ __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ im
                     }
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        incm[c] = c == 4 ? 0.0f : hh * acc[c];
+                        incm[c] = c == 4 ? 0.0f : __fmul_rn(hh, acc[c]);
                         ym[c] = c == 4 ? y[4] : y[c] + from_float(incm[c]);
                         ymf[c] = to_float_rn(ym[c]);
                     }
@@ -432,20 +432,22 @@ __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ im
                     }
                 } else if constexpr (kFRec) {
                     // the quartic through y0, y1, h f0, h f1 and y_mid (Shampine 1986), in FP32
-                    // about y0 (y_mid - y0 is the midpoint increment)
+                    // about y0 (y_mid - y0 is the midpoint increment), roundings written out
                     const float hf = to_float_rn(h);
                     float y0f[8], d0f[8], c2f[8], c3f[8], c4f[8];
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {
-                        const float d0 = c == 4 ? 0.0f : hf * to_float_rn(KX(0, c));
-                        const float D1 = (c == 4 ? 0.0f : to_float_rn(y5[c] - y[c])) - d0;
-                        const float D2 = (c == 4 ? 0.0f : hf * to_float_rn(KX(6, c))) - d0;
-                        const float D3 = incm[c] - 0.5f * d0;
+                        const float k0 = c == 4 ? 0.0f : to_float_rn(KX(0, c));
+                        const float k6 = c == 4 ? 0.0f : to_float_rn(KX(6, c));
+                        const float d0 = __fmul_rn(hf, k0);
+                        const float D1 = __fadd_rn(c == 4 ? 0.0f : to_float_rn(y5[c] - y[c]), -d0);
+                        const float D2 = __fmaf_rn(hf, k6, -d0);
+                        const float D3 = __fmaf_rn(-0.5f, d0, incm[c]);
                         y0f[c] = to_float_rn(y[c]);
                         d0f[c] = d0;
-                        c2f[c] = -5.0f * D1 + D2 + 16.0f * D3;
-                        c3f[c] = 14.0f * D1 - 3.0f * D2 - 32.0f * D3;
-                        c4f[c] = -8.0f * D1 + 2.0f * D2 + 16.0f * D3;
+                        c2f[c] = __fmaf_rn(16.0f, D3, __fmaf_rn(-5.0f, D1, D2));
+                        c3f[c] = __fmaf_rn(-32.0f, D3, __fmaf_rn(14.0f, D1, -__fmul_rn(3.0f, D2)));
+                        c4f[c] = __fmaf_rn(16.0f, D3, __fmaf_rn(-8.0f, D1, __fmul_rn(2.0f, D2)));
                     }
                     ok = emit_quartic_f(sink, wray, nrec, y0f, d0f, c2f, c3f, c4f, nsub, hl);
                 } else {
