@@ -379,7 +379,7 @@ struct DevInfo {
     int mi_occ[2] = {0, 0};         // learned-coefficient model inputs: [fast, slow light]
     int pre_occ[2] = {0, 0};        // FP64 sample pass: [fast, slow light]
     int tr_pre_occ[2] = {0, 0};     // FP64 transfer after the sample pass: [fast, slow light]
-    int fwd_pool_occ = 0;           // the model over the sample pool
+    int fwd_list_occ = 0;           // the model over the work list
     int rk_occ[2] = {0, 0};         // RK2/RK4 geodesic kernel: [double records, float records]
     // CTAs per SM of the transfer variant a launch uses
     int transfer(int precision, const float* mlp, int feat) const {
@@ -447,7 +447,7 @@ int dev_info(DevInfo& out) {
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.tr_mlp_occ[1], bl::transfer_learned_kernel<true>, 128, 0));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.mi_occ[0], bl::mlp_inputs_kernel<false>, 128, 0));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.mi_occ[1], bl::mlp_inputs_kernel<true>, 128, 0));
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.fwd_pool_occ, bl::mlp::forward_pool_kernel, 128, 0));
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.fwd_list_occ, bl::mlp::forward_list_kernel, 128, 0));
         for (int i = 0; i < 2; ++i)
             if (di.mi_occ[i] < 1) di.mi_occ[i] = 1;
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.pre_occ[0], bl::fp64_samples_kernel<false>, 128, 0));
@@ -458,7 +458,7 @@ int dev_info(DevInfo& out) {
             if (di.pre_occ[i] < 1) di.pre_occ[i] = 1;
             if (di.tr_pre_occ[i] < 1) di.tr_pre_occ[i] = 1;
         }
-        if (di.fwd_pool_occ < 1) di.fwd_pool_occ = 1;
+        if (di.fwd_list_occ < 1) di.fwd_list_occ = 1;
         for (int i = 0; i < 2; ++i)
             if (di.tr_mlp_occ[i] < 1) di.tr_mlp_occ[i] = 1;
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.rk_occ[0], bl::geodesic_rk_kernel<double>, 128, 0));
@@ -671,31 +671,46 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                 BL_CUDA(cudaGetLastError());
                 return 0;
             };
+            // the order after a first pass over the samples: warp-sized ray groups by the work from
+            // each ray's farthest plasma sample to the camera
+            auto order_by_plasma = [&]() -> int {
+                BL_CUDA(cudaMemsetAsync(thist, 0, sizeof(unsigned int) * bl::kCostBuckets, st));
+                bl::transport_key_kernel<<<sgrid, 256, 0, st>>>(
+                    (const int32_t*)(ws + L.tfirst), (const int32_t*)(ws + L.tnpl), tkey, cfg.bs, b, e, thist);
+                bl::work_scan_kernel<<<1, 1024, 0, st>>>(thist);
+                bl::work_scatter_kernel<bl::kTransportGroup><<<sgrid, 256, 0, st>>>(tkey, cfg.bs, b, e, thist, tperm);
+                g_launches += 3;
+                BL_CUDA(cudaGetLastError());
+                return 0;
+            };
             if (mlp) {
-                // learned coefficients in three passes: the model inputs of every record, the
-                // model over the record pool in full tensor-core tiles, then the transfer
-                // reading the model's outputs
+                // learned coefficients in three passes: the samples with plasma and their model
+                // inputs, the model over the list of those, then the transfer reading the model's
+                // outputs, its rays longest first by that list
                 float* mpool = (float*)(ws + L.pool);
                 float* my = (float*)(ws + L.mlp_y);
+                int32_t* tfirst = (int32_t*)(ws + L.tfirst);
+                int32_t* tnpl = (int32_t*)(ws + L.tnpl);
+                // per wave ray: farthest plasma sample -1 and no plasma samples until found
+                BL_CUDA(cudaMemsetAsync(tfirst, 0xff, sizeof(int32_t) * (size_t)(e - b), st));
+                BL_CUDA(cudaMemsetAsync(tnpl, 0, sizeof(int32_t) * (size_t)(e - b), st));
                 const unsigned mi_grid = (unsigned)(di.sms * di.mi_occ[slow ? 1 : 0]);
                 if (slow)
                     bl::mlp_inputs_kernel<true><<<mi_grid, 128, 0, st>>>(
-                        d_desc, n_images, b, e, hdr, mpool, chunks, ctr, cfg.bs);
+                        d_desc, n_images, b, e, hdr, mpool, chunks, ctr, cfg.bs, my, tfirst, tnpl);
                 else
                     bl::mlp_inputs_kernel<false><<<mi_grid, 128, 0, st>>>(
-                        d_desc, n_images, b, e, hdr, mpool, chunks, ctr, cfg.bs);
+                        d_desc, n_images, b, e, hdr, mpool, chunks, ctr, cfg.bs, my, tfirst, tnpl);
                 ++g_launches;
                 BL_CUDA(cudaGetLastError());
-                bl::mlp::forward_pool_kernel<<<(unsigned)(di.sms * di.fwd_pool_occ), 128, 0, st>>>(
-                    mlp, fpool, &ctr->pool_next, (unsigned long long)L.pool_chunks, my,
-                    &ctr->mlp_timeouts);
+                bl::mlp::forward_list_kernel<<<(unsigned)(di.sms * di.fwd_list_occ), 128, 0, st>>>(
+                    mlp, &ctr->mlp_rows, my, &ctr->mlp_timeouts);
                 ++g_launches;
                 BL_CUDA(cudaGetLastError());
-                if (cfg.order_transfer && (rc = order_by_records())) return rc;
+                if ((rc = order_by_plasma())) return rc;
                 launch_transfer<float, float>(cfg.feat | bl::kFMlp, tr_grid, st, d_desc, n_images, b,
                                               e, hdr, fpool, chunks, ctr, cfg.bs,
-                                              bl::SideIn{my, mlp, nullptr, nullptr, nullptr,
-                                                         cfg.order_transfer ? tperm : nullptr});
+                                              bl::SideIn{my, mlp, nullptr, nullptr, tfirst, tperm});
             } else if (precision != BL_PREC_FP64) {
                 if (cfg.order_transfer && (rc = order_by_records())) return rc;
                 launch_transfer<float, float>(cfg.feat, tr_grid, st, d_desc, n_images, b, e, hdr,
@@ -713,7 +728,6 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                 // per wave ray: farthest plasma sample -1 and no plasma samples until found
                 BL_CUDA(cudaMemsetAsync(tfirst, 0xff, sizeof(int32_t) * (size_t)(e - b), st));
                 BL_CUDA(cudaMemsetAsync(tnpl, 0, sizeof(int32_t) * (size_t)(e - b), st));
-                BL_CUDA(cudaMemsetAsync(thist, 0, sizeof(unsigned int) * bl::kCostBuckets, st));
                 const unsigned pre_grid = (unsigned)(di.sms * di.pre_occ[slow ? 1 : 0]);
                 if (slow)
                     bl::fp64_samples_kernel<true><<<pre_grid, 128, 0, st>>>(
@@ -723,11 +737,9 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                     bl::fp64_samples_kernel<false><<<pre_grid, 128, 0, st>>>(
                         d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs, pre, pflag,
                         tfirst, tnpl);
-                bl::transport_key_kernel<<<sgrid, 256, 0, st>>>(tfirst, tnpl, tkey, cfg.bs, b, e, thist);
-                bl::work_scan_kernel<<<1, 1024, 0, st>>>(thist);
-                bl::work_scatter_kernel<bl::kTransportGroup><<<sgrid, 256, 0, st>>>(tkey, cfg.bs, b, e, thist, tperm);
-                g_launches += 4;
+                ++g_launches;
                 BL_CUDA(cudaGetLastError());
+                if ((rc = order_by_plasma())) return rc;
                 if (!tr_set && e - b <= bl::kDeep64Rays * di.sms)
                     bl::transport64_wide_kernel<<<(unsigned)(di.sms * bl::kTransport64WideCtas), 128, 0, st>>>(
                         d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs,

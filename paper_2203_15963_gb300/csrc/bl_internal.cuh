@@ -108,7 +108,7 @@ struct BlockSource {
 };
 
 // Side inputs of the transfer variants that split their per-sample work over passes: the
-// learned model's outputs (8 floats a pool record) and its parameters, or, in the FP64 form,
+// learned model's outputs (8 floats a row of its work list) and its parameters, or, in the FP64 form,
 // each record's precomputed scaled coefficients and fluid-frame basis (24 doubles a pool
 // record) with a flag byte (1: the sample carries plasma).
 struct SideIn {
@@ -116,7 +116,7 @@ struct SideIn {
     const float* mlp_params;
     const double* pre;
     const unsigned char* pre_flag;
-    const int32_t* first;    // FP64 transport pass: each ray's farthest plasma sample, or -1
+    const int32_t* first;    // each ray's farthest plasma sample, or -1 (learned and FP64 forms)
     const int32_t* perm;     // the transfer's ray order (wave ray indices), or nullptr
 };
 constexpr int kPreVals = 24;
@@ -126,6 +126,7 @@ struct Counters {
     unsigned long long next_ray_tr;
     unsigned long long pool_next;
     unsigned long long next_ray_mi;    // learned-coefficient model inputs: rays handed out
+    unsigned long long mlp_rows;       // learned-coefficient work list: rows written
     unsigned long long bad_rays;
     unsigned long long mlp_timeouts;   // CTAs whose tensor-core wait ran out (never expected)
 };

@@ -1841,6 +1841,8 @@ __device__ __forceinline__ int64_t record_index(const int32_t* __restrict__ chun
 // exact constant-coefficient Stokes step, and S -> N. A lane whose ray is done reads out the
 // Stokes parameters in the camera basis (H, V) and takes the next ray.
 // ---------------------------------------------------------------------------------------
+// What the learned-coefficient form's first pass found at a sample (a record's last value).
+enum : unsigned { kSampleEmpty = 0u, kSampleExact = 1u, kSampleModel = 2u };
 // Features of a transfer-kernel variant (compile-time, so that each variant carries only the
 // registers it needs).
 enum { kFSlow = 1, kFUnpol = 2, kFAux = 4, kFMlp = 8 };
@@ -1950,11 +1952,11 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
     constexpr bool kSlow = (kF & kFSlow) != 0;
     constexpr bool kUnpol = (kF & kFUnpol) != 0;
     constexpr bool kAux = (kF & kFAux) != 0;
-    // learned coefficients: the model's outputs come from the pool pass (mlp_y, 8 floats a
-    // record), the record's last value flags the samples the model evaluated
+    // learned coefficients: the first pass (mlp_inputs_kernel) has found the samples that carry
+    // plasma; the model's outputs are in mlp_y, 8 floats a row of its work list
     constexpr bool kMlp = (kF & kFMlp) != 0;
     static_assert(!kMlp || std::is_same<R, float>::value, "the learned model needs FP32 records");
-    constexpr bool kIdx = kMlp;   // the transfer needs each record's pool index
+    constexpr int kGroup = kMlp ? kTransportGroup : kFusedGroup;
     // the stencil field test of plasma_at: always in the FP64 form; in FP32 where the rays are
     // not queued by record count -- that order predicts a ray's cost from its records, which
     // stops holding once field-free records are cheap (nine 256^2 images, fast form: cell-layout
@@ -1965,10 +1967,9 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
     // register budgets of the slow-light, auxiliary-image and learned variants.
     constexpr bool kFieldTestable = sizeof(T) == sizeof(double) || (!kSlow && !kAux && !kMlp);
     const bool field_test = kFieldTestable && (sizeof(T) == sizeof(double) || side.perm == nullptr);
-    int64_t nxt_k = 0;
     const int64_t re = wave_end(bs, ray_end);
     const int64_t n_rays = re > ray_begin ? re - ray_begin : 0;
-    const int64_t total_rays = side.perm ? ordered_total<kFusedGroup>(n_rays) : n_rays;
+    const int64_t total_rays = side.perm ? ordered_total<kGroup>(n_rays) : n_rays;
     int64_t wray = 0;
     bool active = false;
     int64_t ray = 0, opix = 0;
@@ -1991,7 +1992,7 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
             if ((int64_t)got >= total_rays) exhausted = true;
             else {
                 // the wave's rays in the order of their record counts where there is one
-                wray = side.perm ? ordered_ray<kFusedGroup>(side.perm, got, n_rays) : (int64_t)got;
+                wray = side.perm ? ordered_ray<kGroup>(side.perm, got, n_rays) : (int64_t)got;
                 ray = ray_begin + wray;
             }
         }
@@ -2019,9 +2020,10 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
                 }
                 continue;
             }
-            idx = transfer_start(hd);
+            // (the learned form from the farthest plasma sample: N = 0 beyond it)
+            if constexpr (kMlp) idx = side.first[wray] > 0 ? side.first[wray] : 0;
+            else idx = transfer_start(hd);
             load_record<R>(record_ptr(pool, chunks, wray, idx), nxt);
-            if constexpr (kIdx) nxt_k = record_index(chunks, wray, idx);
             kt = (T)hd.kt;
             nu_norm = (T)(hd.nnorm * im.freq);
             a = ic<T>(im, kcSpin);
@@ -2042,19 +2044,17 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
         const bool finishing = idx < 0;
         T cur[kRecVals];
         T nxt_t = T(0);   // the sample's coordinate time
-        int64_t cur_k = 0;
-        bool cur_flag = false;
+        unsigned cur_row = 0u, cur_what = 0u;
         if (!finishing) {
             // record idx was prefetched into nxt; start fetching idx - 1 before using it
 #pragma unroll
             for (int c = 0; c < kRecVals; ++c) cur[c] = (T)nxt[c];
             nxt_t = (T)nxt[13];
-            if constexpr (kIdx) cur_k = nxt_k;
-            if constexpr (kMlp) cur_flag = __float_as_uint((float)nxt[15]) != 0u;
-            if (idx > 0) {
-                load_record<R>(record_ptr(pool, chunks, wray, idx - 1), nxt);
-                if constexpr (kIdx) nxt_k = record_index(chunks, wray, idx - 1);
+            if constexpr (kMlp) {
+                cur_row = __float_as_uint((float)nxt[14]);
+                cur_what = __float_as_uint((float)nxt[15]);
             }
+            if (idx > 0) load_record<R>(record_ptr(pool, chunks, wray, idx - 1), nxt);
         }
         if (!kUnpol && started) {
             // merged N half-steps from the previous sample to this one (to the camera node on
@@ -2090,7 +2090,7 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
             active = false;
             continue;
         }
-        {
+        if (!kMlp || cur_what != kSampleEmpty) {
             const T xs[3] = {cur[0], cur[1], cur[2]};
             KSGeom<T> G;
             ks_geom<T>(xs[0], xs[1], xs[2], a, m, flat, false, G);
@@ -2108,10 +2108,10 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
                 bool learned = false;
                 if constexpr (kMlp) {
                     const mlp::ModelIn mi = mlp::model_inputs(P.th, P.bg, nu_fl, cth);
-                    if (cur_flag && mi.ok && P.ne > T(0)) {
+                    if (cur_what == kSampleModel && mi.ok && P.ne > T(0)) {
                         // (loaded here: loading them one sample ahead with the record measured
                         // slower, 61.2 against 58.9 ms at 1024^2)
-                        const float4* yq = reinterpret_cast<const float4*>(mlp_y + 8 * cur_k);
+                        const float4* yq = reinterpret_cast<const float4*>(mlp_y + 8 * (size_t)cur_row);
                         const float4 y0 = __ldg(yq), y1 = __ldg(yq + 1);
                         const float y[7] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z};
                         float o[7];
@@ -2622,63 +2622,198 @@ __global__ void __launch_bounds__(128, kTransport64WideCtas) transport64_wide_ke
 }
 
 // ---------------------------------------------------------------------------------------
-// Learned coefficients, first pass: the model inputs of every sample record. One warp takes a
-// ray, its lanes 32 consecutive records at a time (the records of a chunk lie together in the
-// pool): geometry, plasma state and the fluid-frame frequency and pitch angle at the sample,
-// as the transfer computes them, then the model's input row (mlp::input_row) into the record's
-// last 8 bytes -- zeros where the sample has no plasma or lies outside the model's domain.
+// Learned coefficients, first pass: which samples carry plasma, and their model inputs. Work is
+// compacted per warp as in the FP64 sample pass: a warp takes rays in turn, tests a chunk of 32
+// records at a time by position alone (the grid's radial shell with 1e-4 margins, the stencil
+// certainly without magnetic field; the next chunk's positions are loaded meanwhile), queues the
+// records that may carry plasma in shared memory and evaluates 32 of them at a time, whatever
+// rays they belong to: geometry, plasma state, fluid-frame frequency and pitch angle as the
+// transfer computes them. A record's last value says what the later passes find there:
+// kSampleEmpty (no plasma; the geodesic kernels write it so), kSampleExact (plasma outside the
+// model's domain) or kSampleModel, with the sample's row of the model's work list in the value
+// before it. The rows wait in shared memory until 128 are together, so the list fills densely
+// with one atomic for each 128, and the model pass neither scans the pool nor holds empty rows.
+// Each ray's farthest plasma sample and its number of plasma samples (atomics, one a ray and
+// batch; tfirst -1 and tnpl 0 beforehand) start and order the transfer. Bound by the latency of
+// the record and stencil reads: 10.7 ms at 1024^2 on the 512x256x256 torus (11.1 without the
+// work list, the order's inputs and the start they buy; one warp a ray with the list 14.5).
 // ---------------------------------------------------------------------------------------
+struct LearnedItem {
+    float* rec;
+    int32_t wray, idx, q, pad_;
+};
+constexpr int kListFlush = 128, kListQueue = kListFlush + 31;
 template <bool kSlow>
-__global__ void __launch_bounds__(128) mlp_inputs_kernel(const ImageDesc* __restrict__ imgs,
+__global__ void __launch_bounds__(128, 6) mlp_inputs_kernel(const ImageDesc* __restrict__ imgs,
                                                          int n_images, int64_t ray_begin,
                                                          int64_t ray_end,
                                                          const RayHdr* __restrict__ hdr,
                                                          float* __restrict__ pool,
                                                          const int32_t* __restrict__ chunks,
-                                                         Counters* ctr, BlockSource bs) {
+                                                         Counters* ctr, BlockSource bs,
+                                                         float* __restrict__ mlp_y,
+                                                         int32_t* __restrict__ tfirst,
+                                                         int32_t* __restrict__ tnpl) {
     using T = float;
+    __shared__ LearnedItem items[4][kSampleQueue];
+    __shared__ uint2 rows[4][kListQueue];
+    __shared__ float* recs[4][kListQueue];
     const int lane = threadIdx.x & 31;
-    const int64_t re = wave_end(bs, ray_end);
-    const int64_t total_rays = re > ray_begin ? re - ray_begin : 0;
-    while (true) {
-        unsigned long long got = 0;
-        if (lane == 0) got = atomicAdd(&ctr->next_ray_mi, 1ull);
-        got = __shfl_sync(0xffffffffu, got, 0);
-        if ((int64_t)got >= total_rays) break;
-        const int64_t wray = (int64_t)got, ray = ray_begin + wray;
-        int q, pi, pj;
-        int64_t opix;
-        setup_ray(imgs, n_images, bs, ray, q, opix, pi, pj);
-        const RayHdr hd = hdr[wray];
-        if (hd.status == BL_RAY_OVERFLOW || hd.nrec == 0) continue;
-        const ImageDesc& im = imgs[q];
-        const T kt = (T)hd.kt, nu_norm = (T)(hd.nnorm * im.freq);
-        const T a = ic<T>(im, kcSpin), m = ic<T>(im, kcMass);
-        const bool flat = im.flat != 0;
-        for (int32_t base = 0; base < hd.nrec; base += 32) {
-            const int32_t idx = base + lane;
-            if (idx >= hd.nrec) break;
-            float* rec = pool + record_index(chunks, wray, idx) * RecStride<float>::v;
+    LearnedItem* const Q = items[threadIdx.x >> 5];
+    uint2* const row_q = rows[threadIdx.x >> 5];
+    float** const rec_q = recs[threadIdx.x >> 5];
+    int qn = 0, rn = 0;   // items and rows waiting (warp-uniform)
+    auto flush = [&]() {
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(&ctr->mlp_rows, (unsigned long long)rn);
+        base = __shfl_sync(0xffffffffu, base, 0);
+        __syncwarp();
+        for (int i = lane; i < rn; i += 32) {
+            *reinterpret_cast<uint2*>(mlp_y + 8 * (base + i)) = row_q[i];
+            *reinterpret_cast<uint2*>(rec_q[i] + 14) = make_uint2((unsigned)(base + i), kSampleModel);
+        }
+        __syncwarp();
+        rn = 0;
+    };
+    // the queue's first n items, lane i taking item i
+    auto evaluate = [&](int n) {
+        unsigned what = kSampleEmpty;
+        uint2 row = make_uint2(0u, 0u);
+        float* rec = nullptr;
+        int32_t wray = -1, idx = -1;
+        if (lane < n) {
+            const LearnedItem it = Q[lane];
+            rec = it.rec;
+            wray = it.wray;
+            idx = it.idx;
+            const ImageDesc& im = imgs[it.q];
             float v[RecStride<float>::v];
             load_record<float>(rec, v);
             const T xs[3] = {v[0], v[1], v[2]};
             KSGeom<T> G;
-            ks_geom<T>(xs[0], xs[1], xs[2], a, m, flat, false, G);
+            ks_geom_pinned(xs[0], xs[1], xs[2], ic<T>(im, kcSpin), ic<T>(im, kcMass), im.flat != 0, G);
             Plasma<T> P;
-            uint2 row = make_uint2(0u, 0u);
-            if (plasma_at<T, kSlow>(im, xs, v[13], G, P, false)) {
-                const T kl[4] = {kt, v[3], v[4], v[5]};
+            if (plasma_at<T, kSlow>(im, xs, v[13], G, P, true)) {
+                const RayHdr hd = hdr[wray];
+                const T kl[4] = {(T)hd.kt, v[3], v[4], v[5]};
                 const T kdu = kl[0] * P.u[0] + kl[1] * P.u[1] + kl[2] * P.u[2] + kl[3] * P.u[3];
                 const T kdb = kl[0] * P.b[0] + kl[1] * P.b[1] + kl[2] * P.b[2] + kl[3] * P.b[3];
-                const T nu_fl = nu_norm * (-kdu);
+                const T nu_fl = (T)(hd.nnorm * im.freq) * (-kdu);
                 T cth = fq(kdb, (-kdu) * fsqrt(P.bsq));
                 cth = cth > T(1) ? T(1) : (cth < T(-1) ? T(-1) : cth);
                 const mlp::ModelIn mi = mlp::model_inputs(P.th, P.bg, nu_fl, cth);
-                if (mi.ok && P.ne > T(0)) row = mlp::input_row(mi.f);
+                what = kSampleExact;
+                if (mi.ok && P.ne > T(0)) {
+                    what = kSampleModel;
+                    row = mlp::input_row(mi.f);
+                } else {
+                    *reinterpret_cast<uint2*>(rec + 14) = make_uint2(0u, kSampleExact);
+                }
             }
-            *reinterpret_cast<uint2*>(rec + 14) = row;
         }
+        const bool plasma = what != kSampleEmpty;
+        const unsigned model = __ballot_sync(0xffffffffu, what == kSampleModel);
+        if (what == kSampleModel) {
+            const int at = rn + __popc(model & ((1u << lane) - 1u));
+            row_q[at] = row;
+            rec_q[at] = rec;
+        }
+        rn += __popc(model);
+        // per ray of the batch: its plasma samples lie at increasing lanes (records enter the
+        // queue in order), so the highest lane of a ray's group holds its farthest one
+        const unsigned grp = __match_any_sync(0xffffffffu, plasma ? wray : -1 - lane);
+        if (plasma && lane == 31 - __clz(grp)) {
+            atomicMax(&tfirst[wray], idx);
+            atomicAdd(&tnpl[wray], __popc(grp));
+        }
+        if (rn >= kListFlush) flush();
+    };
+    const int64_t re = wave_end(bs, ray_end);
+    const int64_t total_rays = re > ray_begin ? re - ray_begin : 0;
+    int64_t wray = 0;
+    int32_t base = 0, nrec = 0, cid = 0;
+    int q = 0;
+    float aa = 0.0f, r2lo = 0.0f, r2hi = 0.0f;
+    float4 pos = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    bool exhausted = false;
+    while (true) {
+        if (base >= nrec && !exhausted) {
+            unsigned long long got = 0;
+            if (lane == 0) got = atomicAdd(&ctr->next_ray_mi, 1ull);
+            got = __shfl_sync(0xffffffffu, got, 0);
+            if ((int64_t)got >= total_rays) {
+                exhausted = true;
+            } else {
+                wray = (int64_t)got;
+                int pi, pj;
+                int64_t opix;
+                setup_ray(imgs, n_images, bs, ray_begin + wray, q, opix, pi, pj);
+                const RayHdr hd = hdr[wray];
+                base = 0;
+                nrec = 0;
+                if (hd.status != BL_RAY_OVERFLOW && hd.nrec > 0) {
+                    const ImageDesc& im = imgs[q];
+                    aa = (float)(im.spin * im.spin);
+                    r2lo = (float)(im.r_min * im.r_min * (1.0 - 1e-4));
+                    r2hi = (float)(im.r_max * im.r_max * (1.0 + 1e-4));
+                    nrec = hd.last_in + 1 < hd.nrec ? hd.last_in + 1 : hd.nrec;
+                }
+            }
+        }
+        if (base < nrec) {
+            // chunk number base / 32 of the ray: lanes hold 32 chunk ids at a time
+            const int cj = (base / kChunk) & 31;
+            if (cj == 0) {
+                const int c = base / kChunk + lane;
+                cid = c * kChunk < nrec ? chunks[wray * kMaxChunks + c] : 0;
+            }
+            const int32_t idx = base + lane;
+            float* rec = pool + ((int64_t)__shfl_sync(0xffffffffu, cid, cj) * kChunk + lane) * RecStride<float>::v;
+            if (base == 0 && idx < nrec) pos = __ldg(reinterpret_cast<const float4*>(rec));
+            const float4 v = pos;
+            // the next chunk's positions (its id is at hand unless 32 ids are used up)
+            const int cn = (cj + 1) & 31;
+            const int32_t nid = __shfl_sync(0xffffffffu, cid, cn);
+            if (idx + kChunk < nrec) {
+                const int64_t nc = cn != 0 ? nid : chunks[wray * kMaxChunks + base / kChunk + 1];
+                pos = __ldg(reinterpret_cast<const float4*>(pool + (nc * kChunk + lane) * RecStride<float>::v));
+            }
+            bool cand = false;
+            if (idx < nrec) {
+                const float qq = v.x * v.x + v.y * v.y + v.z * v.z - aa;
+                const float r2 = 0.5f * (qq + sqrtf(qq * qq + 4.0f * aa * v.z * v.z));
+                cand = r2 >= r2lo && r2 <= r2hi;
+                // a stencil without magnetic field holds no plasma (stencil_field_free);
+                // one snapshot only
+                if (!kSlow && cand) cand = !stencil_field_free(imgs[q], v.x, v.y, v.z, r2, aa);
+            }
+            const unsigned mask = __ballot_sync(0xffffffffu, cand);
+            if (cand) {
+                LearnedItem& it = Q[qn + __popc(mask & ((1u << lane) - 1u))];
+                it.rec = rec;
+                it.wray = (int32_t)wray;
+                it.idx = idx;
+                it.q = q;
+            }
+            qn += __popc(mask);
+            base += kChunk;
+            __syncwarp();
+        }
+        if (qn >= 32 || (exhausted && qn > 0)) {
+            const int n = qn < 32 ? qn : 32;
+            evaluate(n);
+            __syncwarp();
+            LearnedItem keep;
+            const bool moves = lane < qn - n;
+            if (moves) keep = Q[n + lane];
+            __syncwarp();
+            if (moves) Q[lane] = keep;
+            qn -= n;
+            __syncwarp();
+        }
+        if (exhausted && qn == 0) break;
     }
+    if (rn > 0) flush();
 }
 
 // ---------------------------------------------------------------------------------------

@@ -158,6 +158,29 @@ __device__ __forceinline__ void ks_geom(T x, T y, T z, T a, T m, bool flat, bool
     }
 }
 
+// ks_geom in FP32 without derivatives, its roundings written out, for the learned form's model
+// inputs: their bf16 rounding turns a last-bit difference of the geometry into one of 2^-9 in the
+// network, so the inputs are formed from the same bits whatever kernel the call is inlined into.
+__device__ __forceinline__ void ks_geom_pinned(float x, float y, float z, float a, float m, bool flat,
+                                               KSGeom<float>& G) {
+    const float aa = __fmul_rn(a, a), aaz = __fmul_rn(aa, z);
+    const float q = __fadd_rn(__fmaf_rn(z, z, __fmaf_rn(x, x, __fmul_rn(y, y))), -aa);
+    const float D2 = __fmaf_rn(__fmul_rn(4.0f, aaz), z, __fmul_rn(q, q));
+    const float r2 = __fmul_rn(0.5f, __fmaf_rn(D2, rsqrt(D2), q));
+    const float ir = rsqrt(r2);
+    const float r = __fmul_rn(r2, ir);
+    const float s4 = __fmaf_rn(aaz, z, __fmul_rn(r2, r2));
+    const float P = __fadd_rn(r2, aa);
+    const float iPs = 1.0f / __fmul_rn(P, s4);
+    const float is4 = __fmul_rn(P, iPs), iP = __fmul_rn(s4, iPs);
+    G.r = r;
+    G.f = flat ? 0.0f : __fmul_rn(__fmul_rn(__fmul_rn(__fmul_rn(2.0f, m), r), r2), is4);
+    G.l[0] = 1.0f;
+    G.l[1] = __fmul_rn(__fmaf_rn(a, y, __fmul_rn(r, x)), iP);
+    G.l[2] = __fmul_rn(__fmaf_rn(r, y, -__fmul_rn(a, x)), iP);
+    G.l[3] = __fmul_rn(z, ir);
+}
+
 // r of a CKS point (Eq. cks_aux:r).
 template <class T>
 __device__ __forceinline__ T ks_r(T x, T y, T z, T a) {
