@@ -431,11 +431,11 @@ int dev_info(DevInfo& out) {
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGeoSmem));
         BL_CUDA(cudaFuncSetAttribute(bl::geodesic64_kernel<float>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGeoSmem));
-        BL_CUDA(cudaFuncSetAttribute(bl::geodesic_kernel<float, bl::df64>,
+        BL_CUDA(cudaFuncSetAttribute(bl::geodesic_df_kernel,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGeoSmem));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo_blocks[0], bl::geodesic_kernel_fp64, 128, 0));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo_blocks[1], bl::geodesic64_kernel<float>, 128, kGeoSmem));
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo_blocks[2], bl::geodesic_kernel<float, bl::df64>, 128, kGeoSmem));
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo_blocks[2], bl::geodesic_df_kernel, 128, kGeoSmem));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.geo64_wide, bl::geodesic64_kernel<double>, 128, kGeoSmem));
         if (di.geo64_wide < 1) di.geo64_wide = 1;
         for (int i = 0; i < 3; ++i)
@@ -584,7 +584,7 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
         // few rays: at most one CTA an SM, so each runs at its latency
         const int64_t pg = (nb + 127) / 128, pcap = (int64_t)di.sms * di.geo_blocks[2];
         bl::RecordSink<float> psink{nullptr, nullptr, 0ull, pctr};
-        bl::geodesic_kernel<float, bl::df64><<<(unsigned)(pg < pcap ? pg : pcap), 128, kGeoSmem, st>>>(
+        bl::geodesic_df_kernel<<<(unsigned)(pg < pcap ? pg : pcap), 128, kGeoSmem, st>>>(
             pdesc, n_images, 0, nb, (bl::RayHdr*)(ws + po.hdr), psink, 0, pbs,
             (const bl::RayInit*)(ws + po.init));
         bl::cost_sort_kernel<<<1, 1024, 0, st>>>(pcost, plist, nb, psorted, pcount + 1);
@@ -643,7 +643,7 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                         d_desc, n_images, b, e, hdr, sink, record, cfg.bs,
                         geo_set ? 0 : di.sms);
                 else
-                    bl::geodesic_kernel<float, bl::df64><<<geo_grid, 128, kGeoSmem, st>>>(
+                    bl::geodesic_df_kernel<<<geo_grid, 128, kGeoSmem, st>>>(
                         d_desc, n_images, b, e, hdr, sink, record, cfg.bs, init);
             }
         }

@@ -43,7 +43,11 @@ __device__ __forceinline__ double min_nonneg(double a, double b) {
 __device__ __forceinline__ float to_float_rn(double x) {
     const int hi = __double2hiint(x);
     const unsigned ahi = (unsigned)hi & 0x7fffffffu;
-    if (ahi - 0x38100000u >= 0x47e00000u - 0x38100000u) return (float)x;
+    if (ahi - 0x38100000u >= 0x47e00000u - 0x38100000u) {
+        float f;   // (volatile: the compiler may not run the instruction ahead of the test)
+        asm volatile("cvt.rn.f32.f64 %0, %1;" : "=f"(f) : "d"(x));
+        return f;
+    }
     const unsigned long long v =
         ((unsigned long long)(ahi - 0x38000000u) << 32) | (unsigned)__double2loint(x);
     const unsigned long long q = v + 0x0fffffffull + ((v >> 29) & 1ull);
@@ -59,7 +63,11 @@ __device__ __forceinline__ float to_float_est(double x) {
 // float -> double, exact (zero and normal values by integer operations).
 __device__ __forceinline__ double from_float(float f) {
     const unsigned b = __float_as_uint(f), ab = b & 0x7fffffffu;
-    if (ab - 0x00800000u >= 0x7f800000u - 0x00800000u && ab != 0u) return (double)f;
+    if (ab - 0x00800000u >= 0x7f800000u - 0x00800000u && ab != 0u) {
+        double d;
+        asm volatile("cvt.f64.f32 %0, %1;" : "=d"(d) : "f"(f));
+        return d;
+    }
     const unsigned hi = (b & 0x80000000u) | (ab == 0u ? 0u : (ab >> 3) + 0x38000000u);
     return __hiloint2double((int)hi, (int)(ab << 29));
 }
@@ -79,9 +87,19 @@ __device__ __forceinline__ double mul3(double a, double b, double c) {
     return __dmul_rn(__dmul_rn(a, b), c);
 }
 
-// Eq. (geodesic) as geodesic_rhs_g writes it, in native double with its exact scalings folded
-// away: the same operations and roundings. d_c f is carried halved (F1, so that 1/2 L need not
-// be formed).
+// Eq. (geodesic) right-hand side; returns r at the evaluation point.
+// With g^ab = eta^ab - f l^a l^b and L = l^a k_a, dx^a/dl = g^ab k_b and
+// dk_c/dl = L (1/2 d_c f L + f d_c L), where d_c L is the derivative at fixed k. Instead of the
+// nine derivatives d_c l_b, d_c L is formed directly: with A = x k_x + y k_y and B = y k_x - x k_y,
+// l_x k_x + l_y k_y = (r A + a B) / (r^2 + a^2) =: L_xy and l_z k_z = z k_z / r, so
+//   d_c L = d_c r V + (r k_x - a k_y, r k_y + a k_x, k_z)_c / (r^2 + a^2 or r),
+//   V = (A - 2 r L_xy) / (r^2 + a^2) - k_z z / r^2,
+// and d_c f = F1 d_c r - [c = z] 2 a^2 z f / (r^4 + a^2 z^2), F1 = f (3 / r - 4 r^3 / (r^4 + a^2 z^2)).
+// The same quantities as the nine-derivative form, in about 40 fewer operations.
+// Exact scalings are folded away: d_c f is carried halved (F1), so that 1/2 L need not be formed.
+// The order of operations and the roundings are part of the method: rays that graze the photon
+// orbit amplify them, and every kernel integrates with the same ones (bl_geodf.cuh in
+// double-float).
 __device__ __forceinline__ double geodesic_rhs64(const double y[8], const Rhs64& C, double dy[8]) {
     const double x = y[1], yy = y[2], z = y[3];
     const double kt = y[4], kx = y[5], ky = y[6], kz = y[7];
@@ -96,7 +114,7 @@ __device__ __forceinline__ double geodesic_rhs64(const double y[8], const Rhs64&
     const double r = __dmul_rn(r2, ir);
     const double s4 = __fma_rn(r2, r2, aaz2);
     const double P = __dadd_rn(r2, aa);
-    const double iPs = g_rcp(__dmul_rn(P, s4));
+    const double iPs = 1.0 / __dmul_rn(P, s4);
     const double is4 = __dmul_rn(P, iPs);
     const double iP = __dmul_rn(s4, iPs);
     const double f = C.flat ? 0.0 : __dmul_rn(mul3(C.m2, r, r2), is4);
@@ -172,6 +190,18 @@ __device__ __forceinline__ int step_parts_est(const float ym[8], float a, float 
     return hi < 1.0f ? 1 : (int)hi;
 }
 
+// Stage derivatives, 7 stages x 7 components: in dynamic shared memory, thread-fastest and
+// conflict-free, or a per-thread local array (the 64-warp shape leaves no shared memory for them).
+template <bool kSmem> struct KStore64;
+template <> struct KStore64<true> {
+    double* p;
+    __device__ __forceinline__ double& at(int j, int s) { return p[(j * 7 + s) * 128]; }
+};
+template <> struct KStore64<false> {
+    double k[7][7];
+    __device__ __forceinline__ double& at(int j, int s) { return k[j][s]; }
+};
+
 template <class R, bool kKsmem>
 __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ imgs, int n_images,
                                                 int64_t ray_begin, int64_t ray_end,
@@ -192,7 +222,7 @@ __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ im
     double y[8];
     // K(0, c) = f(y); K(1..6, c) stage derivatives of the current attempt. dk_t/dl = 0, so the
     // k_t slot is left out: 7 slots a stage.
-    KStore<double, kKsmem> Ks;
+    KStore64<kKsmem> Ks;
     if constexpr (kKsmem) {
         extern __shared__ __align__(16) unsigned char geo_smem[];
         Ks.p = reinterpret_cast<double*>(geo_smem) + threadIdx.x;
@@ -426,9 +456,9 @@ __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ im
                         float yf[8];
 #pragma unroll
                         for (int c = 0; c < 8; ++c) yf[c] = to_float_rn(y[c]);
-                        ok = append_record<float, float>(sink, wray, nrec, ymf, yf, hl);
+                        ok = append_record<float, float, double>(sink, wray, nrec, ymf, yf, hl);
                     } else {
-                        ok = append_record<double, double>(sink, wray, nrec, ym, y, hl);
+                        ok = append_record<double, double, double>(sink, wray, nrec, ym, y, hl);
                     }
                 } else if constexpr (kFRec) {
                     // the quartic through y0, y1, h f0, h f1 and y_mid (Shampine 1986), in FP32
@@ -449,7 +479,7 @@ __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ im
                         c3f[c] = __fmaf_rn(-32.0f, D3, __fmaf_rn(14.0f, D1, -__fmul_rn(3.0f, D2)));
                         c4f[c] = __fmaf_rn(16.0f, D3, __fmaf_rn(-8.0f, D1, __fmul_rn(2.0f, D2)));
                     }
-                    ok = emit_quartic_f(sink, wray, nrec, y0f, d0f, c2f, c3f, c4f, nsub, hl);
+                    ok = emit_quartic_f(sink, wray, nrec, y0f, d0f, c2f, c3f, c4f, nsub, hl / nsub);
                 } else {
                     double d0[8], c2[8], c3[8], c4[8];
 #pragma unroll
@@ -482,7 +512,7 @@ __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ im
                             ynd[c] = (s == 0) ? y[c]
                                               : y[c] + tn * (d0[c] + tn * (c2[c] + tn * (c3[c] + tn * c4[c])));
                         }
-                        ok = append_record<double, double>(sink, wray, nrec, ysm, ynd, dls);
+                        ok = append_record<double, double, double>(sink, wray, nrec, ysm, ynd, dls);
                     }
                 }
                 if (!ok) { status = BL_RAY_OVERFLOW; done = true; }
@@ -574,9 +604,9 @@ __device__ __forceinline__ bool append_state(const RecordSink<R>& sink, int64_t 
         float a[8], b[8];
 #pragma unroll
         for (int c = 0; c < 8; ++c) { a[c] = to_float_rn(ys[c]); b[c] = to_float_rn(yn[c]); }
-        return append_record<float, float>(sink, wray, nrec, a, b, dl);
+        return append_record<float, float, double>(sink, wray, nrec, a, b, dl);
     } else {
-        return append_record<double, double>(sink, wray, nrec, ys, yn, dl);
+        return append_record<double, double, double>(sink, wray, nrec, ys, yn, dl);
     }
 }
 

@@ -587,30 +587,7 @@ struct RecordSink {
     Counters* ctr;
 };
 
-// Arithmetic used by the geodesic integrator: native double, or df64 (double-float).
-template <class G> struct GeoArith;
-template <> struct GeoArith<double> {
-    static __device__ __forceinline__ double from(double d) { return d; }
-    static __device__ __forceinline__ double to(double g) { return g; }
-    static __device__ __forceinline__ float tof(double g) { return (float)g; }
-};
-template <> struct GeoArith<float> {
-    static __device__ __forceinline__ float from(double d) { return (float)d; }
-    static __device__ __forceinline__ double to(float g) { return (double)g; }
-    static __device__ __forceinline__ float tof(float g) { return g; }
-};
-template <> struct GeoArith<df64> {
-    static __device__ __forceinline__ df64 from(double d) { return df64(d); }
-    static __device__ __forceinline__ double to(const df64& g) { return df_to_double(g); }
-    static __device__ __forceinline__ float tof(const df64& g) { return g.hi + g.lo; }
-};
-
-// Short sums of products in the integrator arithmetic: plain expressions in double, the
-// compensated accumulator (one renormalisation per sum) in double-float.
-__device__ __forceinline__ double g_fma(double a, double b, double c) { return a * b + c; }
-__device__ __forceinline__ double g_dot2(double a, double b, double c, double d) { return a * b + c * d; }
-__device__ __forceinline__ double g_dot3(double a, double b, double c, double d, double e,
-                                         double f) { return a * b + c * d + e * f; }
+// Short sums of products in double-float: the compensated accumulator, one renormalisation a sum.
 __device__ __forceinline__ df64 g_fma(const df64& a, const df64& b, const df64& c) {
     DFDot s;
     s.first(a, b);
@@ -632,78 +609,11 @@ __device__ __forceinline__ df64 g_dot3(const df64& a, const df64& b, const df64&
     return s.get();
 }
 
-// 1/x in the integrator arithmetic (no multiplication by an exact 1 in double-float).
-__device__ __forceinline__ double g_rcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ df64 g_rcp(const df64& x) { return rcp(x); }
-
-// A product inside a chain of products: unnormalised in double-float, plain in double.
-__device__ __forceinline__ double g_mul_nn(double a, double b) { return a * b; }
+// A product inside a chain of products: unnormalised.
 __device__ __forceinline__ df64 g_mul_nn(const df64& a, const df64& b) { return df_mul_nn(a, b); }
 
-// Exact scaling by a power of two in the integrator arithmetic.
-__device__ __forceinline__ double scale2(double x, float f) { return x * (double)f; }
+// Exact scaling by a power of two.
 __device__ __forceinline__ df64 scale2(const df64& x, float f) { return df_scale(x, f); }
-
-// Eq. (geodesic) right-hand side in arithmetic G; returns r at the evaluation point.
-// With g^ab = eta^ab - f l^a l^b and L = l^a k_a, dx^a/dl = g^ab k_b and
-// dk_c/dl = L (1/2 d_c f L + f d_c L), where d_c L is the derivative at fixed k. Instead of the
-// nine derivatives d_c l_b (bl_math.cuh's form, kept for the transport matrices), d_c L is
-// formed directly: with A = x k_x + y k_y and B = y k_x - x k_y, l_x k_x + l_y k_y =
-// (r A + a B) / (r^2 + a^2) =: L_xy and l_z k_z = z k_z / r, so
-//   d_c L = d_c r V + (r k_x - a k_y, r k_y + a k_x, k_z)_c / (r^2 + a^2 or r),
-//   V = (A - 2 r L_xy) / (r^2 + a^2) - k_z z / r^2,
-// and d_c f = F1 d_c r - [c = z] 2 a^2 z f / (r^4 + a^2 z^2), F1 = f (3 / r - 4 r^3 / (r^4 + a^2 z^2)).
-// The same quantities as the nine-derivative form, in about 40 fewer operations.
-template <class G>
-__device__ __forceinline__ G geodesic_rhs_g(const G y[8], const G& a, const G& m, bool flat, G dy[8]) {
-    constexpr G c0 = G(0), c3 = G(3);
-    const G x = y[1], yy = y[2], z = y[3];
-    const G kt = y[4], kx = y[5], ky = y[6], kz = y[7];
-    // r (Eq. cks_aux:r), f and l as in ks_geom: two reciprocal square roots, one reciprocal
-    const G aa = a * a;
-    const G q = g_dot3(x, x, yy, yy, z, z) - aa;
-    const G aaz2 = g_mul_nn(aa, z) * z;
-    const G D2 = g_fma(q, q, scale2(aaz2, 4.0f));
-    const G iD = rsqrt(D2);
-    const G r2 = scale2(g_fma(D2, iD, q), 0.5f);
-    const G ir = rsqrt(r2);
-    const G r = r2 * ir;
-    const G s4 = g_fma(r2, r2, aaz2);
-    const G P = r2 + aa;
-    const G iPs = g_rcp(P * s4);
-    const G is4 = P * iPs;
-    const G iP = s4 * iPs;
-    const G f = flat ? c0 : g_mul_nn(g_mul_nn(scale2(m, 2.0f), r), r2) * is4;
-    const G lx = g_dot2(r, x, a, yy) * iP, ly = g_dot2(r, yy, -a, x) * iP, lz = z * ir;
-    // L = l^a k_a (l^t = -1)
-    const G A_ = g_dot2(x, kx, yy, ky);
-    const G B_ = g_dot2(yy, kx, -x, ky);
-    const G Lxy = g_dot2(r, A_, a, B_) * iP;
-    const G L = g_fma(lz, kz, Lxy - kt);
-    const G fL = f * L;
-    dy[0] = fL - kt;
-    dy[1] = g_fma(-lx, fL, kx);
-    dy[2] = g_fma(-ly, fL, ky);
-    dy[3] = g_fma(-lz, fL, kz);
-    dy[4] = c0;
-    // d_c r
-    const G riD = r * iD;
-    const G drx = riD * x, dry = riD * yy, drz = g_mul_nn(g_mul_nn(z, P), ir) * iD;
-    // d_c L at fixed k, and d_c f
-    const G w = kz * ir;
-    const G V = g_dot2(g_fma(-scale2(r, 2.0f), Lxy, A_), iP, -w, lz);
-    const G Sx = g_dot2(drx, V, g_dot2(r, kx, -a, ky), iP);
-    const G Sy = g_dot2(dry, V, g_dot2(r, ky, a, kx), iP);
-    const G Sz = g_fma(drz, V, w);
-    const G F1 = f * g_dot2(c3, ir, -(scale2(r2, 4.0f) * r), is4);
-    const G dfx = F1 * drx, dfy = F1 * dry;
-    const G dfz = g_fma(F1, drz, -(g_mul_nn(g_mul_nn(scale2(aa, 2.0f), z), f) * is4));
-    const G halfL = scale2(L, 0.5f);
-    dy[5] = L * g_dot2(dfx, halfL, f, Sx);
-    dy[6] = L * g_dot2(dfy, halfL, f, Sy);
-    dy[7] = L * g_dot2(dfz, halfL, f, Sz);
-    return r;
-}
 
 template <> struct DPCoef<df64> {
     static __device__ __forceinline__ df64 a(int s, int j) { const float2 v = c_dpf.a[s][j]; return df64(v.x, v.y); }
@@ -711,36 +621,10 @@ template <> struct DPCoef<df64> {
     static __device__ __forceinline__ df64 m(int j) { const float2 v = c_dpf.m[j]; return df64(v.x, v.y); }
 };
 
-// Accumulator of a sum of coefficient x stage-derivative products in the integrator
-// arithmetic: the compensated double-float dot product, or plain (fused) double.
-template <class G> struct StageDot;
-template <> struct StageDot<double> {
-    double s;
-    __device__ __forceinline__ void first(double a, double x) { s = a * x; }
-    __device__ __forceinline__ void add(double a, double x) { s = s + a * x; }
-    __device__ __forceinline__ double get() const { return s; }
-    __device__ __forceinline__ double axpy(double h, double y) const { return y + h * s; }
-};
-template <> struct StageDot<df64> {
-    DFDot d;
-    __device__ __forceinline__ void first(const df64& a, const df64& x) { d.first(a, x); }
-    __device__ __forceinline__ void add(const df64& a, const df64& x) { d.add(a, x); }
-    __device__ __forceinline__ df64 get() const { return d.get(); }
-    __device__ __forceinline__ df64 axpy(const df64& h, const df64& y) const { return d.axpy(h, y); }
-    __device__ __forceinline__ float value_f() const { return d.s + d.c; }
-};
-
-
-template <class R, class G>
-__device__ __forceinline__ R to_rec(const G& v) {
-    if constexpr (sizeof(R) == sizeof(float)) return (R)GeoArith<G>::tof(v);
-    else return (R)GeoArith<G>::to(v);
-}
-
 // Append one record for `ray`; returns false when the store is full.
-template <class R, class G>
+template <class R, class G, class D>
 __device__ __forceinline__ bool append_record(const RecordSink<R>& S, int64_t ray, int32_t& nrec,
-                                              const G ys[8], const G yn[8], double dl) {
+                                              const G ys[8], const G yn[8], D dl) {
     const int32_t slot = nrec % kChunk;
     const int32_t ch = nrec / kChunk;
     if (ch >= kMaxChunks) return false;
@@ -754,10 +638,10 @@ __device__ __forceinline__ bool append_record(const RecordSink<R>& S, int64_t ra
     R* rec = S.pool + idx * RecStride<R>::v;
     // the record is assembled in registers and stored as 16-byte vectors (records are 64 B
     // (float) or 112 B (double) apart from a 256-byte aligned pool)
-    const R v[14] = {to_rec<R>(ys[1]), to_rec<R>(ys[2]), to_rec<R>(ys[3]), to_rec<R>(ys[5]),
-                     to_rec<R>(ys[6]), to_rec<R>(ys[7]), to_rec<R>(yn[1]), to_rec<R>(yn[2]),
-                     to_rec<R>(yn[3]), to_rec<R>(yn[5]), to_rec<R>(yn[6]), to_rec<R>(yn[7]),
-                     (R)dl, to_rec<R>(ys[0])};   // value 13: coordinate time (slow light)
+    const R v[14] = {(R)ys[1], (R)ys[2], (R)ys[3], (R)ys[5],
+                     (R)ys[6], (R)ys[7], (R)yn[1], (R)yn[2],
+                     (R)yn[3], (R)yn[5], (R)yn[6], (R)yn[7],
+                     (R)dl, (R)ys[0]};   // value 13: coordinate time (slow light)
     if constexpr (std::is_same<R, float>::value) {
         float4* q = reinterpret_cast<float4*>(rec);
         q[0] = make_float4(v[0], v[1], v[2], v[3]);
@@ -778,25 +662,13 @@ __device__ __forceinline__ bool append_record(const RecordSink<R>& S, int64_t ra
 #ifndef BL_GEO_MIN_CTAS
 #define BL_GEO_MIN_CTAS 3
 #endif
-// Stage derivatives of a geodesic kernel: in dynamic shared memory, thread-fastest (the
-// double-float and mixed forms), or a per-thread local array (the FP64 form, whose high
-// occupancy leaves no shared memory for them).
-template <class G, bool kSmem> struct KStore;
-template <class G> struct KStore<G, true> {
-    G* p;
-    __device__ __forceinline__ G& at(int j, int s) { return p[(j * 7 + s) * 128]; }
-};
-template <class G> struct KStore<G, false> {
-    G k[7][7];
-    __device__ __forceinline__ G& at(int j, int s) { return k[j][s]; }
-};
 // Records of a subdivided step from the FP32 quartic about the step's start (coefficients
 // y0, d0 = h f0, c2, c3, c4 per component): nsub samples at the centres of equal parts.
-template <class R>
+template <class R, class D>
 __device__ __forceinline__ bool emit_quartic_f(const RecordSink<R>& sink, int64_t wray, int32_t& nrec,
                                        const float y0f[8], const float d0f[8], const float c2f[8],
                                        const float c3f[8], const float c4f[8], int nsub,
-                                       double hd) {
+                                       D dl) {
     bool ok = true;
     const float invf = 1.0f / (float)nsub;
     for (int s = 0; s < nsub && ok; ++s) {
@@ -808,7 +680,7 @@ __device__ __forceinline__ bool emit_quartic_f(const RecordSink<R>& sink, int64_
             ynd[c] = (s == 0) ? y0f[c]
                               : y0f[c] + tn * (d0f[c] + tn * (c2f[c] + tn * (c3f[c] + tn * c4f[c])));
         }
-        ok = append_record(sink, wray, nrec, ysm, ynd, hd / nsub);
+        ok = append_record(sink, wray, nrec, ysm, ynd, dl);
     }
     return ok;
 }
@@ -850,484 +722,14 @@ __device__ __forceinline__ bool sparse_wave(const BlockSource& bs, int64_t ray_b
 
 }  // namespace bl
 #include "bl_geo64.cuh"
+#include "bl_geodf.cuh"
 namespace bl {
 
-template <class R, class G, bool kKsmem>
-__device__ __forceinline__ void geodesic_body(const ImageDesc* __restrict__ imgs,
-                                              int n_images, int64_t ray_begin, int64_t ray_end,
-                                              RayHdr* __restrict__ hdr, RecordSink<R> sink,
-                                              int record, BlockSource bs,
-                                              const RayInit* __restrict__ init) {
-    // rays [ray_begin, ray_end) of the batch form this wave; hdr, init and the chunk tables
-    // are indexed by ray - ray_begin
-    const int64_t re = wave_end(bs, ray_end);
-    const int64_t total_rays = re > ray_begin ? re - ray_begin : 0;
-    using A = GeoArith<G>;
-    // compile-time constants in the integrator arithmetic (a run-time double -> df64 split
-    // would cost FP64 conversions)
-    constexpr G kDP_A21 = G(DP_A21);
-    constexpr G kDP_A31 = G(DP_A31);
-    constexpr G kDP_A32 = G(DP_A32);
-    constexpr G kDP_A41 = G(DP_A41);
-    constexpr G kDP_A42 = G(DP_A42);
-    constexpr G kDP_A43 = G(DP_A43);
-    constexpr G kDP_A51 = G(DP_A51);
-    constexpr G kDP_A52 = G(DP_A52);
-    constexpr G kDP_A53 = G(DP_A53);
-    constexpr G kDP_A54 = G(DP_A54);
-    constexpr G kDP_A61 = G(DP_A61);
-    constexpr G kDP_A62 = G(DP_A62);
-    constexpr G kDP_A63 = G(DP_A63);
-    constexpr G kDP_A64 = G(DP_A64);
-    constexpr G kDP_A65 = G(DP_A65);
-    constexpr G kDP_B1 = G(DP_B1);
-    constexpr G kDP_B3 = G(DP_B3);
-    constexpr G kDP_B4 = G(DP_B4);
-    constexpr G kDP_B5 = G(DP_B5);
-    constexpr G kDP_B6 = G(DP_B6);
-    constexpr G kDP_E1 = G(DP_E1);
-    constexpr G kDP_E3 = G(DP_E3);
-    constexpr G kDP_E4 = G(DP_E4);
-    constexpr G kDP_E5 = G(DP_E5);
-    constexpr G kDP_E6 = G(DP_E6);
-    constexpr G kDP_E7 = G(DP_E7);
-    constexpr G kDP_M1 = G(DP_M1);
-    constexpr G kDP_M3 = G(DP_M3);
-    constexpr G kDP_M4 = G(DP_M4);
-    constexpr G kDP_M5 = G(DP_M5);
-    constexpr G kDP_M6 = G(DP_M6);
-    constexpr G kDP_M7 = G(DP_M7);
-    constexpr G kHalf = G(0.5);
-    constexpr G kM5 = G(-5.0);
-    constexpr G k16 = G(16.0);
-    constexpr G k14 = G(14.0);
-    constexpr G kThree = G(3.0);
-    constexpr G k32 = G(32.0);
-    constexpr G kM8 = G(-8.0);
-    constexpr G k2c = G(2.0);
-    constexpr bool kNative = std::is_same<G, double>::value;
-    Counters* ctr = sink.ctr;
-    bool active = false;
-    int64_t ray = 0;
-    int q = 0, pi = 0, pj = 0;
-    int64_t opix = 0;   // output index of the current ray
-    int64_t wray = 0;   // index of the current ray within this wave
-    G y[8];
-    // K(0, c) = f(y); K(1..6, c) stage derivatives of the current attempt. In shared memory
-    // (thread-fastest, conflict-free): 448 B a thread, which as a local array would take 172 KB
-    // of L1 per SM and miss to L2.
-    // The k_t component is constant along the ray (dk_t/dl = 0), so its derivatives are not
-    // stored: 7 slots a stage, and KR(j, 4) reads as an exact zero.
-#define KSLOT(c) ((c) < 4 ? (c) : (c) - 1)
-    KStore<G, kKsmem> Ks;
-    if constexpr (kKsmem) {
-        extern __shared__ __align__(16) unsigned char geo_smem[];
-        Ks.p = reinterpret_cast<G*>(geo_smem) + threadIdx.x;
-    }
-#define KX(j, c) Ks.at(j, KSLOT(c))
-#define KR(j, c) ((c) == 4 ? G(0) : KX(j, c))
-    G h = G(0);
-    double nnorm = 0.0;
-    bool been_inside = false, prev_rej = false;
-    int64_t attempts = 0;
-    int32_t nrec = 0, status = 0;
-    double r_cam = 0.0, r_in = 0.0, ds_max = 0.0, r_grid = 0.0;
-    G a = G(0), m = G(0);
-    double tol_abs = 0.0, tol_rel = 0.0;
-    int64_t max_steps = 0;
-    bool flat = false;
-    double r_cur = 0.0;     // r at y
-    bool want_aux = false;  // auxiliary images: proper length and affine parameter
-    double aux_len = 0.0, aux_lam = 0.0;
-    int32_t last_in = -1;   // last record of a step reaching within 1.001 r_max
-
-    bool exhausted = false;
-    // All 32 lanes stay in the loop until the whole warp is out of work, so the warp
-    // reconverges every iteration and the attempt is issued once for all lanes that hold a
-    // ray (lanes without one are masked).
-    while (true) {
-        const bool need = !active && !exhausted;
-        const unsigned long long got = warp_refill(&ctr->next_ray_geo, need);
-        if (need) {
-            if ((int64_t)got >= total_rays) {
-                exhausted = true;
-            } else {
-                wray = (int64_t)got;
-                ray = ray_begin + wray;
-                active = true;
-            }
-        }
-        if (!__any_sync(0xffffffffu, active)) break;
-        if (!active) continue;
-        if (need) {   // a ray taken from the queue in this iteration: set it up
-            setup_ray(imgs, n_images, bs, ray, q, opix, pi, pj);
-            const ImageDesc& im = imgs[q];
-            // the pixel's initial state: in the double-float form from ray_init_kernel (its
-            // FP64 set-up stays out of this loop), in the FP64-arithmetic forms computed here
-            // (measured faster for them: mixed form 190 against 235 ms with the precomputed
-            // states)
-            if constexpr (kNative) {
-                double yd[8];
-                pixel_state(im, pi, pj, yd, nnorm);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) y[c] = yd[c];
-            } else {
-                const RayInit& ri = init[wray];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) y[c] = A::from(ri.y[c]);
-                nnorm = ri.nnorm;
-            }
-            a = A::from(im.spin); m = A::from(im.mass); flat = im.flat != 0;
-            r_cam = im.r_cam;
-            r_in = im.r_in_over_rhor * im.r_hor;
-            ds_max = im.ds_max;
-            r_grid = im.r_max;
-            tol_abs = im.tol_abs; tol_rel = im.tol_rel;
-            max_steps = im.max_steps;
-            want_aux = record && im.aux != nullptr;
-            aux_len = aux_lam = 0.0;
-            h = A::from(-im.h0_frac * (r_cam - im.r_hor));
-            prev_rej = false;
-        }
-        // ---- one Dormand-Prince attempt (Table tab:dp) ----
-        // Rolled stage loop: one right-hand-side body run six times keeps the kernel small
-        // enough for the instruction cache. K(0) holds f(y) (first same as last), K(s) the
-        // stage derivatives; stage 6 is evaluated at the fifth-order solution y5. A ray's first
-        // attempt starts at stage 0, which evaluates f(y) at the stage point y, so that the
-        // set-up path needs no copy of the right-hand side.
-        G ys[8], y5[8];
-        double r5 = 0.0;
-#pragma unroll 1
-        for (int st = need ? 0 : 1; st < 7; ++st) {
-            if (st == 0) {
-#pragma unroll
-                for (int c = 0; c < 8; ++c) ys[c] = y[c];
-            } else {
-                // earlier stages outer (rolled), components inner: each coefficient is read
-                // once per stage term; every component keeps its order of operations
-                StageDot<G> acc[8];
-                {
-                    const G a0 = DPCoef<G>::a(st, 0);
-#pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        if (c != 4) acc[c].first(a0, KX(0, c));
-                }
-                // the last row's second coefficient (b_2 of the fifth-order weights) is zero
-#pragma unroll 1
-                for (int j = st == 6 ? 2 : 1; j < st; ++j) {
-                    const G aj = DPCoef<G>::a(st, j);
-#pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        if (c != 4) acc[c].add(aj, KX(j, c));
-                }
-#pragma unroll
-                for (int c = 0; c < 8; ++c) ys[c] = (c == 4) ? y[4] : acc[c].axpy(h, y[c]);
-            }
-            G fs[8];
-            const G rr = geodesic_rhs_g<G>(ys, a, m, flat, fs);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) if (c != 4) KX(st, c) = fs[c];
-            if (st == 0) {
-                r_cur = A::to(rr);
-                been_inside = r_cur < r_cam;
-            }
-            if (st == 6) {
-                r5 = kNative ? A::to(rr) : (double)A::tof(rr);
-#pragma unroll
-                for (int c = 0; c < 8; ++c) y5[c] = ys[c];
-            }
-        }
-        // Error norm eps = max_c |y5_c - y4_c| / (f_abs + f_rel max(|y_c|, |y5_c|)) with
-        // y5 - y4 = h sum (b5 - b4) k. Native double keeps the FP64 form's arithmetic; the
-        // df64 form takes the ratio in float (it only steers the step size).
-        double eps;
-        bool finite = true;
-        {
-            G errv[8];
-            float errf[8];
-            {
-                StageDot<G> acc[8];
-                {
-                    const G e0 = DPCoef<G>::e(0);
-#pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        if (c != 4) acc[c].first(e0, KX(0, c));
-                }
-#pragma unroll 1
-                for (int j = 2; j < 7; ++j) {
-                    const G ej = DPCoef<G>::e(j);
-#pragma unroll
-                    for (int c = 0; c < 8; ++c)
-                        if (c != 4) acc[c].add(ej, KX(j, c));
-                }
-                if constexpr (kNative) {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) errv[c] = (c == 4) ? G(0) : h * acc[c].get();
-                } else {
-                    // the double-float form uses the estimate in FP32 only: h_hi (s + c) there
-                    const float hf = A::tof(h);
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) errf[c] = (c == 4) ? 0.0f : hf * acc[c].value_f();
-                }
-            }
-            if constexpr (kNative) {
-                double num = 0.0, den = 1.0;
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const double err = fabs(A::to(errv[c]));
-                    const double sc = tol_abs + tol_rel * fmax(fabs(A::to(y[c])), fabs(A::to(y5[c])));
-                    finite = finite && isfinite(err) && isfinite(A::to(y5[c]));
-                    if (err * den > num * sc) { num = err; den = sc; }
-                }
-                eps = num / den;
-            } else {
-                float num = 0.0f, den = 1.0f;
-                const float ta = (float)tol_abs, tr = (float)tol_rel;
-#pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const float err = fabsf(errf[c]);
-                    const float sc = ta + tr * fmaxf(fabsf(A::tof(y[c])), fabsf(A::tof(y5[c])));
-                    finite = finite && isfinite(err) && isfinite(A::tof(y5[c]));
-                    if (err * den > num * sc) { num = err; den = sc; }
-                }
-                eps = (double)(num / den);
-            }
-        }
-        ++attempts;
-        bool done = false;
-        if (!finite) {
-            status = BL_RAY_NAN;
-            done = true;
-        } else if (eps <= 1.0) {
-            // accepted: samples of this step (camera side first)
-            if (record) {
-                // FP32 records (fast and mixed forms): the midpoint's increment
-                // (h/2) sum_j b_mid,j k_j and the quartic coefficients are formed in FP32 from the
-                // state; they move a record by about one FP32 ulp and leave the integration and
-                // its step decisions untouched. FP64 records (FP64 form): all in double.
-                constexpr bool kFRec = sizeof(R) == sizeof(float);
-                G ym[8];
-                float ymf[8], incm[8];
-                if constexpr (kFRec) {
-                    const float hh = 0.5f * A::tof(h);
-                    float acc[8];
-                    {
-                        const float m0 = c_dpf.m[0].x;
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) acc[c] = m0 * A::tof(KR(0, c));
-                    }
-#pragma unroll 1
-                    for (int j = 2; j < 7; ++j) {
-                        const float mj = c_dpf.m[j].x;
-#pragma unroll
-                        for (int c = 0; c < 8; ++c)
-                            if (c != 4) acc[c] = fmaf(mj, A::tof(KX(j, c)), acc[c]);
-                    }
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        incm[c] = hh * acc[c];
-                        if constexpr (!kNative) ymf[c] = y[c].hi + (y[c].lo + incm[c]);
-                    }
-                } else {
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        G acc = DPCoef<G>::m(0) * KR(0, c);
-#pragma unroll 1
-                        for (int j = 2; j < 7; ++j) acc = acc + DPCoef<G>::m(j) * KR(j, c);
-                        ym[c] = y[c] + (kHalf * h) * acc;
-                    }
-                }
-                const double r0 = r_cur, r1 = r5;
-                const double hd = kNative ? A::to(h) : (double)A::tof(h);
-                double rmid, kt_up, fmid;
-                if constexpr (kNative) {
-                    double ymd[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        if constexpr (kFRec) {
-                            ymd[c] = A::to(y[c]) + (double)incm[c];
-                            ymf[c] = (float)ymd[c];
-                        } else {
-                            ymd[c] = A::to(ym[c]);
-                        }
-                    }
-                    KSGeom<double> Gm;
-                    ks_geom<double>(ymd[1], ymd[2], ymd[3], im_spin(imgs, q), im_mass(imgs, q), flat, false, Gm);
-                    const double L = -ymd[4] + Gm.l[1] * ymd[5] + Gm.l[2] * ymd[6] + Gm.l[3] * ymd[7];
-                    kt_up = -ymd[4] + Gm.f * L;
-                    rmid = Gm.r;
-                    fmid = Gm.f;
-                } else {
-                    KSGeom<float> Gm;
-                    ks_geom<float>(ymf[1], ymf[2], ymf[3], (float)im_spin(imgs, q), (float)im_mass(imgs, q),
-                                   flat, false, Gm);
-                    const float L = -ymf[4] + Gm.l[1] * ymf[5] + Gm.l[2] * ymf[6] + Gm.l[3] * ymf[7];
-                    kt_up = -ymf[4] + Gm.f * L;
-                    rmid = Gm.r;
-                    fmid = Gm.f;
-                }
-                if (want_aux) {
-                    aux_lam += fabs(hd);
-                    aux_len += fabs(hd) * fabs(kt_up) / sqrt(1.0 + fmid);
-                }
-                const double rmin = fmin(rmid, fmin(r0, r1));
-                int nsub = 1;
-                if (rmin < r_grid) {
-                    // ds/dl = (g_pq k^p k^q)^1/2 = alpha |k^t| for a null ray
-                    if constexpr (kNative) {
-                        const double ds = fabs(hd) * fabs(kt_up) / sqrt(1.0 + fmid);
-                        if (ds > ds_max) {
-                            const double nd = ceil(ds / ds_max);
-                            nsub = nd > 4096.0 ? 4097 : (int)nd;
-                        }
-                    } else {
-                        const float ds = fabsf((float)hd) * fabsf((float)kt_up) * rsqrtf(1.0f + (float)fmid);
-                        if (ds > (float)ds_max) {
-                            const float nd = ceilf(ds / (float)ds_max);
-                            nsub = nd > 4096.0f ? 4097 : (int)nd;
-                        }
-                    }
-                }
-                bool ok = true;
-                if (nsub == 1) {
-                    if constexpr (kFRec) {
-                        float yf[8];
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) yf[c] = A::tof(y[c]);
-                        ok = append_record(sink, wray, nrec, ymf, yf, fabs(hd));
-                    } else {
-                        ok = append_record(sink, wray, nrec, ym, y, fabs(hd));
-                    }
-                } else if constexpr (kFRec) {
-                    // float records: the quartic through y0, y1, h f0, h f1 and y_mid
-                    // (Shampine 1986), in FP32 about y0 (y_mid - y0 is the midpoint increment)
-                    const float hf = A::tof(h);
-                    float y0f[8], d0f[8], c2f[8], c3f[8], c4f[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const float d0 = hf * A::tof(KR(0, c));
-                        const float D1 = A::tof(y5[c] - y[c]) - d0;
-                        const float D2 = hf * A::tof(KR(6, c)) - d0;
-                        const float D3 = incm[c] - 0.5f * d0;
-                        y0f[c] = A::tof(y[c]);
-                        d0f[c] = d0;
-                        c2f[c] = -5.0f * D1 + D2 + 16.0f * D3;
-                        c3f[c] = 14.0f * D1 - 3.0f * D2 - 32.0f * D3;
-                        c4f[c] = -8.0f * D1 + 2.0f * D2 + 16.0f * D3;
-                    }
-                    ok = emit_quartic_f(sink, wray, nrec, y0f, d0f, c2f, c3f, c4f, nsub, fabs(hd));
-                } else {
-                    double y0d[8], d0[8], c2[8], c3[8], c4[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        y0d[c] = A::to(y[c]);
-                        d0[c] = hd * A::to(KR(0, c));
-                        const double D1 = A::to(y5[c]) - y0d[c] - d0[c];
-                        const double D2 = hd * A::to(KR(6, c)) - d0[c];
-                        const double D3 = A::to(ym[c]) - y0d[c] - 0.5 * d0[c];
-                        c2[c] = -5.0 * D1 + D2 + 16.0 * D3;
-                        c3[c] = 14.0 * D1 - 3.0 * D2 - 32.0 * D3;
-                        c4[c] = -8.0 * D1 + 2.0 * D2 + 16.0 * D3;
-                    }
-                    const double inv = 1.0 / nsub;
-                    for (int s = 0; s < nsub && ok; ++s) {
-                        double ysm[8], ynd[8];
-                        const double ts = (s + 0.5) * inv, tn = s * inv;
-#pragma unroll
-                        for (int c = 0; c < 8; ++c) {
-                            ysm[c] = y0d[c] + ts * (d0[c] + ts * (c2[c] + ts * (c3[c] + ts * c4[c])));
-                            ynd[c] = (s == 0) ? y0d[c]
-                                              : y0d[c] + tn * (d0[c] + tn * (c2[c] + tn * (c3[c] + tn * c4[c])));
-                        }
-                        ok = append_record(sink, wray, nrec, ysm, ynd, fabs(hd) * inv);
-                    }
-                }
-                if (!ok) { status = BL_RAY_OVERFLOW; done = true; }
-                else if (kNative && rmin <= r_grid * 1.001) last_in = nrec - 1;
-            }
-#pragma unroll
-            for (int c = 0; c < 8; ++c) { y[c] = y5[c]; if (c != 4) KX(0, c) = KX(6, c); }
-            if constexpr (kNative) {
-                double fac = (eps == 0.0) ? 10.0 : 0.9 * inv_fifth_root(eps);
-                fac = fmin(10.0, fmax(0.2, fac));
-                if (prev_rej) fac = fmin(fac, 1.0);
-                h = h * A::from(fac);
-            } else {
-                const float ef = (float)eps;
-                float fac = (ef == 0.0f) ? 10.0f : 0.9f * powf(ef, -0.2f);
-                fac = fminf(10.0f, fmaxf(0.2f, fac));
-                if (prev_rej) fac = fminf(fac, 1.0f);
-                h = h * G(fac);
-            }
-            prev_rej = false;
-            r_cur = r5;
-            if (!done) {
-                if (r_cur < r_in) { status = BL_RAY_HORIZON; done = true; }
-                else if (been_inside && r_cur > r_cam) { status = BL_RAY_ESCAPED; done = true; }
-                else if (r_cur < r_cam) been_inside = true;
-            }
-        } else {
-            double fac;
-            if constexpr (kNative) {
-                fac = fmax(0.2, 0.9 * inv_fifth_root(eps));
-                h = h * A::from(fac);
-            } else {
-                h = h * G(fmaxf(0.2f, 0.9f * powf((float)eps, -0.2f)));
-            }
-            prev_rej = true;
-        }
-        if (!done) {
-            if ((kNative ? fabs(A::to(h)) : (double)fabsf(A::tof(h))) < 1e-12 * r_cur) {
-                status = BL_RAY_UNDERFLOW;
-                done = true;
-            }
-            else if (attempts >= max_steps) { status = BL_RAY_MAX_STEPS; done = true; }
-        }
-        if (done) {
-            const ImageDesc& im = imgs[q];
-            const int64_t pix = opix;
-            if (im.status) im.status[pix] = status;
-            if (im.steps) im.steps[pix] = (int32_t)(attempts < 2147483647 ? attempts : 2147483647);
-            if (im.end_state)
-                for (int c = 0; c < 8; ++c) im.end_state[pix * 8 + c] = A::to(y[c]);
-            if (im.samples) im.samples[pix] = nrec;
-            if (want_aux) {
-                aux_store(im, 0, pix, -A::to(y[0]));
-                aux_store(im, 1, pix, aux_len);
-                aux_store(im, 2, pix, aux_lam);
-            }
-            RayHdr hd;
-            hd.kt = A::to(y[4]);
-            hd.nnorm = nnorm;
-            hd.nrec = nrec;
-            hd.status = status;
-            // (the double-float kernel, issue bound at its register limit, does not track it:
-            // 27.3 -> 29.9 ms when it did; its rays start from the far end)
-            hd.last_in = kNative ? last_in : nrec - 1;
-            hdr[wray] = hd;
-            if (status != BL_RAY_HORIZON && status != BL_RAY_ESCAPED)
-                atomicAdd(&ctr->bad_rays, 1ull);
-            active = false;
-            attempts = 0;
-            nrec = 0;
-            status = 0;
-            last_in = -1;
-        }
-    }
-}
-#undef KX
-#undef KR
-#undef KSLOT
-
-template <class R, class G>
-__global__ void __launch_bounds__(128, BL_GEO_MIN_CTAS) geodesic_kernel(const ImageDesc* __restrict__ imgs,
-                                                          int n_images, int64_t ray_begin,
-                                                          int64_t ray_end,
-                                                          RayHdr* __restrict__ hdr,
-                                                          RecordSink<R> sink, int record,
-                                                          BlockSource bs,
-                                                          const RayInit* __restrict__ init) {
-    geodesic_body<R, G, true>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs, init);
+__global__ void __launch_bounds__(128, BL_GEO_MIN_CTAS) geodesic_df_kernel(
+        const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
+        RayHdr* __restrict__ hdr, RecordSink<float> sink, int record, BlockSource bs,
+        const RayInit* __restrict__ init) {
+    geodesic_df_body(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs, init);
 }
 
 // The FP64-arithmetic geodesic kernels (bl_geo64.cuh). Two shapes:
