@@ -345,6 +345,45 @@ void fill_desc(bl::ImageDesc& d, const bl_camera_t& c, const bl_metric_t& m, con
     d.ilv_shift = bl::kIlvShift;
 }
 
+// The FP32 transfer runs in two passes (samples, then transport) except for auxiliary images and,
+// without learned coefficients, plane-layout grids: those keep the consecutive queue and the single
+// kernel.
+bool two_pass32(int precision, const float* mlp, int feat, bool cells) {
+    return precision != BL_PREC_FP64 && !(feat & bl::kFAux) && (mlp || cells);
+}
+
+// Give every image's grid a field mask in the workspace's RayInit region, which is free while a
+// wave's transfer runs: images with the same grid share one. All or none: false (no masks) where
+// they do not fit, or where the wave has too few rays for reading the whole grid to pay (at most
+// 256 cells a ray and snapshot: 8 KB of grid, 1.2 ns of a ray's 25 ns or more).
+bool assign_masks(bl::ImageDesc* d, size_t n, char* ws, const Layout& L) {
+    const size_t room = L.chunks - L.init;
+    size_t used = 0;
+    double read = 0.0;
+    std::vector<size_t> at(n);
+    bool fits = true;
+    for (size_t q = 0; q < n && fits; ++q) {
+        d[q].mask_pitch = (d[q].nr + 31) / 32;
+        d[q].mask_own = 0;
+        size_t u = 0;
+        while (u < q && !(d[u].prim == d[q].prim && d[u].nr == d[q].nr && d[u].nt == d[q].nt &&
+                          d[u].nph == d[q].nph && d[u].layout == d[q].layout &&
+                          d[u].interp == d[q].interp && d[u].n_snap == d[q].n_snap)) ++u;
+        if (u < q) { at[q] = at[u]; continue; }
+        const size_t rows = (size_t)d[q].nt * d[q].nph;
+        at[q] = used;
+        d[q].mask_own = 1;
+        used += align_up(4 * rows * (size_t)d[q].mask_pitch);
+        read += (double)rows * d[q].nr * d[q].n_snap;
+        fits = used <= room && read <= 256.0 * (double)L.wave;
+    }
+    for (size_t q = 0; q < n; ++q) {
+        d[q].mask = fits ? (uint32_t*)(ws + L.init + at[q]) : nullptr;
+        if (!fits) d[q].mask_own = 0;
+    }
+    return fits;
+}
+
 // Queue the rays of a batch of equal images interleaved (see setup_ray) when every image has
 // the same number of rays, a whole number of kIlvBlock-ray blocks, at consecutive offsets, and
 // its grid (if any) in the cell layout. Grids in the plane layout keep the consecutive queue:
@@ -376,7 +415,7 @@ struct DevInfo {
     int geo64_wide = 0;             // FP64 form, the shape for fewer rays
     int tr_occ[2][8] = {};          // transfer variants: [double, float][feature bits]
     int tr_mlp_occ[2] = {0, 0};     // learned-coefficient transfer: [fast light, slow light]
-    int mi_occ[2] = {0, 0};         // learned-coefficient model inputs: [fast, slow light]
+    int s32_occ[4] = {0, 0, 0, 0};  // FP32 sample pass: [slow light + 2 learned]
     int pre_occ[2] = {0, 0};        // FP64 sample pass: [fast, slow light]
     int tr_pre_occ[2] = {0, 0};     // FP64 transfer after the sample pass: [fast, slow light]
     int fwd_list_occ = 0;           // the model over the work list
@@ -445,11 +484,13 @@ int dev_info(DevInfo& out) {
         if (rc) { di.sms = 0; return rc; }
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.tr_mlp_occ[0], bl::transfer_learned_kernel<false>, 128, 0));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.tr_mlp_occ[1], bl::transfer_learned_kernel<true>, 128, 0));
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.mi_occ[0], bl::mlp_inputs_kernel<false>, 128, 0));
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.mi_occ[1], bl::mlp_inputs_kernel<true>, 128, 0));
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.s32_occ[0], bl::fp32_samples_kernel<false, false>, 128, 0));
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.s32_occ[1], bl::fp32_samples_kernel<true, false>, 128, 0));
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.s32_occ[2], bl::fp32_samples_kernel<false, true>, 128, 0));
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.s32_occ[3], bl::fp32_samples_kernel<true, true>, 128, 0));
+        for (int i = 0; i < 4; ++i)
+            if (di.s32_occ[i] < 1) di.s32_occ[i] = 1;
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.fwd_list_occ, bl::mlp::forward_list_kernel, 128, 0));
-        for (int i = 0; i < 2; ++i)
-            if (di.mi_occ[i] < 1) di.mi_occ[i] = 1;
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.pre_occ[0], bl::fp64_samples_kernel<false>, 128, 0));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.pre_occ[1], bl::fp64_samples_kernel<true>, 128, 0));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.tr_pre_occ[0], bl::transport_fp64_kernel, bl::kTransferFp64Threads, 0));
@@ -525,6 +566,7 @@ struct LaunchCfg {
     // order mixes images, whose 64 scalar gathers a sample then miss L2 more: fast form on nine
     // plane-layout images, transfer 25.8 -> 32.5 ms)
     bool order_transfer = true;
+    bool masks = false;           // the descriptors name field masks to build (assign_masks)
 };
 
 // Every image's grid in the cell layout.
@@ -683,34 +725,47 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                 BL_CUDA(cudaGetLastError());
                 return 0;
             };
-            if (mlp) {
-                // learned coefficients in three passes: the samples with plasma and their model
-                // inputs, the model over the list of those, then the transfer reading the model's
-                // outputs, its rays longest first by that list
+            if (two_pass32(precision, mlp, cfg.feat, cfg.order_transfer)) {
+                // two passes: the samples with plasma (with learned coefficients then the model over
+                // their list), and transport and Stokes steps, rays longest first
                 float* mpool = (float*)(ws + L.pool);
                 float* my = (float*)(ws + L.mlp_y);
                 int32_t* tfirst = (int32_t*)(ws + L.tfirst);
                 int32_t* tnpl = (int32_t*)(ws + L.tnpl);
+                const unsigned long long pc = (unsigned long long)L.pool_chunks;
                 // per wave ray: farthest plasma sample -1 and no plasma samples until found
                 BL_CUDA(cudaMemsetAsync(tfirst, 0xff, sizeof(int32_t) * (size_t)(e - b), st));
                 BL_CUDA(cudaMemsetAsync(tnpl, 0, sizeof(int32_t) * (size_t)(e - b), st));
-                const unsigned mi_grid = (unsigned)(di.sms * di.mi_occ[slow ? 1 : 0]);
-                if (slow)
-                    bl::mlp_inputs_kernel<true><<<mi_grid, 128, 0, st>>>(
-                        d_desc, n_images, b, e, hdr, mpool, chunks, ctr, cfg.bs, my, tfirst, tnpl);
-                else
-                    bl::mlp_inputs_kernel<false><<<mi_grid, 128, 0, st>>>(
-                        d_desc, n_images, b, e, hdr, mpool, chunks, ctr, cfg.bs, my, tfirst, tnpl);
+                BL_CUDA(cudaMemsetAsync(thist, 0, sizeof(unsigned int) * bl::kCostBuckets, st));
+                if (cfg.masks) {
+                    bl::field_mask_kernel<<<(unsigned)(di.sms * 8), bl::kMaskThreads, 0, st>>>(d_desc, n_images);
+                    ++g_launches;
+                    BL_CUDA(cudaGetLastError());
+                }
+                const int mi = (slow ? 1 : 0) + (mlp ? 2 : 0);
+                const unsigned s_grid = (unsigned)(di.sms * di.s32_occ[mi]);
+                auto samples = mi == 0 ? bl::fp32_samples_kernel<false, false>
+                             : mi == 1 ? bl::fp32_samples_kernel<true, false>
+                             : mi == 2 ? bl::fp32_samples_kernel<false, true>
+                                       : bl::fp32_samples_kernel<true, true>;
+                samples<<<s_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, mpool, pc, chunks, ctr,
+                                                cfg.bs, my, tfirst, tnpl);
                 ++g_launches;
                 BL_CUDA(cudaGetLastError());
-                bl::mlp::forward_list_kernel<<<(unsigned)(di.sms * di.fwd_list_occ), 128, 0, st>>>(
-                    mlp, &ctr->mlp_rows, my, &ctr->mlp_timeouts);
+                if (mlp) {
+                    bl::mlp::forward_list_kernel<<<(unsigned)(di.sms * di.fwd_list_occ), 128, 0, st>>>(
+                        mlp, &ctr->mlp_rows, my, &ctr->mlp_timeouts);
+                    ++g_launches;
+                    BL_CUDA(cudaGetLastError());
+                }
+                const int64_t ob = (e - b + 1023) / 1024;
+                bl::order_groups_kernel<<<(unsigned)(ob < di.sms ? (ob > 0 ? ob : 1) : di.sms), 1024, 0, st>>>(
+                    tfirst, tnpl, tkey, cfg.bs, b, e, thist, tperm, ctr);
                 ++g_launches;
                 BL_CUDA(cudaGetLastError());
-                if ((rc = order_by_plasma())) return rc;
-                launch_transfer<float, float>(cfg.feat | bl::kFMlp, tr_grid, st, d_desc, n_images, b,
-                                              e, hdr, fpool, chunks, ctr, cfg.bs,
-                                              bl::SideIn{my, mlp, nullptr, nullptr, tfirst, tperm});
+                const bl::SideIn side{mlp ? my : nullptr, mlp, nullptr, nullptr, tfirst, tperm, pc};
+                launch_transfer<float, float>(cfg.feat | (mlp ? bl::kFMlp : 0), tr_grid, st, d_desc, n_images,
+                                              b, e, hdr, fpool, chunks, ctr, cfg.bs, side);
             } else if (precision != BL_PREC_FP64) {
                 if (cfg.order_transfer && (rc = order_by_records())) return rc;
                 launch_transfer<float, float>(cfg.feat, tr_grid, st, d_desc, n_images, b, e, hdr,
@@ -765,11 +820,9 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
 }
 
 // Upload the image descriptors, then launch_kernels.
-int launch_all(int32_t n_images, const std::vector<bl::ImageDesc>& descs, char* ws,
+int launch_all(int32_t n_images, std::vector<bl::ImageDesc>& descs, char* ws,
                const Layout& L, int precision, bool transfer, cudaStream_t st, bool timing,
                const float* mlp = nullptr, const LaunchCfg& cfg = LaunchCfg()) {
-    BL_CUDA(cudaMemcpyAsync(ws + L.descs, descs.data(), sizeof(bl::ImageDesc) * n_images,
-                            cudaMemcpyHostToDevice, st));
     LaunchCfg c = cfg;
     for (const auto& d : descs) {
         if (d.n_snap > 1) c.feat |= bl::kFSlow;
@@ -777,6 +830,10 @@ int launch_all(int32_t n_images, const std::vector<bl::ImageDesc>& descs, char* 
     }
     c.integrator = descs.empty() ? BL_INT_DP : descs[0].integrator;
     c.order_transfer = all_cells(descs.data(), descs.size());
+    c.masks = transfer && two_pass32(precision, mlp, c.feat, c.order_transfer) &&
+              assign_masks(descs.data(), descs.size(), ws, L);
+    BL_CUDA(cudaMemcpyAsync(ws + L.descs, descs.data(), sizeof(bl::ImageDesc) * n_images,
+                            cudaMemcpyHostToDevice, st));
     return launch_kernels(n_images, ws, L, precision, transfer, st, timing, mlp, c);
 }
 
@@ -962,6 +1019,7 @@ struct bl_plan {
     int ilv_shift = bl::kIlvShift;
     LaunchCfg cfg;
     float run_ms = 0.0f;
+    bool masks = false;      // the descriptors name field masks
     int64_t kernels_per_run = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -998,6 +1056,7 @@ int plan_time(bl_plan& P, const LaunchCfg& cfg, cudaStream_t st, float* ms) {
         c.integrator = P.descs[0].integrator;
         c.cost_order = P.order == 2;
         c.order_transfer = all_cells(P.descs.data(), P.descs.size());
+        c.masks = P.masks;
         if (!rc) rc = launch_kernels(P.n_images, P.ws, P.L, P.precision, true, st, false, P.mlp, c);
         if (!rc && it > 0) {
             if ((ce = cudaEventRecord(e1, st)) != cudaSuccess) rc = cuda_fail(ce, "record");
@@ -1110,6 +1169,7 @@ int plan_capture(bl_plan& P, cudaStream_t user) {
             c.integrator = P.descs[0].integrator;
             c.cost_order = P.order == 2;
             c.order_transfer = all_cells(P.descs.data(), P.descs.size());
+            c.masks = P.masks;
             rc = launch_kernels(P.n_images, P.ws, P.L, P.precision, true, st, false, P.mlp, c);
         }
         cudaGraph_t g = nullptr;
@@ -1208,6 +1268,7 @@ struct AdaptRun {
     std::vector<int32_t> h_root;
     std::vector<unsigned long long> h_counts0;
     std::vector<bl::OutDesc> h_outd;
+    bool masks = false;                     // the descriptors name field masks
 };
 
 int adapt_prepare(AdaptRun& R, int32_t n_images, const bl_camera_t* cams, const bl_metric_t* mets,
@@ -1281,6 +1342,9 @@ int adapt_prepare(AdaptRun& R, int32_t n_images, const bl_camera_t* cams, const 
             d.stokes = R.lvl;
             d.n_rays = R.cap_blocks[l] * b2;
         }
+    if (two_pass32(R.precision, R.mlp, R.feat, all_cells(R.h_descs.data(), (size_t)n_images)))
+        for (int l = 0; l < levels; ++l)
+            R.masks = assign_masks(R.h_descs.data() + (size_t)l * n_images, n_images, R.ws, R.L);
     // root block list (image-major, blocks row by row) and level-0 counts
     R.h_root.clear();
     R.h_counts0.assign(n_counts, 0ull);
@@ -1329,6 +1393,7 @@ int adapt_enqueue(AdaptRun& R, cudaStream_t st) {
         cfg.keep_bad = true;
         cfg.bs = bl::BlockSource{R.entries[l], R.counts + l, R.B};
         cfg.order_transfer = all_cells(R.h_descs.data(), (size_t)R.n_images);
+        cfg.masks = R.masks;
         int rc = launch_kernels(R.n_images, R.ws, Ll, R.precision, true, st, false, R.mlp, cfg);
         if (rc) return rc;
         const int s = 1 << (R.max_level - l);
@@ -1543,6 +1608,8 @@ int blacklight_plan_create(int32_t n_images, const bl_camera_t* cams, const bl_m
         delete P;
         return fail(BL_ENOMEM, "cudaMalloc(%zu bytes): %s", P->L.total, cudaGetErrorString(e));
     }
+    P->masks = two_pass32(precision, mlp, P->feat, all_cells(P->descs.data(), P->descs.size())) &&
+               assign_masks(P->descs.data(), P->descs.size(), P->ws, P->L);
     if (flags & BL_PLAN_AUTOTUNE) {
         rc = plan_autotune(*P, st);
     } else {

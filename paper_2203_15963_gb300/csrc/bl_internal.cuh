@@ -55,6 +55,10 @@ struct ImageDesc {
     int64_t n_rays;         // rays traced for this image (n * n, or blocks x block^2)
     int32_t order;          // ray order: 0 Morton (n a power of 2), 1 rows
     int32_t layout;         // grid memory order: 0 planes [8][phi][theta][r], 1 cells [...][8]
+    // field mask of the grid (field_mask_kernel), rows of mask_pitch words; nullptr: none.
+    // mask_own: this image's launch builds it
+    uint32_t* mask;
+    int32_t mask_own, mask_pitch;
     // filled by the camera-frame kernel
     double x_cam[4], u_cam[4], kk[4], hh[4], vv[4];
     double r_cam, r_hor;
@@ -118,6 +122,7 @@ struct SideIn {
     const unsigned char* pre_flag;
     const int32_t* first;    // each ray's farthest plasma sample, or -1 (learned and FP64 forms)
     const int32_t* perm;     // the transfer's ray order (wave ray indices), or nullptr
+    unsigned long long pool_chunks = 0;   // after the FP32 sample pass: the record pool's chunks
 };
 constexpr int kPreVals = 24;
 
@@ -125,8 +130,10 @@ struct Counters {
     unsigned long long next_ray_geo;
     unsigned long long next_ray_tr;
     unsigned long long pool_next;
-    unsigned long long next_ray_mi;    // learned-coefficient model inputs: rays handed out
+    unsigned long long next_ray_mi;    // sample passes: rays handed out
     unsigned long long mlp_rows;       // learned-coefficient work list: rows written
+    unsigned long long order_blocks;   // order_groups_kernel: CTAs done
+    unsigned long long exact_rows;     // FP32 sample pass: rows of samples with exact coefficients
     unsigned long long bad_rays;
     unsigned long long mlp_timeouts;   // CTAs whose tensor-core wait ran out (never expected)
 };

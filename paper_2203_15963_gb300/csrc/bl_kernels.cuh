@@ -852,10 +852,83 @@ __device__ __forceinline__ unsigned int cell_field_bits(const float* __restrict_
            __float_as_uint(__ldg(prim + 7 * plane + cell));
 }
 
+// Field mask of a grid: one bit a cell, set when a trilinear lookup with that lower cell (nearest:
+// the cell itself) reads a cell with magnetic field in any snapshot; rows of mask_pitch words. A
+// clear bit proves "no plasma" for a sample as the eight field reads would (b = 0), for one load
+// of a few bytes a row instead of eight 32-byte sectors; the grid is read once a wave to build it.
+// A CTA takes a tile of kMaskR x kMaskJ x kMaskK cells: first the own bits of the tile's rows and
+// of the next row, plane and cell (a word a warp and ballot, so reads are coalesced; 1.4 times the
+// tile's cells, the excess mostly from L2), then the stencils' bits from those, word by word.
+// 256x128x128 cells: 105 us (two launches over linear cells and bits: 183).
+constexpr int kMaskR = 512, kMaskJ = 8, kMaskK = 4, kMaskThreads = 256;
+__device__ __forceinline__ bool mask_clear(const ImageDesc& im, size_t row, int i) {
+    return ((__ldg(im.mask + row * (size_t)im.mask_pitch + (i >> 5)) >> (i & 31)) & 1u) == 0u;
+}
+__global__ void __launch_bounds__(kMaskThreads) field_mask_kernel(const ImageDesc* __restrict__ imgs,
+                                                                  int n_images) {
+    constexpr int kW = kMaskR / 32 + 1, kJ = kMaskJ + 1, kK = kMaskK + 1;
+    __shared__ uint32_t own[kK][kJ][kW];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int q = 0; q < n_images; ++q) {
+        const ImageDesc& im = imgs[q];
+        if (!im.mask_own) continue;
+        const int nr = im.nr, nt = im.nt, np = im.nph, ns = im.n_snap, layout = im.layout;
+        const bool tri = im.interp != 0;
+        const int64_t cells = (int64_t)nr * nt * np;
+        const int tr = (nr + kMaskR - 1) / kMaskR, tj = (nt + kMaskJ - 1) / kMaskJ;
+        const int64_t tiles = (int64_t)tr * tj * ((np + kMaskK - 1) / kMaskK);
+        for (int64_t t = blockIdx.x; t < tiles; t += gridDim.x) {
+            const int i0 = (int)(t % tr) * kMaskR, j0 = (int)(t / tr % tj) * kMaskJ;
+            const int k0 = (int)(t / tr / tj) * kMaskK;
+            // words that hold cells: those of the segment and the first of the next
+            const int nw = min(kW, (nr - i0 + 31) >> 5);
+            const int rows_j = tri ? kJ : kMaskJ, rows = rows_j * (tri ? kK : kMaskK);
+            for (int row = warp; row < rows; row += kMaskThreads / 32) {
+                const int jj = row % rows_j, kk = row / rows_j;
+                // phi is periodic; a tile needs at most plane np, which is plane 0
+                const int k = k0 + kk;
+                const bool in = j0 + jj < nt && (k < np || (tri && k == np));
+                const int64_t c0 = ((int64_t)(k == np ? 0 : k) * nt + j0 + jj) * nr + i0 + lane;
+                for (int w = 0; w < nw; w += 4) {
+                    // four words a turn, so that four loads are in flight
+                    unsigned bits[4] = {0u, 0u, 0u, 0u};
+                    for (int sn = 0; sn < ns; ++sn) {
+                        const float* __restrict__ p = im.prim + (size_t)sn * 8 * cells;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            if (in && i0 + 32 * (w + u) + lane < nr && w + u < nw)
+                                bits[u] |= cell_field_bits(p, layout, cells, c0 + 32 * (w + u));
+                    }
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const unsigned word = __ballot_sync(0xffffffffu, (bits[u] & 0x7fffffffu) != 0u);
+                        if (lane == 0 && w + u < nw) own[kk][jj][w + u] = word;
+                    }
+                }
+            }
+            __syncthreads();
+            for (int it = threadIdx.x; it < kMaskK * kMaskJ * (kW - 1); it += kMaskThreads) {
+                const int w = it % (kW - 1), jj = it / (kW - 1) % kMaskJ, kk = it / (kW - 1) / kMaskJ;
+                if (i0 + 32 * w >= nr || j0 + jj >= nt || k0 + kk >= np) continue;
+                unsigned o = own[kk][jj][w];
+                if (tri) {
+                    o |= own[kk][jj + 1][w] | own[kk + 1][jj][w] | own[kk + 1][jj + 1][w];
+                    const unsigned n = w + 1 >= nw ? 0u
+                        : own[kk][jj][w + 1] | own[kk][jj + 1][w + 1] |
+                          own[kk + 1][jj][w + 1] | own[kk + 1][jj + 1][w + 1];
+                    o |= (o >> 1) | (n << 31);
+                }
+                im.mask[((int64_t)(k0 + kk) * nt + j0 + jj) * im.mask_pitch + (i0 >> 5) + w] = o;
+            }
+            __syncthreads();
+        }
+    }
+}
+
 // field_test: first read the stencil's magnetic field alone and return false (no plasma) when
 // every corner's field is zero -- exact (b = 0 fails the b^2 > 0 test below), and it skips the
 // interpolation and the plasma state at such samples.
-template <class T, bool kSlow = false>
+template <class T, bool kSlow = false, bool kPinned = false>
 __device__ __forceinline__ bool plasma_at(const ImageDesc& im, const T x[3], T t,
                                           const KSGeom<T>& G, Plasma<T>& P, bool field_test) {
     const T a = ic<T>(im, kcSpin);
@@ -869,7 +942,12 @@ __device__ __forceinline__ bool plasma_at(const ImageDesc& im, const T x[3], T t
     // phi = arg(x + i y) - arg(r + i a) = arg((x + i y)(r - i a)), in (-pi, pi]; one wrap
     // puts it in [0, 2 pi) (fmod by 2 pi would return such a value unchanged). Its sine and
     // cosine are that complex number normalised (on the axis, where it vanishes, phi = 0).
-    const T zre = x[0] * r + x[1] * a, zim = x[1] * r - x[0] * a;
+    // (kPinned: the FP32 roundings of ks_geom_pinned, whose l_x and l_y share these)
+    T zre = x[0] * r + x[1] * a, zim = x[1] * r - x[0] * a;
+    if constexpr (kPinned) {
+        zre = __fmaf_rn(a, x[1], __fmul_rn(r, x[0]));
+        zim = __fmaf_rn(-a, x[0], __fmul_rn(r, x[1]));
+    }
     T ph = atan2(zim, zre);
     if (ph < T(0)) ph += twopi;
     if (ph >= twopi) ph -= twopi;
@@ -911,7 +989,9 @@ __device__ __forceinline__ bool plasma_at(const ImageDesc& im, const T x[3], T t
         const size_t base = ((size_t)k * nt + j) * nr + i;
         // a cell without magnetic field holds no plasma (b = 0, below): its field
         // components alone decide that
-        if (field_test) {
+        if (sizeof(T) == sizeof(float) && im.mask) {
+            if (mask_clear(im, (size_t)k * nt + j, i)) return false;
+        } else if (field_test) {
             unsigned int fb = cell_field_bits(prim, im.layout, plane, base);
             if (kSlow && prim1) fb |= cell_field_bits(prim1, im.layout, plane, base);
             if ((fb & 0x7fffffffu) == 0u) return false;
@@ -968,7 +1048,9 @@ __device__ __forceinline__ bool plasma_at(const ImageDesc& im, const T x[3], T t
         const size_t o10 = ((size_t)k1 * nt + j0) * nr, o11 = ((size_t)k1 * nt + j1) * nr;
         // a stencil whose eight cells carry no magnetic field holds no plasma (b = 0, below):
         // the field components alone decide that, before the interpolation
-        if (field_test) {
+        if (sizeof(T) == sizeof(float) && im.mask) {
+            if (mask_clear(im, (size_t)k0 * nt + j0, i0)) return false;
+        } else if (field_test) {
             const size_t cell[8] = {o00 + i0, o00 + i1, o01 + i0, o01 + i1,
                                     o10 + i0, o10 + i1, o11 + i0, o11 + i1};
             unsigned int fb = 0u;
@@ -1194,8 +1276,16 @@ __device__ __forceinline__ void stokes_to_coh(const T e1[4], const T e2[4], cons
 #pragma unroll
     for (int a_ = 0; a_ < 4; ++a_)
 #pragma unroll
-        for (int b_ = a_; b_ < 4; ++b_)
-            n.re[k++] = pe1[a_] * e1[b_] + qe2[a_] * e2[b_] + ue1[a_] * e2[b_] + ue2[a_] * e1[b_];
+        for (int b_ = a_; b_ < 4; ++b_) {
+            if constexpr (sizeof(T) == sizeof(float)) {
+                // roundings written out: the same bits in the single kernel and the transport pass
+                const T pq = b_ & 1 ? __fmaf_rn(qe2[a_], e2[b_], __fmul_rn(pe1[a_], e1[b_]))
+                                    : __fmaf_rn(pe1[a_], e1[b_], __fmul_rn(qe2[a_], e2[b_]));
+                n.re[k++] = __fmaf_rn(ue2[a_], e1[b_], __fmaf_rn(ue1[a_], e2[b_], pq));
+            } else {
+                n.re[k++] = pe1[a_] * e1[b_] + qe2[a_] * e2[b_] + ue1[a_] * e2[b_] + ue2[a_] * e1[b_];
+            }
+        }
     k = 0;
 #pragma unroll
     for (int a_ = 0; a_ < 4; ++a_)
@@ -1245,6 +1335,24 @@ __device__ __forceinline__ int64_t record_index(const int32_t* __restrict__ chun
 // ---------------------------------------------------------------------------------------
 // What the learned-coefficient form's first pass found at a sample (a record's last value).
 enum : unsigned { kSampleEmpty = 0u, kSampleExact = 1u, kSampleModel = 2u };
+
+// The FP32 sample pass's results, kPreVals floats a plasma sample, live in the part of the record
+// pool that the wave's geodesics left unused (the pool is sized for the longest rays): model rows
+// from its start, at their work list's index, the others from its end. Where they do not all fit,
+// the pass's rows are not used and the single-kernel transfer runs instead.
+__device__ __forceinline__ unsigned long long sample_rows_cap(const Counters* ctr,
+                                                              unsigned long long pool_chunks) {
+    const unsigned long long used = ctr->pool_next < pool_chunks ? ctr->pool_next : pool_chunks;
+    return (pool_chunks - used) * (unsigned long long)(kChunk * RecStride<float>::v) / kPreVals;
+}
+__device__ __forceinline__ float* sample_rows(float* pool, const Counters* ctr,
+                                              unsigned long long pool_chunks) {
+    const unsigned long long used = ctr->pool_next < pool_chunks ? ctr->pool_next : pool_chunks;
+    return pool + used * (unsigned long long)(kChunk * RecStride<float>::v);
+}
+__device__ __forceinline__ bool sample_rows_fit(const Counters* ctr, unsigned long long pool_chunks) {
+    return ctr->mlp_rows + ctr->exact_rows <= sample_rows_cap(ctr, pool_chunks);
+}
 // Features of a transfer-kernel variant (compile-time, so that each variant carries only the
 // registers it needs).
 enum { kFSlow = 1, kFUnpol = 2, kFAux = 4, kFMlp = 8 };
@@ -1354,11 +1462,13 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
     constexpr bool kSlow = (kF & kFSlow) != 0;
     constexpr bool kUnpol = (kF & kFUnpol) != 0;
     constexpr bool kAux = (kF & kFAux) != 0;
-    // learned coefficients: the first pass (mlp_inputs_kernel) has found the samples that carry
-    // plasma; the model's outputs are in mlp_y, 8 floats a row of its work list
+    // learned coefficients: the model's outputs are in mlp_y, 8 floats a row of its work list
     constexpr bool kMlp = (kF & kFMlp) != 0;
     static_assert(!kMlp || std::is_same<R, float>::value, "the learned model needs FP32 records");
-    constexpr int kGroup = kMlp ? kTransportGroup : kFusedGroup;
+    // after the FP32 sample pass this body runs only where that pass's rows did not fit: the rays
+    // come in warp-sized groups by their plasma work, start at their farthest plasma sample and look
+    // up plasma samples only
+    const bool marked = sizeof(R) == sizeof(float) && side.pool_chunks != 0ull;
     // the stencil field test of plasma_at: always in the FP64 form; in FP32 where the rays are
     // not queued by record count -- that order predicts a ray's cost from its records, which
     // stops holding once field-free records are cheap (nine 256^2 images, fast form: cell-layout
@@ -1371,7 +1481,8 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
     const bool field_test = kFieldTestable && (sizeof(T) == sizeof(double) || side.perm == nullptr);
     const int64_t re = wave_end(bs, ray_end);
     const int64_t n_rays = re > ray_begin ? re - ray_begin : 0;
-    const int64_t total_rays = side.perm ? ordered_total<kGroup>(n_rays) : n_rays;
+    const int64_t total_rays = !side.perm ? n_rays : marked ? ordered_total<kTransportGroup>(n_rays)
+                                                             : ordered_total<kFusedGroup>(n_rays);
     int64_t wray = 0;
     bool active = false;
     int64_t ray = 0, opix = 0;
@@ -1394,7 +1505,9 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
             if ((int64_t)got >= total_rays) exhausted = true;
             else {
                 // the wave's rays in the order of their record counts where there is one
-                wray = side.perm ? ordered_ray<kGroup>(side.perm, got, n_rays) : (int64_t)got;
+                wray = !side.perm ? (int64_t)got
+                       : marked ? ordered_ray<kTransportGroup>(side.perm, got, n_rays)
+                                : ordered_ray<kFusedGroup>(side.perm, got, n_rays);
                 ray = ray_begin + wray;
             }
         }
@@ -1422,9 +1535,8 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
                 }
                 continue;
             }
-            // (the learned form from the farthest plasma sample: N = 0 beyond it)
-            if constexpr (kMlp) idx = side.first[wray] > 0 ? side.first[wray] : 0;
-            else idx = transfer_start(hd);
+            // (from the farthest plasma sample: N = 0 beyond it)
+            idx = marked ? max(side.first[wray], 0) : transfer_start(hd);
             load_record<R>(record_ptr(pool, chunks, wray, idx), nxt);
             kt = (T)hd.kt;
             nu_norm = (T)(hd.nnorm * im.freq);
@@ -1452,10 +1564,8 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
 #pragma unroll
             for (int c = 0; c < kRecVals; ++c) cur[c] = (T)nxt[c];
             nxt_t = (T)nxt[13];
-            if constexpr (kMlp) {
-                cur_row = __float_as_uint((float)nxt[14]);
-                cur_what = __float_as_uint((float)nxt[15]);
-            }
+            if constexpr (kMlp) cur_row = __float_as_uint((float)nxt[14]);
+            if constexpr (std::is_same<R, float>::value) cur_what = __float_as_uint((float)nxt[15]);
             if (idx > 0) load_record<R>(record_ptr(pool, chunks, wray, idx - 1), nxt);
         }
         if (!kUnpol && started) {
@@ -1492,12 +1602,16 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
             active = false;
             continue;
         }
-        if (!kMlp || cur_what != kSampleEmpty) {
+        if (!marked || cur_what != kSampleEmpty) {
             const T xs[3] = {cur[0], cur[1], cur[2]};
             KSGeom<T> G;
-            ks_geom<T>(xs[0], xs[1], xs[2], a, m, flat, false, G);
+            // the sample pass's roundings (the auxiliary images, which it does not make, and the
+            // learned form keep the compiler's)
+            constexpr bool kPinned = sizeof(T) == sizeof(float) && !kAux && !kMlp;
+            if constexpr (kPinned) ks_geom_pinned<false>(xs[0], xs[1], xs[2], a, m, flat, G);
+            else ks_geom<T>(xs[0], xs[1], xs[2], a, m, flat, false, G);
             Plasma<T> P;
-            if (plasma_at<T, kSlow>(im, xs, nxt_t, G, P, field_test)) {
+            if (plasma_at<T, kSlow, kPinned>(im, xs, nxt_t, G, P, field_test)) {
                 const T kl[4] = {kt, cur[3], cur[4], cur[5]};
                 T ku[4];
                 raise4(G, kl, ku);
@@ -1547,15 +1661,162 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
         --idx;
     }
 }
-// The transfer kernel: FP32 (mixed and fast forms) in CTAs of 128 threads, the polarized and
-// unpolarized variants held to 4 CTAs an SM (128 registers; with the field test uncapped they
-// take 142 and 3 CTAs), the slow-light and auxiliary-image variants uncapped; FP64 capped
+// FP32 forms, second pass of the transfer: along each ray from its farthest plasma sample, the
+// merged N half-steps and at each plasma sample the Stokes step with the first pass's row
+// (learned coefficients: from the model's outputs), the operations of the single kernel
+// (transfer_body) in its order. The row of the sample is asked for when the sample's record
+// arrives and read after the transport step. Bound by the latency of its serial chain of matrix
+// steps (nine 256^2 images 3.26 ms with 4 CTAs an SM; 3: 3.7, 5: 3.3, 6: 3.7).
+template <bool kUnpol, bool kMlp>
+__device__ __forceinline__ void transport32_body(
+        const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
+        const RayHdr* __restrict__ hdr, const float* __restrict__ pool,
+        const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side) {
+    using T = float;
+    const float* const row_base = sample_rows(const_cast<float*>(pool), ctr, side.pool_chunks);
+    const int64_t re = wave_end(bs, ray_end);
+    const int64_t n_rays = re > ray_begin ? re - ray_begin : 0;
+    const int64_t total_rays = ordered_total<kTransportGroup>(n_rays);
+    int64_t wray = 0, opix = 0;
+    bool active = false, started = false, exhausted = false;
+    int q = 0;
+    int32_t idx = 0;
+    Coh<T> N;
+    T Iu = T(0);
+    T prev[kRecVals];
+    T nxt[RecStride<float>::v];
+    T kt = T(0), a = T(0), m = T(0);
+    bool flat = false;
+    while (true) {
+        const bool need = !active && !exhausted;
+        const unsigned long long got = warp_refill(&ctr->next_ray_tr, need);
+        if (need) {
+            if ((int64_t)got >= total_rays) exhausted = true;
+            else wray = ordered_ray<kTransportGroup>(side.perm, got, n_rays);
+        }
+        if (!__any_sync(0xffffffffu, active || (need && !exhausted))) break;
+        if (!active && !(need && !exhausted)) continue;
+        if (!active && wray < 0) continue;   // a partial order group's empty position
+        if (!active) {
+            int pi, pj;
+            setup_ray(imgs, n_images, bs, ray_begin + wray, q, opix, pi, pj);
+            const ImageDesc& im = imgs[q];
+            const RayHdr hd = hdr[wray];
+            if (hd.status == BL_RAY_OVERFLOW || hd.nrec == 0) {
+                const double val = hd.status == BL_RAY_OVERFLOW ? nan("") : 0.0;
+                for (int s = 0; s < 4; ++s) {
+                    if (im.dtype == 0) ((double*)im.stokes)[s * (int64_t)im.n_rays + opix] = val;
+                    else ((float*)im.stokes)[s * (int64_t)im.n_rays + opix] = (float)val;
+                }
+                continue;
+            }
+            idx = max(side.first[wray], 0);
+            load_record<float>(record_ptr(pool, chunks, wray, idx), nxt);
+            kt = (T)hd.kt;
+            a = ic<T>(im, kcSpin);
+            m = ic<T>(im, kcMass);
+            flat = im.flat != 0;
+#pragma unroll
+            for (int c = 0; c < 10; ++c) N.re[c] = T(0);
+#pragma unroll
+            for (int c = 0; c < 6; ++c) N.im[c] = T(0);
+            Iu = T(0);
+            started = false;
+            active = true;
+        }
+        const ImageDesc& im = imgs[q];
+        // idx < 0: the last half-step to the camera node and the read-out
+        const bool finishing = idx < 0;
+        T cur[kRecVals];
+        unsigned what = kSampleEmpty, at = 0u;
+        const float4* row = nullptr;
+        if (!finishing) {
+#pragma unroll
+            for (int c = 0; c < kRecVals; ++c) cur[c] = nxt[c];
+            at = __float_as_uint(nxt[14]);
+            what = __float_as_uint(nxt[15]);
+            if (idx > 0) load_record<float>(record_ptr(pool, chunks, wray, idx - 1), nxt);
+            if (what != kSampleEmpty) {
+                row = reinterpret_cast<const float4*>(row_base + kPreVals * (size_t)at);
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(row));
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(row + 5));
+            }
+        }
+        if (!kUnpol && started) {
+            const T kp[4] = {kt, prev[3], prev[4], prev[5]};
+            const T kn[4] = {kt, prev[9], prev[10], prev[11]};
+            coh_pc_step<T>(N, prev, kp, prev + 6, kn, a, m, flat,
+                           T(0.5) * (prev[12] + (finishing ? T(0) : cur[12])));
+        }
+        if (finishing) {
+            const int64_t npix = im.n_rays;
+            T sv[4] = {Iu, T(0), T(0), T(0)};
+            if constexpr (!kUnpol) {
+                // read out in the camera basis at the camera-side node
+                KSGeom<T> G;
+                ks_geom<T>(prev[6], prev[7], prev[8], a, m, flat, false, G);
+                T hl[4], vl[4];
+                lower4(G, im.f_hh, hl);
+                lower4(G, im.f_vv, vl);
+                coh_to_stokes(N, hl, vl, sv);
+            }
+            for (int c = 0; c < 4; ++c) {
+                if (im.dtype == 0) ((double*)im.stokes)[c * npix + opix] = (double)sv[c];
+                else ((float*)im.stokes)[c * npix + opix] = (float)sv[c];
+            }
+            active = false;
+            continue;
+        }
+        if (what != kSampleEmpty) {
+            T v[kPreVals];
+#pragma unroll
+            for (int i = 0; i < (kUnpol ? 2 : kPreVals / 4); ++i) {
+                const float4 d = __ldg(row + i);
+                v[4 * i] = d.x;
+                v[4 * i + 1] = d.y;
+                v[4 * i + 2] = d.z;
+                v[4 * i + 3] = d.w;
+            }
+            if constexpr (kMlp) {
+                if (what == kSampleModel) {
+                    const mlp::ModelIn mi = mlp::model_inputs(v[1], v[2], v[3], v[4]);
+                    const float4* yq = reinterpret_cast<const float4*>(side.mlp_y + 8 * (size_t)at);
+                    const float4 y0 = __ldg(yq), y1 = __ldg(yq + 1);
+                    const float y[7] = {y0.x, y0.y, y0.z, y0.w, y1.x, y1.y, y1.z};
+                    float o[7], co[8];
+                    mlp::model_outputs_from_y(side.mlp_params, y, mi.f, o);
+                    mlp::coefficients_from(o, v[0], v[1], v[2], v[3], v[4], co);
+                    const T eg = v[5], path = v[6];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) v[c] = co[c] * (c < 3 ? eg : path);
+                }
+            }
+            if constexpr (kUnpol) {
+                Iu = unpolarized_step<T>(v[0], v[3], cur[12], Iu);
+            } else {
+                T s0[4], s1[4];
+                coh_to_stokes(N, v + 16, v + 20, s0);
+                stokes_step<T>(v, s0, cur[12], s1);
+                stokes_to_coh(v + 8, v + 12, s1, N);
+            }
+            started = true;
+        }
+#pragma unroll
+        for (int c = 0; c < kRecVals; ++c) prev[c] = cur[c];
+        --idx;
+    }
+}
+
+// The transfer kernels. FP32: after the sample pass the transport body, or, where its rows did not
+// fit, the single-kernel body; the latter alone for auxiliary images and plane-layout grids. CTAs
+// of 128 threads, 4 an SM (128 registers), the auxiliary-image variants uncapped. FP64: unpolarized
+// and auxiliary images, capped
 // (BL_TR64_MAXNREG) in CTAs of 64 threads, which keeps more warps an SM resident.
 #ifndef BL_TR32_MIN_CTAS
 #define BL_TR32_MIN_CTAS 4
 #endif
 template <class T, class R, int kF>
-__global__ void __launch_bounds__(128, (kF & (kFSlow | kFAux)) ? 0 : BL_TR32_MIN_CTAS) transfer_kernel(const ImageDesc* __restrict__ imgs,
+__global__ void __launch_bounds__(128, (kF & kFAux) ? 0 : BL_TR32_MIN_CTAS) transfer_kernel(const ImageDesc* __restrict__ imgs,
                                                        int n_images, int64_t ray_begin,
                                                        int64_t ray_end,
                                                        const RayHdr* __restrict__ hdr,
@@ -1563,6 +1824,13 @@ __global__ void __launch_bounds__(128, (kF & (kFSlow | kFAux)) ? 0 : BL_TR32_MIN
                                                        const int32_t* __restrict__ chunks,
                                                        Counters* ctr, BlockSource bs,
                                                        SideIn side) {
+    if constexpr ((kF & kFAux) == 0) {
+        if (side.pool_chunks != 0ull && sample_rows_fit(ctr, side.pool_chunks)) {
+            transport32_body<(kF & kFUnpol) != 0, false>(imgs, n_images, ray_begin, ray_end, hdr,
+                                                         pool, chunks, ctr, bs, side);
+            return;
+        }
+    }
     transfer_body<T, R, kF>(imgs, n_images, ray_begin, ray_end, hdr, pool, chunks, ctr, bs, side);
 }
 // Register cap and CTA size of the FP64 transfer kernel. Its FP64 arithmetic runs at 1/64 of
@@ -1576,14 +1844,16 @@ __global__ void __launch_bounds__(128, (kF & (kFSlow | kFAux)) ? 0 : BL_TR32_MIN
 #ifndef BL_TR64_THREADS
 #define BL_TR64_THREADS 64
 #endif
-// The transfer of the learned-coefficient form (its model outputs from the pool pass),
-// compiled for 4 resident CTAs an SM (128 registers; uncapped it takes 142 registers and 3
-// CTAs, measured 62.5 against 58.9 ms at 1024^2).
+// The learned-coefficient form's.
 template <bool kSlow>
 __global__ void __launch_bounds__(128, 4) transfer_learned_kernel(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         const RayHdr* __restrict__ hdr, const float* __restrict__ pool,
         const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side) {
+    if (sample_rows_fit(ctr, side.pool_chunks)) {
+        transport32_body<false, true>(imgs, n_images, ray_begin, ray_end, hdr, pool, chunks, ctr, bs, side);
+        return;
+    }
     transfer_body<float, float, kFMlp | (kSlow ? kFSlow : 0)>(
         imgs, n_images, ray_begin, ray_end, hdr, pool, chunks, ctr, bs, side);
 }
@@ -1655,10 +1925,12 @@ __device__ __forceinline__ int certain_cell_periodic(float u, float m) {
 // (x^2 + y^2 = (r^2 + a^2) sin^2 theta in Cartesian Kerr-Schild), the azimuth as plasma_at
 // forms it. Each fractional coordinate carries a margin of 1e-3 cells plus four times a bound
 // on its FP32 error (the rounding of r^2 grows with (R^2 + a^2) / r^2, R^2 = x^2 + y^2 + z^2)
-// and the rounding of the FP32 scale factors;
+// and the rounding of the FP32 scale factors; theta's is divided by sin theta, which covers the
+// FP32 lookup's acos as well (the FP32 transfers read their marks from here);
 // a coordinate whose margin interval straddles a cell boundary, or a point within 1e-15 of
 // the axis, is reported as not certain (false: the FP64 lookup decides). A true answer is
 // exact: the FP64 lookup then reads the same stencil and returns no plasma.
+template <bool kMask>   // the image's field mask, where it has one
 __device__ __forceinline__ bool stencil_field_free(const ImageDesc& im, float x, float y, float z,
                                                    float r2, float aa) {
     const float rho2 = x * x + y * y;
@@ -1667,7 +1939,8 @@ __device__ __forceinline__ bool stencil_field_free(const ImageDesc& im, float x,
     const float eps = 3e-7f * (R2 + aa) / r2 + 2e-7f;
     const float r = sqrtf(r2);
     const float a = im.f_c[kcSpin];
-    const float th = atan2f(sqrtf(rho2 / (r2 + aa)), z / r);
+    const float sth = sqrtf(rho2 / (r2 + aa));
+    const float th = atan2f(sth, z / r);
     float ph = atan2f(y * r - x * a, x * r + y * a);
     const float twopi = 6.28318530717958648f;
     if (ph < 0.0f) ph += twopi;
@@ -1683,12 +1956,13 @@ __device__ __forceinline__ bool stencil_field_free(const ImageDesc& im, float x,
     const float ut = th * idth - off;
     const float up = ph * idph - off;
     const int i0 = certain_cell(ur, 1e-3f + idlr * (4.0f * eps + 1e-6f) + 4e-7f * fabsf(ur), nr, tri);
-    const int j0 = certain_cell(ut, 1e-3f + idth * (4.0f * eps + 1e-6f) + 4e-7f * fabsf(ut), nt, tri);
+    const int j0 = certain_cell(ut, 1e-3f + idth * (4.0f * eps / fminf(sth, 1.0f) + 1e-6f) + 4e-7f * fabsf(ut), nt, tri);
     const int kf = certain_cell_periodic(up, 1e-3f + idph * (2.0f * eps + 1e-6f) + 4e-7f * fabsf(up));
     if (i0 < 0 || j0 < 0 || kf == INT_MIN) return false;
     const int k0 = ((kf % np) + np) % np;
     const int i1 = (tri && nr > 1) ? i0 + 1 : i0, j1 = (tri && nt > 1) ? j0 + 1 : j0;
     const int k1 = tri ? (k0 + 1) % np : k0;
+    if (kMask && im.mask) return mask_clear(im, (size_t)k0 * nt + j0, i0);
     const size_t plane = (size_t)np * nt * nr;
     unsigned int bits = 0u;
 #pragma unroll
@@ -1830,7 +2104,7 @@ __global__ void __launch_bounds__(128, BL_PRE64_MIN_CTAS) fp64_samples_kernel(co
                 cand = r2 >= r2lo && r2 <= r2hi;
                 // a stencil without magnetic field holds no plasma (stencil_field_free);
                 // one snapshot only
-                if (!kSlow && cand) cand = !stencil_field_free(imgs[q], x, y, z, r2, aa);
+                if (!kSlow && cand) cand = !stencil_field_free<false>(imgs[q], x, y, z, r2, aa);
                 if (!cand) pre_flag[k] = 0;
             }
             const unsigned mask = __ballot_sync(0xffffffffu, cand);
@@ -1878,6 +2152,39 @@ __global__ void transport_key_kernel(const int32_t* __restrict__ tfirst,
         const int32_t k = on ? tfirst[w] + 1 + (npl[w] >> 1) : -1;
         group_key<kTransportGroup>(k, on, w, key, hist);
     }
+}
+
+// The same keys and the whole order in one launch, for the FP32 forms: the CTA that finishes its
+// keys last scans the histogram and lists the groups (one for 32 rays, so a single CTA's scatter
+// of a million rays takes about as long as the two launches it replaces).
+__global__ void __launch_bounds__(1024) order_groups_kernel(const int32_t* __restrict__ tfirst,
+                                                            const int32_t* __restrict__ npl,
+                                                            int32_t* key, BlockSource bs,
+                                                            int64_t ray_begin, int64_t ray_end,
+                                                            unsigned int* hist,
+                                                            int32_t* __restrict__ perm, Counters* ctr) {
+    __shared__ unsigned int start[kCostBuckets];
+    __shared__ bool last;
+    const int64_t re = wave_end(bs, ray_end);
+    const int64_t n = re > ray_begin ? re - ray_begin : 0;
+    for (int64_t w0 = (int64_t)blockIdx.x * 1024; w0 < n; w0 += (int64_t)gridDim.x * 1024) {
+        const int64_t w = w0 + threadIdx.x;
+        const bool on = w < n;
+        const int32_t k = on ? tfirst[w] + 1 + (npl[w] >> 1) : -1;
+        group_key<kTransportGroup>(k, on, w, key, hist);
+    }
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(&ctr->order_blocks, 1ull) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int b = threadIdx.x; b < kCostBuckets; b += 1024) start[b] = __ldcg(hist + b);
+    __syncthreads();
+    bucket_scan(start);
+    const int64_t groups = (n + kTransportGroup - 1) / kTransportGroup;
+    for (int64_t g = threadIdx.x; g < groups; g += 1024)
+        perm[atomicAdd(&start[cost_bucket(__ldcg(key + g))], 1u)] = (int32_t)g;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -2024,103 +2331,132 @@ __global__ void __launch_bounds__(128, kTransport64WideCtas) transport64_wide_ke
 }
 
 // ---------------------------------------------------------------------------------------
-// Learned coefficients, first pass: which samples carry plasma, and their model inputs. Work is
-// compacted per warp as in the FP64 sample pass: a warp takes rays in turn, tests a chunk of 32
-// records at a time by position alone (the grid's radial shell with 1e-4 margins, the stencil
-// certainly without magnetic field; the next chunk's positions are loaded meanwhile), queues the
-// records that may carry plasma in shared memory and evaluates 32 of them at a time, whatever
-// rays they belong to: geometry, plasma state, fluid-frame frequency and pitch angle as the
-// transfer computes them. A record's last value says what the later passes find there:
-// kSampleEmpty (no plasma; the geodesic kernels write it so), kSampleExact (plasma outside the
-// model's domain) or kSampleModel, with the sample's row of the model's work list in the value
-// before it. The rows wait in shared memory until 128 are together, so the list fills densely
-// with one atomic for each 128, and the model pass neither scans the pool nor holds empty rows.
-// Each ray's farthest plasma sample and its number of plasma samples (atomics, one a ray and
-// batch; tfirst -1 and tnpl 0 beforehand) start and order the transfer. Bound by the latency of
-// the record and stencil reads: 10.7 ms at 1024^2 on the 512x256x256 torus (11.1 without the
-// work list, the order's inputs and the start they buy; one warp a ray with the list 14.5).
+// FP32 forms, first pass of the transfer: everything a sample needs that does not depend on the
+// ray's running coherency, for the samples with plasma. Work is compacted per warp as in the FP64
+// sample pass: a warp takes rays in turn, tests a chunk of 32 records at a time by position alone
+// (the grid's radial shell with 1e-4 margins, the stencil certainly without magnetic field; the
+// next chunk's positions are loaded meanwhile), queues the records that may carry plasma in shared
+// memory and evaluates 32 of them at a time, whatever rays they belong to: in the single kernel
+// a warp's lanes meet plasma at different steps (12.7 of 32 lanes active on nine 256^2 images).
+// A record's last value says what the second pass finds there: kSampleEmpty (no plasma; the
+// geodesic kernels write it so), kSampleExact (a row of scaled coefficients and fluid basis) or,
+// with learned coefficients inside the model's domain, kSampleModel (a row of the model's
+// denormalisation and the basis, and an input row of the model's work list); its row's index is in
+// the value before it. Each ray's farthest plasma sample and its number of plasma samples
+// (atomics, one a ray and batch; tfirst -1 and tnpl 0 beforehand) start and order the second pass.
+// Bound by instruction issue and the latency of the record and stencil reads: nine 256^2 images
+// 3.7 ms in 72 registers and 7 CTAs an SM (8 CTAs 3.8, 6: 3.9, 5: 4.4, 4: 5.0), the learned form at 1024^2 6.7 in
+// 64 and 8 CTAs (7: 7.0, 5: 7.2, 4: 9.0). Both passes: nine images 11.3 -> 7.0 ms, slow light at
+// 512^2 6.6 -> 3.4, learned without the model 20.1 -> 13.2.
 // ---------------------------------------------------------------------------------------
-struct LearnedItem {
+struct Sample32Item {
     float* rec;
     int32_t wray, idx, q, pad_;
 };
-constexpr int kListFlush = 128, kListQueue = kListFlush + 31;
-template <bool kSlow>
-__global__ void __launch_bounds__(128, 6) mlp_inputs_kernel(const ImageDesc* __restrict__ imgs,
+#ifndef BL_S32_MIN_CTAS
+#define BL_S32_MIN_CTAS 7
+#endif
+template <bool kSlow, bool kMlp>
+__global__ void __launch_bounds__(128, kMlp ? 8 : BL_S32_MIN_CTAS) fp32_samples_kernel(const ImageDesc* __restrict__ imgs,
                                                          int n_images, int64_t ray_begin,
                                                          int64_t ray_end,
                                                          const RayHdr* __restrict__ hdr,
                                                          float* __restrict__ pool,
+                                                         unsigned long long pool_chunks,
                                                          const int32_t* __restrict__ chunks,
                                                          Counters* ctr, BlockSource bs,
                                                          float* __restrict__ mlp_y,
                                                          int32_t* __restrict__ tfirst,
                                                          int32_t* __restrict__ tnpl) {
     using T = float;
-    __shared__ LearnedItem items[4][kSampleQueue];
-    __shared__ uint2 rows[4][kListQueue];
-    __shared__ float* recs[4][kListQueue];
+    __shared__ Sample32Item items[4][kSampleQueue];
     const int lane = threadIdx.x & 31;
-    LearnedItem* const Q = items[threadIdx.x >> 5];
-    uint2* const row_q = rows[threadIdx.x >> 5];
-    float** const rec_q = recs[threadIdx.x >> 5];
-    int qn = 0, rn = 0;   // items and rows waiting (warp-uniform)
-    auto flush = [&]() {
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(&ctr->mlp_rows, (unsigned long long)rn);
-        base = __shfl_sync(0xffffffffu, base, 0);
-        __syncwarp();
-        for (int i = lane; i < rn; i += 32) {
-            *reinterpret_cast<uint2*>(mlp_y + 8 * (base + i)) = row_q[i];
-            *reinterpret_cast<uint2*>(rec_q[i] + 14) = make_uint2((unsigned)(base + i), kSampleModel);
-        }
-        __syncwarp();
-        rn = 0;
-    };
+    Sample32Item* const Q = items[threadIdx.x >> 5];
+    int qn = 0;   // items waiting (warp-uniform)
+    const unsigned long long cap = sample_rows_cap(ctr, pool_chunks);
+    float* const row_base = sample_rows(pool, ctr, pool_chunks);
     // the queue's first n items, lane i taking item i
     auto evaluate = [&](int n) {
         unsigned what = kSampleEmpty;
-        uint2 row = make_uint2(0u, 0u);
+        uint2 in_row = make_uint2(0u, 0u);
         float* rec = nullptr;
         int32_t wray = -1, idx = -1;
+        T v[kPreVals];
         if (lane < n) {
-            const LearnedItem it = Q[lane];
+            const Sample32Item it = Q[lane];
             rec = it.rec;
             wray = it.wray;
             idx = it.idx;
             const ImageDesc& im = imgs[it.q];
-            float v[RecStride<float>::v];
-            load_record<float>(rec, v);
-            const T xs[3] = {v[0], v[1], v[2]};
+            float cur[RecStride<float>::v];
+            load_record<float>(rec, cur);
+            const T xs[3] = {cur[0], cur[1], cur[2]};
             KSGeom<T> G;
-            ks_geom_pinned(xs[0], xs[1], xs[2], ic<T>(im, kcSpin), ic<T>(im, kcMass), im.flat != 0, G);
+            ks_geom_pinned<kMlp>(xs[0], xs[1], xs[2], ic<T>(im, kcSpin), ic<T>(im, kcMass), im.flat != 0, G);
             Plasma<T> P;
-            if (plasma_at<T, kSlow>(im, xs, v[13], G, P, true)) {
+            if (plasma_at<T, kSlow, !kMlp>(im, xs, cur[13], G, P, true)) {
                 const RayHdr hd = hdr[wray];
-                const T kl[4] = {(T)hd.kt, v[3], v[4], v[5]};
+                const T kl[4] = {(T)hd.kt, cur[3], cur[4], cur[5]};
+                T ku[4];
+                raise4(G, kl, ku);
                 const T kdu = kl[0] * P.u[0] + kl[1] * P.u[1] + kl[2] * P.u[2] + kl[3] * P.u[3];
                 const T kdb = kl[0] * P.b[0] + kl[1] * P.b[1] + kl[2] * P.b[2] + kl[3] * P.b[3];
                 const T nu_fl = (T)(hd.nnorm * im.freq) * (-kdu);
                 T cth = fq(kdb, (-kdu) * fsqrt(P.bsq));
                 cth = cth > T(1) ? T(1) : (cth < T(-1) ? T(-1) : cth);
-                const mlp::ModelIn mi = mlp::model_inputs(P.th, P.bg, nu_fl, cth);
+                const T g = fq(ic<T>(im, kcFreq), nu_fl);
+                const T path = ic<T>(im, kcLen) * (-kdu);
+                const T eg = g * g * g * path;
                 what = kSampleExact;
-                if (mi.ok && P.ne > T(0)) {
-                    what = kSampleModel;
-                    row = mlp::input_row(mi.f);
-                } else {
-                    *reinterpret_cast<uint2*>(rec + 14) = make_uint2(0u, kSampleExact);
+                if constexpr (kMlp) {
+                    const mlp::ModelIn mi = mlp::model_inputs(P.th, P.bg, nu_fl, cth);
+                    if (mi.ok && P.ne > T(0)) {
+                        what = kSampleModel;
+                        in_row = mlp::input_row(mi.f);
+                        v[0] = P.ne; v[1] = P.th; v[2] = P.bg; v[3] = nu_fl;
+                        v[4] = cth; v[5] = eg; v[6] = path; v[7] = T(0);
+                    }
                 }
+                if (!kMlp || what == kSampleExact) {
+                    T co[8];
+                    synchrotron_coefficients<T>(P.ne, P.th, P.bg, nu_fl, cth, co);
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) v[c] = co[c] * (c < 3 ? eg : path);
+                }
+                fluid_basis<T>(G, P, kl, ku, v + 8, v + 12, v + 16, v + 20);
             }
         }
         const bool plasma = what != kSampleEmpty;
-        const unsigned model = __ballot_sync(0xffffffffu, what == kSampleModel);
-        if (what == kSampleModel) {
-            const int at = rn + __popc(model & ((1u << lane) - 1u));
-            row_q[at] = row;
-            rec_q[at] = rec;
+        const unsigned exact = __ballot_sync(0xffffffffu, what == kSampleExact);
+        const unsigned model = kMlp ? __ballot_sync(0xffffffffu, what == kSampleModel) : 0u;
+        unsigned long long eb = 0, mb = 0;
+        if (lane == 0) {
+            if (exact) eb = atomicAdd(&ctr->exact_rows, (unsigned long long)__popc(exact));
+            if (kMlp && model) mb = atomicAdd(&ctr->mlp_rows, (unsigned long long)__popc(model));
         }
-        rn += __popc(model);
+        eb = __shfl_sync(0xffffffffu, eb, 0);
+        if constexpr (kMlp) mb = __shfl_sync(0xffffffffu, mb, 0);
+        if (plasma) {
+            const unsigned below = (1u << lane) - 1u;
+            unsigned long long row = 0;
+            bool fits;
+            if (kMlp && what == kSampleModel) {
+                row = mb + __popc(model & below);
+                fits = row < cap;
+                *reinterpret_cast<uint2*>(mlp_y + 8 * row) = in_row;
+            } else {
+                const unsigned long long at = eb + __popc(exact & below);
+                fits = at < cap;
+                row = fits ? cap - 1 - at : 0;
+            }
+            *reinterpret_cast<uint2*>(rec + 14) = make_uint2((unsigned)row, what);
+            if (fits) {
+                float4* out = reinterpret_cast<float4*>(row_base + kPreVals * row);
+#pragma unroll
+                for (int i = 0; i < kPreVals / 4; ++i)
+                    out[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+            }
+        }
         // per ray of the batch: its plasma samples lie at increasing lanes (records enter the
         // queue in order), so the highest lane of a ray's group holds its farthest one
         const unsigned grp = __match_any_sync(0xffffffffu, plasma ? wray : -1 - lane);
@@ -2128,7 +2464,6 @@ __global__ void __launch_bounds__(128, 6) mlp_inputs_kernel(const ImageDesc* __r
             atomicMax(&tfirst[wray], idx);
             atomicAdd(&tnpl[wray], __popc(grp));
         }
-        if (rn >= kListFlush) flush();
     };
     const int64_t re = wave_end(bs, ray_end);
     const int64_t total_rays = re > ray_begin ? re - ray_begin : 0;
@@ -2186,12 +2521,12 @@ __global__ void __launch_bounds__(128, 6) mlp_inputs_kernel(const ImageDesc* __r
                 const float r2 = 0.5f * (qq + sqrtf(qq * qq + 4.0f * aa * v.z * v.z));
                 cand = r2 >= r2lo && r2 <= r2hi;
                 // a stencil without magnetic field holds no plasma (stencil_field_free);
-                // one snapshot only
-                if (!kSlow && cand) cand = !stencil_field_free(imgs[q], v.x, v.y, v.z, r2, aa);
+                // one snapshot only, or by the mask of all snapshots
+                if (cand && (!kSlow || imgs[q].mask)) cand = !stencil_field_free<true>(imgs[q], v.x, v.y, v.z, r2, aa);
             }
             const unsigned mask = __ballot_sync(0xffffffffu, cand);
             if (cand) {
-                LearnedItem& it = Q[qn + __popc(mask & ((1u << lane) - 1u))];
+                Sample32Item& it = Q[qn + __popc(mask & ((1u << lane) - 1u))];
                 it.rec = rec;
                 it.wray = (int32_t)wray;
                 it.idx = idx;
@@ -2205,7 +2540,7 @@ __global__ void __launch_bounds__(128, 6) mlp_inputs_kernel(const ImageDesc* __r
             const int n = qn < 32 ? qn : 32;
             evaluate(n);
             __syncwarp();
-            LearnedItem keep;
+            Sample32Item keep;
             const bool moves = lane < qn - n;
             if (moves) keep = Q[n + lane];
             __syncwarp();
@@ -2215,7 +2550,6 @@ __global__ void __launch_bounds__(128, 6) mlp_inputs_kernel(const ImageDesc* __r
         }
         if (exhausted && qn == 0) break;
     }
-    if (rn > 0) flush();
 }
 
 // ---------------------------------------------------------------------------------------

@@ -158,9 +158,12 @@ __device__ __forceinline__ void ks_geom(T x, T y, T z, T a, T m, bool flat, bool
     }
 }
 
-// ks_geom in FP32 without derivatives, its roundings written out, for the learned form's model
-// inputs: their bf16 rounding turns a last-bit difference of the geometry into one of 2^-9 in the
-// network, so the inputs are formed from the same bits whatever kernel the call is inlined into.
+// ks_geom in FP32 without derivatives, its roundings written out, for the FP32 sample pass: rays
+// that graze the horizon amplify a last-bit difference of a sample's plasma state a thousandfold, and
+// the bf16 rounding of the learned form's model inputs one to 2^-9, so both are formed from the same
+// bits whatever kernel the call is inlined into. The two forms round the numerator of l_y in
+// either order (kModel: the one of the model inputs).
+template <bool kModel>
 __device__ __forceinline__ void ks_geom_pinned(float x, float y, float z, float a, float m, bool flat,
                                                KSGeom<float>& G) {
     const float aa = __fmul_rn(a, a), aaz = __fmul_rn(aa, z);
@@ -177,7 +180,7 @@ __device__ __forceinline__ void ks_geom_pinned(float x, float y, float z, float 
     G.f = flat ? 0.0f : __fmul_rn(__fmul_rn(__fmul_rn(__fmul_rn(2.0f, m), r), r2), is4);
     G.l[0] = 1.0f;
     G.l[1] = __fmul_rn(__fmaf_rn(a, y, __fmul_rn(r, x)), iP);
-    G.l[2] = __fmul_rn(__fmaf_rn(r, y, -__fmul_rn(a, x)), iP);
+    G.l[2] = __fmul_rn(kModel ? __fmaf_rn(r, y, -__fmul_rn(a, x)) : __fmaf_rn(-a, x, __fmul_rn(r, y)), iP);
     G.l[3] = __fmul_rn(z, ir);
 }
 
