@@ -85,14 +85,6 @@ PredOff pred_offsets(size_t base, int32_t n_images, int64_t nb) {
     return o;
 }
 
-// The FP64 transfer runs as two passes (fp64_samples_kernel, then the transport and Stokes
-// steps) when set; 0 keeps the single fused kernel.
-#ifndef BL_TR64_SPLIT
-#define BL_TR64_SPLIT 1
-#endif
-constexpr bool kFp64Split = BL_TR64_SPLIT != 0;
-
-
 // mlp: room for the learned model's outputs, 8 floats for every record of the pool
 Layout make_layout_wave(int32_t n_images, int64_t rays, int64_t wave, int precision,
                         bool transfer, int64_t cpr = kChunksPerRay, bool mlp = false,
@@ -116,7 +108,7 @@ Layout make_layout_wave(int32_t n_images, int64_t rays, int64_t wave, int precis
     // FP64 form: the sample pass's coefficients and basis, and a flag byte, a pool record
     L.pre = off;
     L.pre_flag = off;
-    if (precision == BL_PREC_FP64 && transfer && kFp64Split) {
+    if (precision == BL_PREC_FP64 && transfer) {
         off = align_up(off + bl::kPreVals * sizeof(double) * bl::kChunk * (size_t)L.pool_chunks);
         L.pre_flag = off;
         off = align_up(off + bl::kChunk * (size_t)L.pool_chunks);
@@ -416,43 +408,41 @@ struct DevInfo {
     int tr_occ[2][8] = {};          // transfer variants: [double, float][feature bits]
     int tr_mlp_occ[2] = {0, 0};     // learned-coefficient transfer: [fast light, slow light]
     int s32_occ[4] = {0, 0, 0, 0};  // FP32 sample pass: [slow light + 2 learned]
-    int pre_occ[2] = {0, 0};        // FP64 sample pass: [fast, slow light]
-    int tr_pre_occ[2] = {0, 0};     // FP64 transfer after the sample pass: [fast, slow light]
+    int pre_occ[8] = {};            // FP64 sample pass: [feature bits]
+    int tr_pre_occ = 0;             // FP64 transport pass
+    int un64_occ[2] = {0, 0};       // FP64 second pass of unpolarized images: [plain, auxiliary images]
     int fwd_list_occ = 0;           // the model over the work list
     int rk_occ[2] = {0, 0};         // RK2/RK4 geodesic kernel: [double records, float records]
     // CTAs per SM of the transfer variant a launch uses
     int transfer(int precision, const float* mlp, int feat) const {
         if (mlp) return tr_mlp_occ[(feat & bl::kFSlow) ? 1 : 0];
-        if (precision == BL_PREC_FP64 && kFp64Split && !(feat & (bl::kFUnpol | bl::kFAux)))
-            return tr_pre_occ[(feat & bl::kFSlow) ? 1 : 0];
+        if (precision == BL_PREC_FP64 && (feat & bl::kFUnpol)) return un64_occ[(feat & bl::kFAux) ? 1 : 0];
+        if (precision == BL_PREC_FP64 && !(feat & bl::kFAux)) return tr_pre_occ;
         return tr_occ[precision == BL_PREC_FP64 ? 0 : 1][feat & 7];
     }
 };
 
-template <class T, class R, int F>
-int occ_transfer(int* out) {
-    if constexpr (std::is_same<T, double>::value) {
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bl::transfer_kernel_fp64<F>,
-                                                              bl::kTransferFp64Threads, 0));
-    } else {
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(out, bl::transfer_kernel<T, R, F>, 128, 0));
-    }
-    if (*out < 1) *out = 1;
-    return 0;
+template <int F>
+int occ_transfer32(int out[8]) {
+    BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&out[F], bl::transfer_kernel<float, float, F>, 128, 0));
+    if (out[F] < 1) out[F] = 1;
+    if constexpr (F < 7) return occ_transfer32<F + 1>(out);
+    else return 0;
 }
 
-template <class T, class R>
-int occ_transfer_all(int out[8]) {
-    int rc = 0;
-    if (!rc) rc = occ_transfer<T, R, 0>(&out[0]);
-    if (!rc) rc = occ_transfer<T, R, 1>(&out[1]);
-    if (!rc) rc = occ_transfer<T, R, 2>(&out[2]);
-    if (!rc) rc = occ_transfer<T, R, 3>(&out[3]);
-    if (!rc) rc = occ_transfer<T, R, 4>(&out[4]);
-    if (!rc) rc = occ_transfer<T, R, 5>(&out[5]);
-    if (!rc) rc = occ_transfer<T, R, 6>(&out[6]);
-    if (!rc) rc = occ_transfer<T, R, 7>(&out[7]);
-    return rc;
+// FP64: the sample pass (all but polarized auxiliary images) or the single kernel (those)
+template <int F>
+int occ_fp64(int pre[8], int tr[8]) {
+    if constexpr ((F & bl::kFAux) != 0 && (F & bl::kFUnpol) == 0) {
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&tr[F], bl::transfer_kernel_fp64<F>,
+                                                              bl::kTransferFp64Threads, 0));
+        if (tr[F] < 1) tr[F] = 1;
+    } else {
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pre[F], bl::fp64_samples_kernel<F>, 128, 0));
+        if (pre[F] < 1) pre[F] = 1;
+    }
+    if constexpr (F < 7) return occ_fp64<F + 1>(pre, tr);
+    else return 0;
 }
 
 int dev_info(DevInfo& out) {
@@ -479,8 +469,8 @@ int dev_info(DevInfo& out) {
         if (di.geo64_wide < 1) di.geo64_wide = 1;
         for (int i = 0; i < 3; ++i)
             if (di.geo_blocks[i] < 1) di.geo_blocks[i] = 1;
-        int rc = occ_transfer_all<double, double>(di.tr_occ[0]);
-        if (!rc) rc = occ_transfer_all<float, float>(di.tr_occ[1]);
+        int rc = occ_fp64<0>(di.pre_occ, di.tr_occ[0]);
+        if (!rc) rc = occ_transfer32<0>(di.tr_occ[1]);
         if (rc) { di.sms = 0; return rc; }
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.tr_mlp_occ[0], bl::transfer_learned_kernel<false>, 128, 0));
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.tr_mlp_occ[1], bl::transfer_learned_kernel<true>, 128, 0));
@@ -491,14 +481,12 @@ int dev_info(DevInfo& out) {
         for (int i = 0; i < 4; ++i)
             if (di.s32_occ[i] < 1) di.s32_occ[i] = 1;
         BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.fwd_list_occ, bl::mlp::forward_list_kernel, 128, 0));
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.pre_occ[0], bl::fp64_samples_kernel<false>, 128, 0));
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.pre_occ[1], bl::fp64_samples_kernel<true>, 128, 0));
-        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.tr_pre_occ[0], bl::transport_fp64_kernel, bl::kTransferFp64Threads, 0));
-        di.tr_pre_occ[1] = di.tr_pre_occ[0];
-        for (int i = 0; i < 2; ++i) {
-            if (di.pre_occ[i] < 1) di.pre_occ[i] = 1;
-            if (di.tr_pre_occ[i] < 1) di.tr_pre_occ[i] = 1;
-        }
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.tr_pre_occ, bl::transport_fp64_kernel, bl::kTransferFp64Threads, 0));
+        if (di.tr_pre_occ < 1) di.tr_pre_occ = 1;
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.un64_occ[0], bl::unpolarized64_kernel<false>, 128, 0));
+        BL_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&di.un64_occ[1], bl::unpolarized64_kernel<true>, 128, 0));
+        for (int i = 0; i < 2; ++i)
+            if (di.un64_occ[i] < 1) di.un64_occ[i] = 1;
         if (di.fwd_list_occ < 1) di.fwd_list_occ = 1;
         for (int i = 0; i < 2; ++i)
             if (di.tr_mlp_occ[i] < 1) di.tr_mlp_occ[i] = 1;
@@ -520,16 +508,8 @@ void launch_transfer(int feat, unsigned grid, cudaStream_t st, const bl::ImageDe
                      bl::SideIn side = bl::SideIn{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr}) {
     if constexpr (std::is_same<T, double>::value) {
         constexpr int th = bl::kTransferFp64Threads;
-        switch (feat & 7) {
-            case 0: bl::transfer_kernel_fp64<0><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side); break;
-            case 1: bl::transfer_kernel_fp64<1><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side); break;
-            case 2: bl::transfer_kernel_fp64<2><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side); break;
-            case 3: bl::transfer_kernel_fp64<3><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side); break;
-            case 4: bl::transfer_kernel_fp64<4><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side); break;
-            case 5: bl::transfer_kernel_fp64<5><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side); break;
-            case 6: bl::transfer_kernel_fp64<6><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side); break;
-            default: bl::transfer_kernel_fp64<7><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side); break;
-        }
+        if (feat & bl::kFSlow) bl::transfer_kernel_fp64<5><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side);
+        else bl::transfer_kernel_fp64<4><<<grid, th, 0, st>>>(d, n, b, e, hdr, pool, chunks, ctr, bs, side);
     } else {
         if (feat & bl::kFMlp) {
             if constexpr (std::is_same<R, float>::value) {
@@ -772,7 +752,7 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                                               fpool, chunks, ctr, cfg.bs,
                                               bl::SideIn{nullptr, nullptr, nullptr, nullptr, nullptr,
                                                          cfg.order_transfer ? tperm : nullptr});
-            } else if (kFp64Split && !(cfg.feat & (bl::kFUnpol | bl::kFAux))) {
+            } else if ((cfg.feat & bl::kFUnpol) || !(cfg.feat & bl::kFAux)) {
                 // FP64 in two passes: the sample pass, then transport and Stokes steps
                 // then the transport pass takes the wave's rays longest first (a counting sort
                 // of the sample pass's work estimates)
@@ -783,19 +763,27 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                 // per wave ray: farthest plasma sample -1 and no plasma samples until found
                 BL_CUDA(cudaMemsetAsync(tfirst, 0xff, sizeof(int32_t) * (size_t)(e - b), st));
                 BL_CUDA(cudaMemsetAsync(tnpl, 0, sizeof(int32_t) * (size_t)(e - b), st));
-                const unsigned pre_grid = (unsigned)(di.sms * di.pre_occ[slow ? 1 : 0]);
-                if (slow)
-                    bl::fp64_samples_kernel<true><<<pre_grid, 128, 0, st>>>(
-                        d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs, pre, pflag,
-                        tfirst, tnpl);
-                else
-                    bl::fp64_samples_kernel<false><<<pre_grid, 128, 0, st>>>(
-                        d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs, pre, pflag,
-                        tfirst, tnpl);
+                const unsigned pre_grid = (unsigned)(di.sms * di.pre_occ[cfg.feat & 7]);
+                auto samples = bl::fp64_samples_kernel<0>;
+                switch (cfg.feat & 7) {
+                    case 0: break;
+                    case 1: samples = bl::fp64_samples_kernel<1>; break;
+                    case 2: samples = bl::fp64_samples_kernel<2>; break;
+                    case 3: samples = bl::fp64_samples_kernel<3>; break;
+                    case 6: samples = bl::fp64_samples_kernel<6>; break;
+                    default: samples = bl::fp64_samples_kernel<7>; break;
+                }
+                samples<<<pre_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs,
+                                                  pre, pflag, tfirst, tnpl);
                 ++g_launches;
                 BL_CUDA(cudaGetLastError());
                 if ((rc = order_by_plasma())) return rc;
-                if (!tr_set && e - b <= bl::kDeep64Rays * di.sms)
+                if (cfg.feat & bl::kFUnpol) {
+                    auto second = (cfg.feat & bl::kFAux) ? bl::unpolarized64_kernel<true>
+                                                         : bl::unpolarized64_kernel<false>;
+                    second<<<tr_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs,
+                                                    bl::SideIn{nullptr, nullptr, pre, pflag, tfirst, tperm});
+                } else if (!tr_set && e - b <= bl::kDeep64Rays * di.sms)
                     bl::transport64_wide_kernel<<<(unsigned)(di.sms * bl::kTransport64WideCtas), 128, 0, st>>>(
                         d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs,
                         bl::SideIn{nullptr, nullptr, pre, pflag, tfirst}, tperm, di.sms);
