@@ -2262,7 +2262,10 @@ __device__ __forceinline__ void transport_fp64_body(
             if (hd.status == BL_RAY_OVERFLOW || hd.nrec == 0) {
                 const int64_t npix = im.n_rays;
                 const double val = hd.status == BL_RAY_OVERFLOW ? nan("") : 0.0;
-                for (int s = 0; s < 4; ++s) ((double*)im.stokes)[s * npix + opix] = val;
+                for (int s = 0; s < 4; ++s) {
+                    if (im.dtype == 0) ((double*)im.stokes)[s * npix + opix] = val;
+                    else ((float*)im.stokes)[s * npix + opix] = (float)val;
+                }
                 continue;
             }
             // from the farthest plasma sample where the sample pass found it (the records
@@ -2309,7 +2312,10 @@ __device__ __forceinline__ void transport_fp64_body(
                 T sv[4];
                 coh_to_stokes(N, hl, vl, sv);
                 const int64_t npix = im.n_rays;
-                for (int c = 0; c < 4; ++c) ((double*)im.stokes)[c * npix + opix] = sv[c];
+                for (int c = 0; c < 4; ++c) {
+                    if (im.dtype == 0) ((double*)im.stokes)[c * npix + opix] = sv[c];
+                    else ((float*)im.stokes)[c * npix + opix] = (float)sv[c];
+                }
                 active = false;
                 continue;
             }

@@ -13,7 +13,8 @@ from paper_2203_15963_gb300 import synth as S
 pytestmark = pytest.mark.gpu
 
 
-def _trace(n, precision, aux, snaps=1, layout="planes", workspace=None, dtype=None):
+def _trace(n, precision, aux, snaps=1, layout="planes", workspace=None, dtype=None,
+           flags=native.BL_UNPOLARIZED):
     gp = S.grid_params_for(48, 32, 32)
     prim = torch.from_numpy(S.make_torus(gp, 0.9, S.BASE_SEED)).cuda()
     if snaps > 1:
@@ -26,7 +27,7 @@ def _trace(n, precision, aux, snaps=1, layout="planes", workspace=None, dtype=No
     out = images.alloc_outputs(n, dtype, aux=aux)
     images.trace_images([S.Camera(theta=math.radians(60.0), n=n)],
                         [S.Metric(spin=0.9, precision=precision)], [gp], [prim], [230e9], outs=[out],
-                        workspace=workspace, flags=native.BL_UNPOLARIZED)
+                        workspace=workspace, flags=flags)
     torch.cuda.synchronize()
     return torch.cat([out["stokes"].double()] + ([out["aux"].double()] if aux else []))
 
@@ -51,3 +52,11 @@ def test_against_mixed_and_in_waves(n, aux, snaps, layout):
     assert torch.equal(_trace(n, native.BL_PREC_FP64, aux, snaps, layout, small), ref)
     assert torch.equal(_trace(n, native.BL_PREC_FP64, aux, snaps, layout, dtype=torch.float32)[:4],
                        ref[:4].float().double())
+
+
+@pytest.mark.parametrize("n", [1, 33])
+def test_polarized_float32_output(n):
+    """FP64 polarized images write the output's own type: rounded, and no plane beyond it."""
+    ref = _trace(n, native.BL_PREC_FP64, False, flags=0)
+    assert torch.equal(_trace(n, native.BL_PREC_FP64, False, dtype=torch.float32, flags=0),
+                       ref.float().double())
