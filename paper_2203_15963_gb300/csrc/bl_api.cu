@@ -782,7 +782,8 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                     auto second = (cfg.feat & bl::kFAux) ? bl::unpolarized64_kernel<true>
                                                          : bl::unpolarized64_kernel<false>;
                     second<<<tr_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs,
-                                                    bl::SideIn{nullptr, nullptr, pre, pflag, tfirst, tperm});
+                                                    bl::SideIn{nullptr, nullptr, pre, pflag, tfirst, tperm},
+                                                    tr_set ? 0 : di.sms);
                 } else if (!tr_set && e - b <= bl::kDeep64Rays * di.sms)
                     bl::transport64_wide_kernel<<<(unsigned)(di.sms * bl::kTransport64WideCtas), 128, 0, st>>>(
                         d_desc, n_images, b, e, hdr, dpool, chunks, ctr, cfg.bs,

@@ -617,7 +617,7 @@ __global__ void __launch_bounds__(128, 3) geodesic_rk_kernel(const ImageDesc* __
                                                              RayHdr* __restrict__ hdr,
                                                              RecordSink<R> sink, int record,
                                                              BlockSource bs, int sms) {
-    if (sms > 0 && (int)blockIdx.x >= sms && sparse_wave(bs, ray_begin, ray_end, sms)) return;
+    if (sms > 0 && spare_cta(bs, ray_begin, ray_end, sms)) return;
     const int64_t re = wave_end(bs, ray_end);
     const int64_t total_rays = re > ray_begin ? re - ray_begin : 0;
     Counters* ctr = sink.ctr;

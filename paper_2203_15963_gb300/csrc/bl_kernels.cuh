@@ -711,13 +711,15 @@ __device__ __forceinline__ bool finite_bits(double x) {
     return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
 }
 
-// Rays an SM up to which an FP64-arithmetic launch runs one CTA an SM, and above which it runs
-// the 64-warp shapes (figures at the kernels).
-constexpr int64_t kSparse64Rays = 4 * 128, kDeep64Rays = 20 * 128;   // rays an SM
-// Few enough rays in this wave for one CTA an SM.
-__device__ __forceinline__ bool sparse_wave(const BlockSource& bs, int64_t ray_begin,
-                                            int64_t ray_end, int sms) {
-    return wave_end(bs, ray_end) - ray_begin <= kSparse64Rays * sms;
+// Rays an SM up to which an FP64-arithmetic launch runs one CTA an SM, two, and above which it
+// runs the 64-warp shapes (figures at the kernels).
+constexpr int64_t kSparse64Rays = 4 * 128, kTwo64Rays = 8 * 128, kDeep64Rays = 20 * 128;
+// A CTA this wave has too few rays for: all but the first of an SM, or all but two.
+__device__ __forceinline__ bool spare_cta(const BlockSource& bs, int64_t ray_begin, int64_t ray_end,
+                                          int sms) {
+    if ((int)blockIdx.x < sms) return false;
+    const int64_t n = wave_end(bs, ray_end) - ray_begin;
+    return n <= kSparse64Rays * sms || (n <= kTwo64Rays * sms && (int)blockIdx.x >= 2 * sms);
 }
 
 }  // namespace bl
@@ -744,9 +746,11 @@ __global__ void __launch_bounds__(128, BL_GEO_MIN_CTAS) geodesic_df_kernel(
 // further warp slows the ones there: a launch of few rays ends with its longest rays, which then
 // run at the pace of the crowd. So up to kSparse64Rays rays an SM a single CTA an SM works
 // through the queue (FP64, one 256^2 image: 22.2 ms against 28.5 at 3 CTAs and 33.9 at 16; mixed
-// 17.9 against 27.7; three images, 1293 rays an SM: 61 against 52, so the line lies between). The
-// CTAs beyond the first of an SM decide that for themselves, as a device block list's length is
-// not known to the host.
+// 17.9 against 27.7), and up to kTwo64Rays two (mixed, two 201^2 images, 531 rays an SM: 22.7 ms
+// against 23.6 with one and 26.8 with three; two 256^2, 862: 27.2 / 33.3 / 32.0, FP64 35.5 / 41.7 /
+// 38.9; from 1192 to 2400 rays an SM two and three are within 4 % of each other either way). The
+// CTAs beyond those of an SM decide that for themselves, as a device block list's length is not
+// known to the host.
 #ifndef BL_GEO64_MIN_CTAS
 #define BL_GEO64_MIN_CTAS 16
 #endif
@@ -763,7 +767,7 @@ template <class R>
 __global__ void __launch_bounds__(128, BL_GEO64_WIDE_CTAS) geodesic64_kernel(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         RayHdr* __restrict__ hdr, RecordSink<R> sink, int record, BlockSource bs, int sms) {
-    if (sms > 0 && (int)blockIdx.x >= sms && sparse_wave(bs, ray_begin, ray_end, sms)) return;
+    if (sms > 0 && spare_cta(bs, ray_begin, ray_end, sms)) return;
     geodesic64_body<R, true>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs);
 }
 
@@ -2341,9 +2345,9 @@ __device__ __forceinline__ void transport_fp64_body(
 
 // Two shapes, as for the FP64 geodesics: 32 registers and the SM's 64 warps for dense waves, 3
 // CTAs of 128 threads an SM without spills up to kDeep64Rays rays an SM (three 256^2 images,
-// both transfer passes: 34.3 ms against 48.9), of which all but the first of an SM leave when the
-// wave is sparse (one 256^2 image: 14.3 ms against 22.0 with all and 24.0 in the dense shape; a
-// 32^2 image 5.4 against 7.0). Nine images: 105 ms dense, 109 in the other shape.
+// both transfer passes: 34.3 ms against 48.9), of which all but the first one or two of an SM leave
+// when the wave has few rays (one 256^2 image: 14.3 ms against 22.0 with all and 24.0 in the dense
+// shape; a 32^2 image 5.4 against 7.0; two 201^2 images 16.4 with two, 17.3 with one, 19.9). Nine images: 105 ms dense, 109 in the other shape.
 __global__ void __maxnreg__(BL_TRANSPORT64_MAXNREG) transport_fp64_kernel(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         const RayHdr* __restrict__ hdr, const double* __restrict__ pool,
@@ -2357,7 +2361,7 @@ __global__ void __launch_bounds__(128, kTransport64WideCtas) transport64_wide_ke
         const RayHdr* __restrict__ hdr, const double* __restrict__ pool,
         const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side,
         const int32_t* __restrict__ perm, int sms) {
-    if ((int)blockIdx.x >= sms && sparse_wave(bs, ray_begin, ray_end, sms)) return;
+    if (spare_cta(bs, ray_begin, ray_end, sms)) return;
     transport_fp64_body(imgs, n_images, ray_begin, ray_end, hdr, pool, chunks, ctr, bs, side, perm);
 }
 
@@ -2370,8 +2374,9 @@ template <bool kAux>
 __global__ void __launch_bounds__(128, 4) unpolarized64_kernel(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         const RayHdr* __restrict__ hdr, const double* __restrict__ pool,
-        const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side) {
+        const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side, int sms) {
     using T = double;
+    if (sms > 0 && spare_cta(bs, ray_begin, ray_end, sms)) return;
     const int64_t re = wave_end(bs, ray_end);
     const int64_t n_rays = re > ray_begin ? re - ray_begin : 0;
     const int64_t total_rays = ordered_total<kTransportGroup>(n_rays);

@@ -50,6 +50,22 @@ def test_launch_shapes_give_the_same_bits(torus, n, spin, inc, precision):
         assert torch.equal(a[k], b[k]), k
 
 
+@pytest.mark.parametrize("precision", [native.BL_PREC_FP64, native.BL_PREC_MIXED])
+def test_two_ctas_an_sm_give_the_same_bits(torus, precision):
+    """592 rays an SM: between the waves that one CTA an SM serves and those that all do."""
+    gp, prims = torus
+    cam, met = _image(300, 0.97, 60.0, precision)
+    a, b = _outs(300, precision), _outs(300, precision)
+    images.trace_images([cam], [met], [gp], [prims[0.97]], [FREQ], outs=[a])
+    plan = native.Plan([cam], [met], [gp], [prims[0.97]], [FREQ], [b],
+                       config={"geo_ctas_per_sm": 1, "tr_ctas_per_sm": 1})
+    plan.run()
+    plan.check()
+    plan.close()
+    for k in a:
+        assert torch.equal(a[k], b[k]), k
+
+
 @pytest.mark.parametrize("spin,inc,ds_max,r_in", [
     (0.97, 5.0, 0.5, 1.01), (0.97, 88.0, 0.5, 1.0001), (0.0, 45.0, 0.3, 1.01),
     (0.97, 60.0, 2.0, 1.3), (0.97, 60.0, 40.0, 1.01)])
