@@ -206,7 +206,7 @@ template <class R, bool kKsmem>
 __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ imgs, int n_images,
                                                 int64_t ray_begin, int64_t ray_end,
                                                 RayHdr* __restrict__ hdr, RecordSink<R> sink,
-                                                int record, BlockSource bs) {
+                                                int record, BlockSource bs, int lanes = 32) {
     // rays [ray_begin, ray_end) of the batch form this wave; hdr and the chunk tables are
     // indexed by ray - ray_begin
     const int64_t re = wave_end(bs, ray_end);
@@ -216,7 +216,7 @@ __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ im
     // integration and its step decisions untouched. FP64 records: all in double.
     constexpr bool kFRec = sizeof(R) == sizeof(float);
     Counters* ctr = sink.ctr;
-    bool active = false, exhausted = false;
+    bool active = false, exhausted = (int)(threadIdx.x & 31) >= lanes;   // lanes that take no rays
     int64_t wray = 0, opix = 0;
     int q = 0, pi = 0, pj = 0;
     double y[8];

@@ -721,6 +721,16 @@ __device__ __forceinline__ bool spare_cta(const BlockSource& bs, int64_t ray_beg
     const int64_t n = wave_end(bs, ray_end) - ray_begin;
     return n <= kSparse64Rays * sms || (n <= kTwo64Rays * sms && (int)blockIdx.x >= 2 * sms);
 }
+// Lanes of a warp that take rays: fewer rays than the lanes of `ctas` CTAs are spread over all their
+// warps, because a warp pays for every path any of its lanes is on (the sub-samples of a step,
+// Stokes steps) and an idle scheduler for none (a 32^2 image, geodesics and transport: 20.0 -> 17.1
+// ms; 64^2 with adaptive levels 111.1 -> 110.4).
+__device__ __forceinline__ int wave_lanes(const BlockSource& bs, int64_t ray_begin, int64_t ray_end,
+                                          int ctas) {
+    const int64_t n = wave_end(bs, ray_end) - ray_begin, warps = 4 * (int64_t)ctas;
+    const int64_t lanes = (n + warps - 1) / warps;
+    return lanes < 1 ? 1 : lanes > 32 ? 32 : (int)lanes;
+}
 
 }  // namespace bl
 #include "bl_geo64.cuh"
@@ -768,7 +778,8 @@ __global__ void __launch_bounds__(128, BL_GEO64_WIDE_CTAS) geodesic64_kernel(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         RayHdr* __restrict__ hdr, RecordSink<R> sink, int record, BlockSource bs, int sms) {
     if (sms > 0 && spare_cta(bs, ray_begin, ray_end, sms)) return;
-    geodesic64_body<R, true>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs);
+    geodesic64_body<R, true>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs,
+                             wave_lanes(bs, ray_begin, ray_end, sms > 0 ? sms : (int)gridDim.x));
 }
 
 // Per-image constant in the transfer arithmetic.
@@ -2232,7 +2243,7 @@ __device__ __forceinline__ void transport_fp64_body(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         const RayHdr* __restrict__ hdr, const double* __restrict__ pool,
         const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side,
-        const int32_t* __restrict__ perm) {
+        const int32_t* __restrict__ perm, int lanes = 32) {
     using T = double;
     const int64_t re = wave_end(bs, ray_end);
     const int64_t n_rays = re > ray_begin ? re - ray_begin : 0;
@@ -2244,7 +2255,7 @@ __device__ __forceinline__ void transport_fp64_body(
     Coh<T> N;
     T kt = T(0), a = T(0), m = T(0);
     bool flat = false;
-    bool exhausted = false;
+    bool exhausted = (int)(threadIdx.x & 31) >= lanes;   // lanes that take no rays
     while (true) {
         const bool need = !active && !exhausted;
         const unsigned long long got = warp_refill(&ctr->next_ray_tr, need);
@@ -2362,7 +2373,8 @@ __global__ void __launch_bounds__(128, kTransport64WideCtas) transport64_wide_ke
         const int32_t* __restrict__ chunks, Counters* ctr, BlockSource bs, SideIn side,
         const int32_t* __restrict__ perm, int sms) {
     if (spare_cta(bs, ray_begin, ray_end, sms)) return;
-    transport_fp64_body(imgs, n_images, ray_begin, ray_end, hdr, pool, chunks, ctr, bs, side, perm);
+    transport_fp64_body(imgs, n_images, ray_begin, ray_end, hdr, pool, chunks, ctr, bs, side, perm,
+                        wave_lanes(bs, ray_begin, ray_end, sms));
 }
 
 // FP64 form, second pass of unpolarized images: along each ray from its farthest plasma sample the
