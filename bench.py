@@ -66,13 +66,11 @@ FLOP64_PER_ATTEMPT = 1214
 # least 108 a record.
 FLOP64_EMIT_PER_RECORD = 108
 # Arithmetic per transfer sample of the method (see the module docstring): FP32 flops and
-# special-function instructions of transfer_kernel<float, float, 0> per sample with the
+# special-function instructions of the single-kernel FP32 transfer per sample with the
 # stencil field test on (a sample whose lookup stencil carries no magnetic field stops after
 # the lookup), from the ncu capture of the one-image 256^2 case on plane-layout grids (a =
 # 0.94, i = 60 deg; 18,372,183 samples): 2 x 4.397e9 FFMA + 2.661e9 FMUL + 0.703e9 FADD
-# thread instructions, 2.43e8 MUFU. (Without the test, as the cell-layout FP32 transfer runs
-# for its record-count queue, the kernel executes 848 flops a sample: the difference is work
-# the method does not need.)
+# thread instructions, 2.43e8 MUFU.
 FLOP_PER_SAMPLE = 662
 SFU_PER_SAMPLE = 13.2
 # The CUDA kernel headers (their code hash is printed with the results), and the ones the
@@ -80,28 +78,29 @@ SFU_PER_SAMPLE = 13.2
 # instantiate nothing of the learned model's headers (bl_mlp.cuh, bl_tc.cuh), so a change
 # there leaves their captured figures valid.
 KERNEL_HEADERS = ("bl_kernels.cuh", "bl_math.cuh", "bl_df64.cuh", "bl_internal.cuh",
-                  "bl_mlp.cuh", "bl_tc.cuh")
-TRAFFIC_HEADERS = ("bl_kernels.cuh", "bl_math.cuh", "bl_df64.cuh", "bl_internal.cuh")
+                  "bl_geo64.cuh", "bl_geodf.cuh", "bl_mlp.cuh", "bl_tc.cuh")
+TRAFFIC_HEADERS = ("bl_kernels.cuh", "bl_math.cuh", "bl_df64.cuh", "bl_internal.cuh",
+                   "bl_geo64.cuh", "bl_geodf.cuh")
 # dram__bytes_read.sum + dram__bytes_write.sum per unit of work from one ncu capture of the
 # one-image 256^2 case, with the kernel-source hash of that capture; scaled by the units of a
 # launch of the benchmark step (the kernels' traffic grows with the units they process).
 # fp64_instr: thread-level DFMA + DMUL + DADD instructions per unit from the same capture,
 # which gives the FP64 pipe's issue rate beside the algorithmic roofline.
 DRAM_PER_UNIT = {
-    # FP64 form, 7,845,751 attempts: 0.677 GB read + 5.398 GB written (the FP64 records and the
-    # stage derivatives, held in local memory at 16 CTAs an SM)
-    "geodesic_fp64": {"src": "c20dc1578110e077", "bytes": 774.3, "unit": "attempt",
-                      "fp64_instr": 1091.2},
-    # FP64 form, 18,372,204 samples, the transfer's launches: fp64_samples_kernel 4.190 + 3.815
+    # FP64 form, 7,845,751 attempts, the kernel of large waves at 15 CTAs an SM: 0.793 GB read +
+    # 5.434 GB written (the FP64 records and the stage derivatives, held in local memory)
+    "geodesic_fp64": {"src": "ad6fe3ed8e2f591c", "bytes": 793.7, "unit": "attempt",
+                      "fp64_instr": 975.4},
+    # FP64 form, 18,372,204 samples, the transfer's launches: fp64_samples_kernel 4.179 + 3.872
     # GB (records, the stencils' field values, grid gathers, 193 B of results a plasma sample,
-    # spills) and transport_fp64_kernel 1.501 + 2.439 GB (records, those results, spills)
-    "transfer_fp64": {"src": "c20dc1578110e077", "bytes": 650.2, "unit": "sample",
-                      "fp64_instr": 405.4},
-    # fast form, 7,845,744 attempts: 0.026 GB read + 1.135 GB written
-    "geodesic_df64": {"src": "c20dc1578110e077", "bytes": 147.9, "unit": "attempt"},
-    # fast form on cell-layout grids (record-count queue, no field test), 18,372,183 samples:
-    # 1.434 GB read + 0.006 GB written
-    "transfer_fp32": {"src": "c20dc1578110e077", "bytes": 78.4, "unit": "sample"},
+    # spills) and transport_fp64_kernel 1.258 + 0.660 GB (records, those results, spills)
+    "transfer_fp64": {"src": "ad6fe3ed8e2f591c", "bytes": 542.6, "unit": "sample",
+                      "fp64_instr": 284.5},
+    # fast form, 7,845,744 attempts: 0.023 GB read + 1.134 GB written
+    "geodesic_df64": {"src": "ad6fe3ed8e2f591c", "bytes": 147.5, "unit": "attempt"},
+    # fast form on cell-layout grids, 18,372,183 samples: field mask 0.167 + 0.003 GB, samples
+    # 1.309 + 0.318, transport 0.640 + 0.003
+    "transfer_fp32": {"src": "ad6fe3ed8e2f591c", "bytes": 132.9, "unit": "sample"},
 }
 
 
@@ -386,13 +385,14 @@ def form_rooflines(prec_name, attempts, samples, geo_s, tr_s, peaks):
                     f"least {FLOP64_EMIT_PER_RECORD} a sample record of the FP64 sample emission "
                     f"({samples} records for {attempts} attempts)")
     geo = roofline({"fp64": "geodesic_kernel_fp64",
-                    "mixed": "geodesic_kernel<float, double>",
-                    "fast": "geodesic_kernel<float, df64>"}[prec_name],
+                    "mixed": "geodesic64_kernel<float>",
+                    "fast": "geodesic_df_kernel"}[prec_name],
                    geo_flops, attempts, "DP attempt", geo_s, pk(geo_kind),
                    traffic_key={"fp64": "geodesic_fp64", "fast": "geodesic_df64"}.get(prec_name),
                    note=geo_note)
     tr = roofline("transfer phase: fp64_samples_kernel + transport_fp64_kernel"
-                  if prec_name == "fp64" else "transfer_kernel<float, float, 0>",
+                  if prec_name == "fp64"
+                  else "transfer phase: field_mask + fp32_samples_kernel + transfer_kernel",
                   FLOP_PER_SAMPLE, samples, "transfer sample", tr_s, pk(tr_kind),
                   traffic_key="transfer_fp64" if prec_name == "fp64" else "transfer_fp32",
                   note=("algorithmic flops: the method's per-sample arithmetic as the FP32 "
