@@ -112,15 +112,16 @@ struct BlockSource {
 };
 
 // Side inputs of the transfer variants that split their per-sample work over passes: the
-// learned model's outputs (8 floats a row of its work list) and its parameters, or, in the FP64 form,
+// learned model's outputs (8 floats a row of its work list) and its parameters; in the FP64 form
 // each record's precomputed scaled coefficients and fluid-frame basis (24 doubles a pool
-// record) with a flag byte (1: the sample carries plasma).
+// record) with a flag byte (1: the sample carries plasma); in the FP32 forms the pool whose unused
+// part holds the plasma samples' rows.
 struct SideIn {
     const float* mlp_y;
     const float* mlp_params;
     const double* pre;
     const unsigned char* pre_flag;
-    const int32_t* first;    // each ray's farthest plasma sample, or -1 (learned and FP64 forms)
+    const int32_t* first;    // each ray's farthest plasma sample, or -1 (after a sample pass)
     const int32_t* perm;     // the transfer's ray order (wave ray indices), or nullptr
     unsigned long long pool_chunks = 0;   // after the FP32 sample pass: the record pool's chunks
 };

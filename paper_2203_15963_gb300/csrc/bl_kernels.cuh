@@ -772,7 +772,7 @@ __global__ void __launch_bounds__(128, BL_GEO64_MIN_CTAS) geodesic_kernel_fp64(
         RayHdr* __restrict__ hdr, RecordSink<double> sink, int record, BlockSource bs) {
     geodesic64_body<double, false>(imgs, n_images, ray_begin, ray_end, hdr, sink, record, bs);
 }
-// sms > 0: CTAs from number `sms` on leave at once when the wave is sparse.
+// sms > 0: CTAs that the wave has too few rays for leave at once.
 template <class R>
 __global__ void __launch_bounds__(128, BL_GEO64_WIDE_CTAS) geodesic64_kernel(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
@@ -1492,12 +1492,10 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
     // come in warp-sized groups by their plasma work, start at their farthest plasma sample and look
     // up plasma samples only
     const bool marked = sizeof(R) == sizeof(float) && side.pool_chunks != 0ull;
-    // the stencil field test of plasma_at: always in the FP64 form; in FP32 where the rays are
-    // not queued by record count -- that order predicts a ray's cost from its records, which
-    // stops holding once field-free records are cheap (nine 256^2 images, fast form: cell-layout
-    // grids in the record-count order 11.6 ms with the test switched off there, 13.3 with it on;
-    // plane-layout grids in the consecutive queue 18.9 ms with the test, 25.8 before it). A
-    // run-time switch in one kernel, so that both queue orders run the same arithmetic; FP32
+    // the stencil field test of plasma_at: always in the FP64 form; in FP32 in the consecutive
+    // queue of plane-layout grids (nine 256^2 images, fast form: 18.9 ms with the test, 25.8
+    // without), not after the sample pass, whose marks say as much. A run-time switch in one
+    // kernel, so that both run the same arithmetic; FP32
     // compiles it into the plain polarized and unpolarized variants only, which keeps the
     // register budgets of the slow-light, auxiliary-image and learned variants.
     constexpr bool kFieldTestable = sizeof(T) == sizeof(double) || (!kSlow && !kAux && !kMlp);

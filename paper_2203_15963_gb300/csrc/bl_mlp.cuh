@@ -353,7 +353,7 @@ __global__ void __launch_bounds__(128) forward_kernel(const float* __restrict__ 
 }
 
 // The learned model over a trace's work list (the middle pass of the learned-coefficient
-// transfer): row i of the list (mlp_inputs_kernel) holds a sample's packed inputs in the first 8
+// transfer): row i of the list (fp32_samples_kernel) holds a sample's packed inputs in the first 8
 // of its 32 bytes, which the model's outputs y[7] (padded to 8) replace. Full 128-row tiles, the
 // row count read on the device, so the launch needs no host round trip. 1024^2: 2.6 ms; scanning the
 // pool for the rows, 15.8 ms.
