@@ -1648,13 +1648,16 @@ int blacklight_plan_config(const bl_plan_t* plan, bl_launch_config_t* out) {
     DevInfo di;
     int rc = dev_info(di);
     if (rc) return rc;
+    // (an adaptive plan keeps its images and features in its AdaptRun, and runs the defaults)
     const int geo_max = di.geo_blocks[plan->precision];
-    const int tr_max = di.transfer(plan->precision, plan->mlp, plan->feat);
+    const int tr_max = di.transfer(plan->precision, plan->mlp,
+                                   plan->adapt ? plan->adapt->feat : plan->feat);
     out->ray_order = plan->order;
     out->geo_ctas_per_sm = plan->cfg.geo_ctas > 0 && plan->cfg.geo_ctas < geo_max ? plan->cfg.geo_ctas : geo_max;
     out->tr_ctas_per_sm = plan->cfg.tr_ctas > 0 && plan->cfg.tr_ctas < tr_max ? plan->cfg.tr_ctas : tr_max;
     out->run_ms = plan->run_ms;
-    out->ilv_block = plan->descs[0].ilv > 1 && plan->order != 2 ? (1 << plan->descs[0].ilv_shift) : 0;
+    out->ilv_block = !plan->adapt && plan->descs[0].ilv > 1 && plan->order != 2
+                         ? (1 << plan->descs[0].ilv_shift) : 0;
     return 0;
 }
 
