@@ -290,8 +290,10 @@ typedef struct bl_launch_config {
                                  2 the work-ordered queue of 8x8 blocks described at
                                  blacklight_trace_batch (the default where the batch allows it;
                                  BL_EINVAL elsewhere) */
-    int32_t geo_ctas_per_sm;  /* persistent geodesic CTAs per SM, 0 = occupancy limit */
-    int32_t tr_ctas_per_sm;   /* persistent transfer CTAs per SM, 0 = occupancy limit */
+    int32_t geo_ctas_per_sm;  /* persistent geodesic CTAs per SM; 0 = the kernels' own rules (the
+                                 occupancy limit, fewer for few FP64 rays), reported as the
+                                 limit */
+    int32_t tr_ctas_per_sm;   /* persistent transfer CTAs per SM; 0 as above */
     float run_ms;             /* autotuned plans: device time of one run with this configuration */
     int32_t ilv_block;        /* batches of equal images on cell-layout grids queue their rays
                                  interleaved in blocks of this many rays of one image: a power
@@ -301,8 +303,8 @@ typedef struct bl_launch_config {
 } bl_launch_config_t;
 /* flags for blacklight_plan_create: search ray order, interleave block and CTAs per SM
  * (coordinate descent over timed runs of the plan's own workload; the images' outputs are
- * written while tuning). The choice is cached per device and workload shape for the life of
- * the process. */
+ * written while tuning). The choice is cached per device and workload (form, integrator,
+ * options, grid layout, images, rays and grid cells) for the life of the process. */
 enum { BL_PLAN_AUTOTUNE = 4u };
 /* config: NULL = defaults (the work-ordered queue where the batch allows it, else Morton;
  * occupancy limits), ignored with BL_PLAN_AUTOTUNE. `stream`

@@ -8,6 +8,7 @@
 #include <cstddef>
 #include <map>
 #include <mutex>
+#include <tuple>
 #include <vector>
 
 #include "../../include/blacklight.h"
@@ -413,6 +414,10 @@ struct DevInfo {
     int un64_occ[2] = {0, 0};       // FP64 second pass of unpolarized images: [plain, auxiliary images]
     int fwd_list_occ = 0;           // the model over the work list
     int rk_occ[2] = {0, 0};         // RK2/RK4 geodesic kernel: [double records, float records]
+    // CTAs per SM of the geodesic kernel a launch uses
+    int geodesic(int precision, int integrator) const {
+        return integrator == BL_INT_DP ? geo_blocks[precision] : rk_occ[precision == BL_PREC_FP64 ? 0 : 1];
+    }
     // CTAs per SM of the transfer variant a launch uses
     int transfer(int precision, const float* mlp, int feat) const {
         if (mlp) return tr_mlp_occ[(feat & bl::kFSlow) ? 1 : 0];
@@ -614,12 +619,12 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
         BL_CUDA(cudaGetLastError());
         cfg.bs = bl::BlockSource{psorted, pcount + 1, bl::kCostBlock, 1};
     }
-    const int pidx = precision;
     auto pick = [](int want, int occ) { return want > 0 && want < occ ? want : occ; };
-    const unsigned geo_grid = (unsigned)(di.sms * pick(cfg.geo_ctas, di.geo_blocks[pidx]));
+    const int geo_occ = di.geodesic(precision, cfg.integrator);
+    const unsigned geo_grid = (unsigned)(di.sms * pick(cfg.geo_ctas, geo_occ));
     const unsigned tr_grid = (unsigned)(di.sms * pick(cfg.tr_ctas, di.transfer(precision, mlp, cfg.feat)));
     // a hand-set or tuned number of CTAs an SM (otherwise the kernels' own rules apply)
-    const bool geo_set = cfg.geo_ctas > 0 && cfg.geo_ctas < di.geo_blocks[pidx];
+    const bool geo_set = cfg.geo_ctas > 0 && cfg.geo_ctas < geo_occ;
     const bool tr_set = cfg.tr_ctas > 0 && cfg.tr_ctas < di.transfer(precision, mlp, cfg.feat);
     const int record = transfer ? 1 : 0;
     const bool slow = (cfg.feat & bl::kFSlow) != 0;
@@ -630,14 +635,12 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
         if (w > 0) BL_CUDA(cudaMemsetAsync(ctr, 0, offsetof(bl::Counters, bad_rays), st));
         if (timing) BL_CUDA(cudaEventRecord(g_ev[2 * w], st));
         if (cfg.integrator != BL_INT_DP) {
-            const int ri = precision == BL_PREC_FP64 ? 0 : 1;
-            const unsigned rk_grid = (unsigned)(di.sms * pick(cfg.geo_ctas, di.rk_occ[ri]));
             if (precision == BL_PREC_FP64) {
                 bl::RecordSink<double> sink{(double*)(ws + L.pool), chunks, (unsigned long long)L.pool_chunks, ctr};
-                bl::geodesic_rk_kernel<double><<<rk_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, sink, record, cfg.bs, geo_set ? 0 : di.sms);
+                bl::geodesic_rk_kernel<double><<<geo_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, sink, record, cfg.bs, geo_set ? 0 : di.sms);
             } else {
                 bl::RecordSink<float> sink{(float*)(ws + L.pool), chunks, (unsigned long long)L.pool_chunks, ctr};
-                bl::geodesic_rk_kernel<float><<<rk_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, sink, record, cfg.bs, geo_set ? 0 : di.sms);
+                bl::geodesic_rk_kernel<float><<<geo_grid, 128, 0, st>>>(d_desc, n_images, b, e, hdr, sink, record, cfg.bs, geo_set ? 0 : di.sms);
             }
         } else {
             // double-float form: the wave's pixel initial states first, then the integrator
@@ -972,15 +975,17 @@ int trace_impl(int32_t n_images, const bl_camera_t* cams, const bl_metric_t* met
 // ---------------------------------------------------------------------------------------
 // Plans: prepared batched traces replayed as CUDA graphs, with an optional autotuner.
 // ---------------------------------------------------------------------------------------
+// What a tuned configuration depends on: which kernels run (form, coefficients, features,
+// integrator, grid layout, queue) and on how much (images, rays, grid cells in all snapshots).
 struct TuneKey {
-    int dev, precision, mlp, n_images;
-    int64_t rays;
+    int dev, precision, mlp, feat, integrator, cells, queue, n_images;
+    int64_t rays, grid;
     bool operator<(const TuneKey& o) const {
-        if (dev != o.dev) return dev < o.dev;
-        if (precision != o.precision) return precision < o.precision;
-        if (mlp != o.mlp) return mlp < o.mlp;
-        if (n_images != o.n_images) return n_images < o.n_images;
-        return rays < o.rays;
+        auto all = [](const TuneKey& k) {
+            return std::tie(k.dev, k.precision, k.mlp, k.feat, k.integrator, k.cells, k.queue,
+                            k.n_images, k.rays, k.grid);
+        };
+        return all(*this) < all(o);
     }
 };
 struct TuneVal {
@@ -1065,13 +1070,19 @@ int plan_time(bl_plan& P, const LaunchCfg& cfg, cudaStream_t st, float* ms) {
 
 // Coordinate descent: ray order at the occupancy limits, then geodesic CTAs per SM, then
 // transfer CTAs per SM. A candidate replaces the current choice only if it is faster by more
-// than kTuneMargin (run-to-run variation of these persistent kernels is about 1-2 %).
+// than kTuneMargin (run-to-run variation of these persistent kernels is about 1-2 %); where none
+// is, the number of CTAs stays 0: the kernels' own rules.
 constexpr float kTuneMargin = 0.03f;
 int plan_autotune(bl_plan& P, cudaStream_t st) {
     DevInfo di;
     int rc = dev_info(di);
     if (rc) return rc;
-    const TuneKey key{P.dev, P.precision, P.mlp ? 1 : 0, P.n_images, P.L.rays};
+    int64_t grid = 0;
+    for (const auto& d : P.descs) grid += (int64_t)d.nr * d.nt * d.nph * d.n_snap;
+    const int integrator = P.descs[0].integrator;
+    const TuneKey key{P.dev, P.precision, P.mlp ? 1 : 0, P.feat, integrator,
+                      all_cells(P.descs.data(), P.descs.size()) ? 1 : 0, P.L.pred_blocks > 0 ? 1 : 0,
+                      P.n_images, P.L.rays, grid};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);
         auto it = g_tune_cache.find(key);
@@ -1105,9 +1116,9 @@ int plan_autotune(bl_plan& P, cudaStream_t st) {
         }
         if ((rc = plan_set_order(P, order, st, ilv_shift))) return rc;
     }
-    const int geo_max = di.geo_blocks[P.precision];
+    const int geo_max = di.geodesic(P.precision, integrator);
     const int tr_max = di.transfer(P.precision, P.mlp, P.feat);
-    int geo_best = geo_max;
+    int geo_best = 0;
     for (int c = 1; c < geo_max; ++c) {
         LaunchCfg trial = cfg;
         trial.geo_ctas = c;
@@ -1115,7 +1126,7 @@ int plan_autotune(bl_plan& P, cudaStream_t st) {
         if (t < best * (1.0f - kTuneMargin)) { best = t; geo_best = c; }
     }
     cfg.geo_ctas = geo_best;
-    int tr_best = tr_max;
+    int tr_best = 0;
     for (int c = 1; c < tr_max; ++c) {
         LaunchCfg trial = cfg;
         trial.tr_ctas = c;
@@ -1649,7 +1660,8 @@ int blacklight_plan_config(const bl_plan_t* plan, bl_launch_config_t* out) {
     int rc = dev_info(di);
     if (rc) return rc;
     // (an adaptive plan keeps its images and features in its AdaptRun, and runs the defaults)
-    const int geo_max = di.geo_blocks[plan->precision];
+    const int integrator = plan->adapt ? plan->adapt->h_descs[0].integrator : plan->descs[0].integrator;
+    const int geo_max = di.geodesic(plan->precision, integrator);
     const int tr_max = di.transfer(plan->precision, plan->mlp,
                                    plan->adapt ? plan->adapt->feat : plan->feat);
     out->ray_order = plan->order;
