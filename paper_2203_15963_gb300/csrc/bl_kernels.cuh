@@ -2493,8 +2493,17 @@ __global__ void __launch_bounds__(128, kMlp ? 8 : BL_S32_MIN_CTAS) fp32_samples_
             wray = it.wray;
             idx = it.idx;
             const ImageDesc& im = imgs[it.q];
-            float cur[RecStride<float>::v];
-            load_record<float>(rec, cur);
+            // plain loads of the 14 values that this launch does not write (it writes the last two,
+            // so the record is not read-only for it)
+            float cur[14];
+            const float4* rp = reinterpret_cast<const float4*>(rec);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                const float4 r4 = rp[i];
+                cur[4 * i] = r4.x; cur[4 * i + 1] = r4.y; cur[4 * i + 2] = r4.z; cur[4 * i + 3] = r4.w;
+            }
+            const float2 r2 = *reinterpret_cast<const float2*>(rec + 12);
+            cur[12] = r2.x; cur[13] = r2.y;
             const T xs[3] = {cur[0], cur[1], cur[2]};
             KSGeom<T> G;
             ks_geom_pinned<kMlp>(xs[0], xs[1], xs[2], ic<T>(im, kcSpin), ic<T>(im, kcMass), im.flat != 0, G);
@@ -2611,14 +2620,14 @@ __global__ void __launch_bounds__(128, kMlp ? 8 : BL_S32_MIN_CTAS) fp32_samples_
             }
             const int32_t idx = base + lane;
             float* rec = pool + ((int64_t)__shfl_sync(0xffffffffu, cid, cj) * kChunk + lane) * RecStride<float>::v;
-            if (base == 0 && idx < nrec) pos = __ldg(reinterpret_cast<const float4*>(rec));
+            if (base == 0 && idx < nrec) pos = *reinterpret_cast<const float4*>(rec);
             const float4 v = pos;
             // the next chunk's positions (its id is at hand unless 32 ids are used up)
             const int cn = (cj + 1) & 31;
             const int32_t nid = __shfl_sync(0xffffffffu, cid, cn);
             if (idx + kChunk < nrec) {
                 const int64_t nc = cn != 0 ? nid : chunks[wray * kMaxChunks + base / kChunk + 1];
-                pos = __ldg(reinterpret_cast<const float4*>(pool + (nc * kChunk + lane) * RecStride<float>::v));
+                pos = *reinterpret_cast<const float4*>(pool + (nc * kChunk + lane) * RecStride<float>::v);
             }
             bool cand = false;
             if (idx < nrec) {
