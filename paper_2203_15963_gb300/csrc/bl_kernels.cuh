@@ -1626,10 +1626,10 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
         if (!marked || cur_what != kSampleEmpty) {
             const T xs[3] = {cur[0], cur[1], cur[2]};
             KSGeom<T> G;
-            // the sample pass's roundings (the auxiliary images, which it does not make, and the
-            // learned form keep the compiler's)
+            // the sample pass's roundings (the auxiliary images, which it does not make, keep the
+            // compiler's)
             constexpr bool kPinned = sizeof(T) == sizeof(float) && !kAux && !kMlp;
-            if constexpr (kPinned) ks_geom_pinned<false>(xs[0], xs[1], xs[2], a, m, flat, G);
+            if constexpr (kPinned || kMlp) ks_geom_pinned<kMlp>(xs[0], xs[1], xs[2], a, m, flat, G);
             else ks_geom<T>(xs[0], xs[1], xs[2], a, m, flat, false, G);
             Plasma<T> P;
             if (plasma_at<T, kSlow, kPinned>(im, xs, nxt_t, G, P, field_test)) {
