@@ -346,13 +346,13 @@ bool two_pass32(int precision, const float* mlp, int feat, bool cells) {
 }
 
 // Give every image's grid a field mask in the workspace's RayInit region, which is free while a
-// wave's transfer runs: images with the same grid share one. All or none: false (no masks) where
-// they do not fit, or where the wave has too few rays for reading the whole grid to pay (at most
-// 256 cells a ray and snapshot: 8 KB of grid, 1.2 ns of a ray's 25 ns or more).
-bool assign_masks(bl::ImageDesc* d, size_t n, char* ws, const Layout& L) {
+// wave's transfer runs: images with the same grid share one. Returns the cells (of all snapshots)
+// that building them reads, or 0: no masks, where they do not fit or not even a full wave has rays
+// enough (kMaskCellsPerRay). field_mask_kernel holds each wave's own rays against them.
+int64_t assign_masks(bl::ImageDesc* d, size_t n, char* ws, const Layout& L) {
     const size_t room = L.chunks - L.init;
     size_t used = 0;
-    double read = 0.0;
+    int64_t read = 0;
     std::vector<size_t> at(n);
     bool fits = true;
     for (size_t q = 0; q < n && fits; ++q) {
@@ -367,14 +367,15 @@ bool assign_masks(bl::ImageDesc* d, size_t n, char* ws, const Layout& L) {
         at[q] = used;
         d[q].mask_own = 1;
         used += align_up(4 * rows * (size_t)d[q].mask_pitch);
-        read += (double)rows * d[q].nr * d[q].n_snap;
-        fits = used <= room && read <= 256.0 * (double)L.wave;
+        read += (int64_t)rows * d[q].nr * d[q].n_snap;
+        fits = used <= room && read <= bl::kMaskCellsPerRay * L.wave;
     }
     for (size_t q = 0; q < n; ++q) {
-        d[q].mask = fits ? (uint32_t*)(ws + L.init + at[q]) : nullptr;
+        d[q].mask = nullptr;   // (set on the device)
+        d[q].mask_buf = fits ? (uint32_t*)(ws + L.init + at[q]) : nullptr;
         if (!fits) d[q].mask_own = 0;
     }
-    return fits;
+    return fits ? read : 0;
 }
 
 // Queue the rays of a batch of equal images interleaved (see setup_ray) when every image has
@@ -551,7 +552,7 @@ struct LaunchCfg {
     // order mixes images, whose 64 scalar gathers a sample then miss L2 more: fast form on nine
     // plane-layout images, transfer 25.8 -> 32.5 ms)
     bool order_transfer = true;
-    bool masks = false;           // the descriptors name field masks to build (assign_masks)
+    int64_t mask_cells = 0;       // assign_masks of the descriptors
 };
 
 // Every image's grid in the cell layout.
@@ -720,8 +721,9 @@ int launch_kernels(int32_t n_images, char* ws, const Layout& L, int precision, b
                 BL_CUDA(cudaMemsetAsync(tfirst, 0xff, sizeof(int32_t) * (size_t)(e - b), st));
                 BL_CUDA(cudaMemsetAsync(tnpl, 0, sizeof(int32_t) * (size_t)(e - b), st));
                 BL_CUDA(cudaMemsetAsync(thist, 0, sizeof(unsigned int) * bl::kCostBuckets, st));
-                if (cfg.masks) {
-                    bl::field_mask_kernel<<<(unsigned)(di.sms * 8), bl::kMaskThreads, 0, st>>>(d_desc, n_images);
+                if (cfg.mask_cells > 0) {
+                    bl::field_mask_kernel<<<(unsigned)(di.sms * 8), bl::kMaskThreads, 0, st>>>(
+                        d_desc, n_images, cfg.bs, b, e, cfg.mask_cells);
                     ++g_launches;
                     BL_CUDA(cudaGetLastError());
                 }
@@ -822,8 +824,8 @@ int launch_all(int32_t n_images, std::vector<bl::ImageDesc>& descs, char* ws,
     }
     c.integrator = descs.empty() ? BL_INT_DP : descs[0].integrator;
     c.order_transfer = all_cells(descs.data(), descs.size());
-    c.masks = transfer && two_pass32(precision, mlp, c.feat, c.order_transfer) &&
-              assign_masks(descs.data(), descs.size(), ws, L);
+    if (transfer && two_pass32(precision, mlp, c.feat, c.order_transfer))
+        c.mask_cells = assign_masks(descs.data(), descs.size(), ws, L);
     BL_CUDA(cudaMemcpyAsync(ws + L.descs, descs.data(), sizeof(bl::ImageDesc) * n_images,
                             cudaMemcpyHostToDevice, st));
     return launch_kernels(n_images, ws, L, precision, transfer, st, timing, mlp, c);
@@ -1013,7 +1015,7 @@ struct bl_plan {
     int ilv_shift = bl::kIlvShift;
     LaunchCfg cfg;
     float run_ms = 0.0f;
-    bool masks = false;      // the descriptors name field masks
+    int64_t mask_cells = 0;  // assign_masks of the descriptors
     int64_t kernels_per_run = 0;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
@@ -1050,7 +1052,7 @@ int plan_time(bl_plan& P, const LaunchCfg& cfg, cudaStream_t st, float* ms) {
         c.integrator = P.descs[0].integrator;
         c.cost_order = P.order == 2;
         c.order_transfer = all_cells(P.descs.data(), P.descs.size());
-        c.masks = P.masks;
+        c.mask_cells = P.mask_cells;
         if (!rc) rc = launch_kernels(P.n_images, P.ws, P.L, P.precision, true, st, false, P.mlp, c);
         if (!rc && it > 0) {
             if ((ce = cudaEventRecord(e1, st)) != cudaSuccess) rc = cuda_fail(ce, "record");
@@ -1169,7 +1171,7 @@ int plan_capture(bl_plan& P, cudaStream_t user) {
             c.integrator = P.descs[0].integrator;
             c.cost_order = P.order == 2;
             c.order_transfer = all_cells(P.descs.data(), P.descs.size());
-            c.masks = P.masks;
+            c.mask_cells = P.mask_cells;
             rc = launch_kernels(P.n_images, P.ws, P.L, P.precision, true, st, false, P.mlp, c);
         }
         cudaGraph_t g = nullptr;
@@ -1268,7 +1270,7 @@ struct AdaptRun {
     std::vector<int32_t> h_root;
     std::vector<unsigned long long> h_counts0;
     std::vector<bl::OutDesc> h_outd;
-    bool masks = false;                     // the descriptors name field masks
+    int64_t mask_cells = 0;                 // assign_masks of the descriptors
 };
 
 int adapt_prepare(AdaptRun& R, int32_t n_images, const bl_camera_t* cams, const bl_metric_t* mets,
@@ -1344,7 +1346,7 @@ int adapt_prepare(AdaptRun& R, int32_t n_images, const bl_camera_t* cams, const 
         }
     if (two_pass32(R.precision, R.mlp, R.feat, all_cells(R.h_descs.data(), (size_t)n_images)))
         for (int l = 0; l < levels; ++l)
-            R.masks = assign_masks(R.h_descs.data() + (size_t)l * n_images, n_images, R.ws, R.L);
+            R.mask_cells = assign_masks(R.h_descs.data() + (size_t)l * n_images, n_images, R.ws, R.L);
     // root block list (image-major, blocks row by row) and level-0 counts
     R.h_root.clear();
     R.h_counts0.assign(n_counts, 0ull);
@@ -1393,7 +1395,7 @@ int adapt_enqueue(AdaptRun& R, cudaStream_t st) {
         cfg.keep_bad = true;
         cfg.bs = bl::BlockSource{R.entries[l], R.counts + l, R.B};
         cfg.order_transfer = all_cells(R.h_descs.data(), (size_t)R.n_images);
-        cfg.masks = R.masks;
+        cfg.mask_cells = R.mask_cells;
         int rc = launch_kernels(R.n_images, R.ws, Ll, R.precision, true, st, false, R.mlp, cfg);
         if (rc) return rc;
         const int s = 1 << (R.max_level - l);
@@ -1608,8 +1610,8 @@ int blacklight_plan_create(int32_t n_images, const bl_camera_t* cams, const bl_m
         delete P;
         return fail(BL_ENOMEM, "cudaMalloc(%zu bytes): %s", P->L.total, cudaGetErrorString(e));
     }
-    P->masks = two_pass32(precision, mlp, P->feat, all_cells(P->descs.data(), P->descs.size())) &&
-               assign_masks(P->descs.data(), P->descs.size(), P->ws, P->L);
+    if (two_pass32(precision, mlp, P->feat, all_cells(P->descs.data(), P->descs.size())))
+        P->mask_cells = assign_masks(P->descs.data(), P->descs.size(), P->ws, P->L);
     if (flags & BL_PLAN_AUTOTUNE) {
         rc = plan_autotune(*P, st);
     } else {

@@ -55,9 +55,10 @@ struct ImageDesc {
     int64_t n_rays;         // rays traced for this image (n * n, or blocks x block^2)
     int32_t order;          // ray order: 0 Morton (n a power of 2), 1 rows
     int32_t layout;         // grid memory order: 0 planes [8][phi][theta][r], 1 cells [...][8]
-    // field mask of the grid (field_mask_kernel), rows of mask_pitch words; nullptr: none.
-    // mask_own: this image's launch builds it
+    // field mask of the grid, rows of mask_pitch words; nullptr: none. field_mask_kernel sets it to
+    // mask_buf for a wave that it builds the masks for; mask_own: this image's launch builds it
     uint32_t* mask;
+    uint32_t* mask_buf;
     int32_t mask_own, mask_pitch;
     // filled by the camera-frame kernel
     double x_cam[4], u_cam[4], kk[4], hh[4], vv[4];

@@ -875,15 +875,25 @@ __device__ __forceinline__ unsigned int cell_field_bits(const float* __restrict_
 // of the next row, plane and cell (a word a warp and ballot, so reads are coalesced; 1.4 times the
 // tile's cells, the excess mostly from L2), then the stencils' bits from those, word by word.
 // 256x128x128 cells: 37 us, three such grids 105 (two launches over linear cells and bits: 183).
+// A wave with fewer rays than one for kMaskCellsPerRay cells (8 KB of grid, 1.2 ns of a ray's 25 ns
+// or more) goes without: an adaptive trace launches a wave for each 2^20 rays that a level may hold
+// and knows on the device alone how many it does.
+constexpr int64_t kMaskCellsPerRay = 256;
 constexpr int kMaskR = 512, kMaskJ = 8, kMaskK = 4, kMaskThreads = 256;
 __device__ __forceinline__ bool mask_clear(const ImageDesc& im, size_t row, int i) {
     return ((__ldg(im.mask + row * (size_t)im.mask_pitch + (i >> 5)) >> (i & 31)) & 1u) == 0u;
 }
-__global__ void __launch_bounds__(kMaskThreads) field_mask_kernel(const ImageDesc* __restrict__ imgs,
-                                                                  int n_images) {
+__global__ void __launch_bounds__(kMaskThreads) field_mask_kernel(ImageDesc* imgs, int n_images,
+                                                                  BlockSource bs, int64_t ray_begin,
+                                                                  int64_t ray_end, int64_t cells_read) {
     constexpr int kW = kMaskR / 32 + 1, kJ = kMaskJ + 1, kK = kMaskK + 1;
     __shared__ uint32_t own[kK][kJ][kW];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool on = (wave_end(bs, ray_end) - ray_begin) * kMaskCellsPerRay >= cells_read;
+    if (blockIdx.x == 0)
+        for (int q = threadIdx.x; q < n_images; q += kMaskThreads)
+            imgs[q].mask = on ? imgs[q].mask_buf : nullptr;
+    if (!on) return;
     for (int q = 0; q < n_images; ++q) {
         const ImageDesc& im = imgs[q];
         if (!im.mask_own) continue;
@@ -933,7 +943,7 @@ __global__ void __launch_bounds__(kMaskThreads) field_mask_kernel(const ImageDes
                           own[kk + 1][jj][w + 1] | own[kk + 1][jj + 1][w + 1];
                     o |= (o >> 1) | (n << 31);
                 }
-                im.mask[((int64_t)(k0 + kk) * nt + j0 + jj) * im.mask_pitch + (i0 >> 5) + w] = o;
+                im.mask_buf[((int64_t)(k0 + kk) * nt + j0 + jj) * im.mask_pitch + (i0 >> 5) + w] = o;
             }
             __syncthreads();
         }
