@@ -393,7 +393,7 @@ size_t blacklight_workspace_size(int32_t n_images, const bl_camera_t* cams,
  * b2 [64], W3 [7][64], b3 [7], output offset [7], output scale [7], output trend A [7][3].
  * The model is o = offset + scale * y + A f, y the network output and f the three inputs
  * mapped linearly to [-1, 1]; offset, A and scale are fixed before training. All arrays are DEVICE pointers unless stated; calls are stream-ordered
- * and synchronise `stream` before returning; BL_ECUDA if a tensor-core wait ran out (never
+ * and synchronise `stream` before returning; BL_ETIMEOUT if a tensor-core wait ran out (never
  * expected; the kernels stop instead of waiting forever).
  * --------------------------------------------------------------------------------------- */
 #define BL_MLP_PARAMS 4906
@@ -423,7 +423,9 @@ typedef struct bl_mlp_train {
     double beta1, beta2, eps;/* Adam (Kingma & Ba 2015) */
 } bl_mlp_train_t;
 /* Train params in place (mean squared error of the normalised outputs). loss_history:
- * optional DEVICE float [steps] receiving each step's mean squared error. */
+ * optional DEVICE float [steps] receiving each step's mean squared error. If a tensor-core wait
+ * runs out (BL_ETIMEOUT) training stops there: params keep their values, and the steps from that one
+ * on leave loss_history as it is. */
 int blacklight_mlp_train(const bl_mlp_train_t* cfg, float* params, float* loss_history,
                          void* stream);
 /* Gradient of the mean squared error over the n samples into grad [BL_MLP_PARAMS] (zero for
@@ -473,6 +475,11 @@ int blacklight_set_memory_retention(uint64_t bytes);
  * arrive = 1 it arrives first (returns 0), with arrive = 0 nothing arrives and the wait runs out
  * (returns BL_ETIMEOUT). No fault, no unbounded wait. */
 int blacklight_selftest_wait(int64_t max_cycles, int32_t arrive, void* stream);
+
+/* Self-test of what follows such a wait: blacklight_mlp_train as if one had run out before the
+ * first step. Returns BL_ETIMEOUT; params and loss_history keep their values. */
+int blacklight_selftest_train_stopped(const bl_mlp_train_t* cfg, float* params,
+                                      float* loss_history, void* stream);
 
 /* Arithmetic peaks of the current device, measured (the paper has no counterpart: these are
  * the denominators of the rooflines a benchmark reports). Each probe is a kernel of

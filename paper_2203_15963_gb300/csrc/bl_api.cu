@@ -1818,7 +1818,7 @@ static_assert(BL_MLP_PARAMS == bl::mlp::kParams, "parameter count");
 
 namespace {
 
-// Run `launch(err)` with a zeroed device error flag; BL_ECUDA if a kernel reported a timeout.
+// Run `launch(err)` with a zeroed device error flag; BL_ETIMEOUT if a kernel reported a timeout.
 template <class F>
 int with_tc_flag(cudaStream_t st, F launch) {
     int* err = nullptr;
@@ -1970,8 +1970,13 @@ int blacklight_mlp_grad(const float* params, int64_t n, const float* inputs, con
     return rc;
 }
 
-int blacklight_mlp_train(const bl_mlp_train_t* cfg, float* params, float* loss_history,
-                         void* stream) {
+}  // extern "C"
+
+namespace {
+
+// stopped: as if a wait had run out before the first step (the self-test)
+int mlp_train(const bl_mlp_train_t* cfg, float* params, float* loss_history, void* stream,
+              bool stopped) {
     g_detail[0] = 0;
     if (!cfg || cfg->size != sizeof(bl_mlp_train_t)) return fail(BL_EINVAL, "cfg.size mismatch");
     if (cfg->batch < 128 || cfg->batch % 128 || cfg->n < cfg->batch || cfg->steps < 0)
@@ -2000,6 +2005,7 @@ int blacklight_mlp_train(const bl_mlp_train_t* cfg, float* params, float* loss_h
     float *w = (float*)(buf + img_bytes), *m = w + n_tr, *v = m + n_tr, *part = v + n_tr,
           *part_loss = part + n_part;
     rc = with_tc_flag(st, [&](int* err) -> int {
+        if (stopped) BL_CUDA(cudaMemsetAsync(err, 0xff, sizeof(int), st));
         BL_CUDA(cudaMemsetAsync(buf, 0, img_bytes + sizeof(float) * 3 * n_tr, st));
         bl::mlp::image_kernel<<<(BL_MLP_PARAMS + 127) / 128, 128, 0, st>>>(params, img, w);
         ++g_launches;
@@ -2035,10 +2041,10 @@ int blacklight_mlp_train(const bl_mlp_train_t* cfg, float* params, float* loss_h
                                        (float)cfg->eps, (float)(1.0 - p1), (float)(1.0 - p2),
                                        (const float*)part_loss,
                                        loss_history ? loss_history + t : (float*)nullptr,
-                                       (float)(1.0 / (7.0 * cfg->batch))));
+                                       (float)(1.0 / (7.0 * cfg->batch)), (const int*)err));
             g_launches += 2;
         }
-        bl::mlp::unslot_kernel<<<(unsigned)((n_tr + 127) / 128), 128, 0, st>>>(w, params);
+        bl::mlp::unslot_kernel<<<(unsigned)((n_tr + 127) / 128), 128, 0, st>>>(w, params, err);
         ++g_launches;
         BL_CUDA(cudaGetLastError());
         return 0;
@@ -2047,6 +2053,20 @@ int blacklight_mlp_train(const bl_mlp_train_t* cfg, float* params, float* loss_h
     cudaError_t se = cudaStreamSynchronize(st);
     if (!rc && se != cudaSuccess) rc = cuda_fail(se, "cudaStreamSynchronize");
     return rc;
+}
+
+}  // namespace
+
+extern "C" {
+
+int blacklight_mlp_train(const bl_mlp_train_t* cfg, float* params, float* loss_history,
+                         void* stream) {
+    return mlp_train(cfg, params, loss_history, stream, false);
+}
+
+int blacklight_selftest_train_stopped(const bl_mlp_train_t* cfg, float* params, float* loss_history,
+                                      void* stream) {
+    return mlp_train(cfg, params, loss_history, stream, true);
 }
 
 int blacklight_mlp_forward(const float* params, int64_t n, const float* inputs, float* outputs,

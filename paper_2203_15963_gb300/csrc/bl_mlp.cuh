@@ -520,10 +520,11 @@ __global__ void image_kernel(const float* __restrict__ P, unsigned char* __restr
     image_store(img, i, P[i]);
     if (w && i < kOffMean) w[i] = P[slot_param(i)];
 }
-// The trained parameters back into P.
-__global__ void unslot_kernel(const float* __restrict__ w, float* __restrict__ P) {
+// The trained parameters back into P (not after a step whose wait ran out).
+__global__ void unslot_kernel(const float* __restrict__ w, float* __restrict__ P,
+                              const int* __restrict__ err) {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < kOffMean) P[slot_param(s)] = w[s];
+    if (s < kOffMean && *err == 0) P[slot_param(s)] = w[s];
 }
 
 // Eight consecutive values of a row of a bf16 operand tile: one 16-byte store.
@@ -540,7 +541,8 @@ __device__ __forceinline__ void st_row8(unsigned char* tile, int row, int col, i
 // and *loss atomically (summation order, and so the last bits, vary between runs). Otherwise
 // tile b stores its own sums, part[b][kOffMean] (every trained parameter, in slot order) and
 // part_loss[b], for a reduction in a fixed order (adam_kernel), which makes training
-// reproducible bit for bit.
+// reproducible bit for bit. *err: set where a wait runs out; a launch that finds it set computes
+// nothing, so a run of steps waits out one limit, not one a step.
 __global__ void __launch_bounds__(128, 1) train_kernel(const unsigned char* __restrict__ img,
                                                        int64_t n, const float* __restrict__ in,
                                                        const float* __restrict__ tg,
@@ -625,8 +627,12 @@ __global__ void __launch_bounds__(128, 1) train_kernel(const unsigned char* __re
     // ---- the weights of this step
     tc::grid_dependency_wait();
     tc::grid_launch_dependents();
-    if (t == 0) tc::bulk_load(sm + kTImg, img, kImgBytes, ibar);
-    const bool have = __syncthreads_and(tc::mbar_wait(ibar, 0u, kWaitCycles)) != 0;
+    bool stopped = false;
+    if (t == 0) {
+        tc::bulk_load(sm + kTImg, img, kImgBytes, ibar);
+        stopped = *(volatile const int*)err != 0;
+    }
+    const bool have = __syncthreads_and(tc::mbar_wait(ibar, 0u, kWaitCycles) && !stopped) != 0;
 
     do {
         if (!(ok = have)) break;
@@ -794,15 +800,18 @@ __global__ void __launch_bounds__(128, 1) train_kernel(const unsigned char* __re
 // of 128 tiles into shared memory at once (16 loads in flight a thread; one thread a slot walking
 // the tiles in device memory took twice the time), one warp adds them. c1, c2 are the bias
 // corrections 1 - beta1^t, 1 - beta2^t. Writes the new weight into the next step's image. The
-// last block adds the tiles' squared errors into loss_hist (mean over n_total x 7).
+// last block adds the tiles' squared errors into loss_hist (mean over n_total x 7). Where a tile's
+// wait ran out (*err) its sums are missing: loss_hist stays, and what becomes of w no longer matters
+// (unslot_kernel).
 constexpr int kAdamThreads = 256, kAdamTiles = 128;
 constexpr int kAdamBlocks = (kOffMean + 31) / 32 + 1;
 __global__ void __launch_bounds__(kAdamThreads) adam_kernel(
         float* __restrict__ w, unsigned char* __restrict__ img, const float* __restrict__ part,
         int n_tiles, float* __restrict__ m, float* __restrict__ v, float lr, float beta1,
         float beta2, float eps, float c1, float c2, const float* __restrict__ part_loss,
-        float* loss_hist, float inv_count) {
+        float* loss_hist, float inv_count, const int* err) {
     __shared__ float col[kAdamTiles][32];
+    __shared__ int stopped;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     tc::grid_dependency_wait();
     tc::grid_launch_dependents();
@@ -812,6 +821,8 @@ __global__ void __launch_bounds__(kAdamThreads) adam_kernel(
     const float* src = is_loss ? part_loss : part + s;
     const size_t stride = is_loss ? 1 : kOffMean;
     float mo = 0.0f, vo = 0.0f, wo = 0.0f, g = 0.0f;
+    // (an idle lane's load, beside the others': read by the storing lane it costs 0.9 us a step)
+    if (is_loss && threadIdx.x == 33) stopped = *(volatile const int*)err;
     if (warp == 0 && on && !is_loss) {
         mo = m[s];
         vo = v[s];
@@ -833,7 +844,7 @@ __global__ void __launch_bounds__(kAdamThreads) adam_kernel(
     }
     if (warp != 0 || !on) return;
     if (is_loss) {
-        *loss_hist = g * inv_count;
+        if (!stopped) *loss_hist = g * inv_count;
         return;
     }
     // (roundings written out: a run's bits do not hang on the compiler's choice of products)

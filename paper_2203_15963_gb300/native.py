@@ -172,6 +172,7 @@ def load():
                                                   C.POINTER(C.c_void_p)]
     L.blacklight_plan_level_rays.argtypes = [P, C.POINTER(C.c_int32), P]
     L.blacklight_selftest_wait.argtypes = [C.c_int64, C.c_int32, P]
+    L.blacklight_selftest_train_stopped.argtypes = [C.POINTER(MlpTrain), P, P, P]
     L.blacklight_set_memory_retention.argtypes = [C.c_uint64]
     L.blacklight_measure_peaks.argtypes = [C.POINTER(Peaks), C.c_int32, P]
     L.blacklight_trace_host_batch.argtypes = [C.c_int32, C.POINTER(Camera), C.POINTER(Metric),
@@ -449,11 +450,15 @@ def blacklight_mlp_normalise(inputs, targets, params, stream=None):
                                                   _ptr(params), _stream(stream)))
 
 
+def _train_struct(inputs, targets, batch, steps, lr_start, lr_end, beta1=0.9, beta2=0.999, eps=1e-8):
+    return MlpTrain(C.sizeof(MlpTrain), inputs.shape[0], inputs.data_ptr(), targets.data_ptr(),
+                    int(batch), int(steps), float(lr_start), float(lr_end), float(beta1),
+                    float(beta2), float(eps))
+
+
 def blacklight_mlp_train(params, inputs, targets, batch, steps, lr_start, lr_end, beta1=0.9,
                          beta2=0.999, eps=1e-8, loss_history=None, stream=None):
-    cfg = MlpTrain(C.sizeof(MlpTrain), inputs.shape[0], inputs.data_ptr(), targets.data_ptr(),
-                   int(batch), int(steps), float(lr_start), float(lr_end), float(beta1),
-                   float(beta2), float(eps))
+    cfg = _train_struct(inputs, targets, batch, steps, lr_start, lr_end, beta1, beta2, eps)
     return _check(load().blacklight_mlp_train(C.byref(cfg), _ptr(params), _ptr(loss_history),
                                               _stream(stream)))
 
@@ -496,6 +501,15 @@ def blacklight_selftest_wait(max_cycles, arrive, stream=None) -> int:
     if rc == BL_ETIMEOUT:
         return rc
     return _check(rc)
+
+
+def blacklight_selftest_train_stopped(params, inputs, targets, batch, steps, lr_start, lr_end,
+                                      loss_history=None, stream=None) -> int:
+    """BL_ETIMEOUT (returned, not raised)."""
+    cfg = _train_struct(inputs, targets, batch, steps, lr_start, lr_end)
+    rc = load().blacklight_selftest_train_stopped(C.byref(cfg), _ptr(params), _ptr(loss_history),
+                                                  _stream(stream))
+    return rc if rc == BL_ETIMEOUT else _check(rc)
 
 
 def blacklight_launch_count(reset=False) -> int:
