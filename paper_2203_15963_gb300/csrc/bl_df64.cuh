@@ -75,11 +75,6 @@ __device__ __forceinline__ df64 df_mul_nn(const df64& x, const df64& y) {
     e = fmaf(x.lo, y.hi, e);
     return df64(p, e);
 }
-__device__ __forceinline__ df64 df_mul_f(const df64& x, float b) {
-    df64 p = df_two_prod(x.hi, b);
-    p.lo = fmaf(x.lo, b, p.lo);
-    return df_fast_two_sum(p.hi, p.lo);
-}
 // 1/x: hardware FP32 seed y0 (~1 ulp), residual e = 1 - x y0 formed with FMAs (the product
 // x.hi y0 is exact inside the first one), then 1/x = y0 / (1 - e) = y0 (1 + e + e^2 + ...)
 // to second order; relative error ~5e-14.
@@ -171,6 +166,5 @@ __device__ __forceinline__ bool operator<(const df64& x, const df64& y) {
 __device__ __forceinline__ bool operator>(const df64& x, const df64& y) { return y < x; }
 __device__ __forceinline__ df64 fabs(const df64& x) { return x.hi < 0.0f ? -x : x; }
 __device__ __forceinline__ double df_to_double(const df64& x) { return (double)x.hi + (double)x.lo; }
-__device__ __forceinline__ df64 df_from_double(double d) { return df64(d); }
 
 }  // namespace bl

@@ -432,7 +432,7 @@ __device__ __forceinline__ void geodesic64_body(const ImageDesc* __restrict__ im
                                                      r_grid, near1);
                 if (nsub == 0) {
                     KSGeom<double> Gm;
-                    ks_geom<double>(ym[1], ym[2], ym[3], im.spin, im.mass, C.flat, false, Gm);
+                    ks_geom<double>(ym[1], ym[2], ym[3], im.spin, im.mass, C.flat, Gm);
                     const double L = -ym[4] + Gm.l[1] * ym[5] + Gm.l[2] * ym[6] + Gm.l[3] * ym[7];
                     const double kt_up = -ym[4] + Gm.f * L;
                     // ds/dl = (g_pq k^p k^q)^1/2 = alpha |k^t| for a null ray
@@ -735,7 +735,7 @@ __global__ void __launch_bounds__(128, 3) geodesic_rk_kernel(const ImageDesc* __
                 const double hl = fabs(h);
                 if (nsub == 0) {
                     KSGeom<double> Gm;
-                    ks_geom<double>(ym[1], ym[2], ym[3], C.a, im.mass, C.flat, false, Gm);
+                    ks_geom<double>(ym[1], ym[2], ym[3], C.a, im.mass, C.flat, Gm);
                     const double L = -ym[4] + Gm.l[1] * ym[5] + Gm.l[2] * ym[6] + Gm.l[3] * ym[7];
                     const double kt_up = -ym[4] + Gm.f * L;
                     const double ds = hl * fabs(kt_up) / sqrt(1.0 + Gm.f);

@@ -438,7 +438,7 @@ __device__ __forceinline__ void geodesic_df_body(const ImageDesc* __restrict__ i
                 {
                     KSGeom<float> Gm;
                     ks_geom<float>(ymf[1], ymf[2], ymf[3], imgs[q].f_c[kcSpin], imgs[q].f_c[kcMass],
-                                   C.flat, false, Gm);
+                                   C.flat, Gm);
                     const float L = -ymf[4] + Gm.l[1] * ymf[5] + Gm.l[2] * ymf[6] + Gm.l[3] * ymf[7];
                     kt_up = -ymf[4] + Gm.f * L;
                     rmid = Gm.r;

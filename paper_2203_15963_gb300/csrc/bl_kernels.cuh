@@ -25,7 +25,7 @@ __global__ void camera_frame_kernel(ImageDesc* imgs, int n_images) {
     const double r = im.cam_r;
     double x[4] = {0.0, st * (r * cp - a * sp), st * (r * sp + a * cp), r * ct};
     KSGeom<double> G;
-    ks_geom<double>(x[1], x[2], x[3], a, m, flat, false, G);
+    ks_geom<double>(x[1], x[2], x[3], a, m, flat, G);
     // Jacobian columns d x^a / d (r, theta, phi)
     const double J[3][3] = {{st * cp, ct * (r * cp - a * sp), st * (-r * sp - a * cp)},
                             {st * sp, ct * (r * sp + a * cp), st * (r * cp - a * sp)},
@@ -219,9 +219,6 @@ __device__ __forceinline__ double aux_load(const ImageDesc& im, int a, int64_t p
                          : (double)((const float*)im.aux)[a * npix + pix];
 }
 
-__device__ __forceinline__ double im_spin(const ImageDesc* imgs, int q) { return imgs[q].spin; }
-__device__ __forceinline__ double im_mass(const ImageDesc* imgs, int q) { return imgs[q].mass; }
-
 // Warp-aggregated fetch-and-add: every lane that calls it gets a distinct index.
 __device__ __forceinline__ unsigned long long warp_fetch_add(unsigned long long* ctr) {
     const unsigned mask = __activemask();
@@ -256,7 +253,7 @@ __device__ __forceinline__ void pixel_state(const ImageDesc& im, int i, int j, d
     const double bb = (j - 0.5 * n + 0.5) * im.width / n;
     for (int al = 0; al < 4; ++al) y[al] = im.x_cam[al] + aa * im.hh[al] + bb * im.vv[al];
     KSGeom<double> G;
-    ks_geom<double>(y[1], y[2], y[3], im.spin, im.mass, im.flat != 0, false, G);
+    ks_geom<double>(y[1], y[2], y[3], im.spin, im.mass, im.flat != 0, G);
     const double ka[3] = {im.kk[1], im.kk[2], im.kk[3]};
     // g_tt (k^t)^2 + 2 g_ta k^a k^t + g_ab k^a k^b = 0
     const double lk = G.l[1] * ka[0] + G.l[2] * ka[1] + G.l[3] * ka[2];
@@ -1613,7 +1610,7 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
             if constexpr (!kUnpol) {
                 // read out in the camera basis at the camera-side node
                 KSGeom<T> G;
-                ks_geom<T>(prev[6], prev[7], prev[8], a, m, flat, false, G);
+                ks_geom<T>(prev[6], prev[7], prev[8], a, m, flat, G);
                 T hv[4], vv[4];
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {
@@ -1640,7 +1637,7 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
             // compiler's)
             constexpr bool kPinned = sizeof(T) == sizeof(float) && !kAux && !kMlp;
             if constexpr (kPinned || kMlp) ks_geom_pinned<kMlp>(xs[0], xs[1], xs[2], a, m, flat, G);
-            else ks_geom<T>(xs[0], xs[1], xs[2], a, m, flat, false, G);
+            else ks_geom<T>(xs[0], xs[1], xs[2], a, m, flat, G);
             Plasma<T> P;
             if (plasma_at<T, kSlow, kPinned>(im, xs, nxt_t, G, P, field_test)) {
                 const T kl[4] = {kt, cur[3], cur[4], cur[5]};
@@ -1789,7 +1786,7 @@ __device__ __forceinline__ void transport32_body(
             if constexpr (!kUnpol) {
                 // read out in the camera basis at the camera-side node
                 KSGeom<T> G;
-                ks_geom<T>(prev[6], prev[7], prev[8], a, m, flat, false, G);
+                ks_geom<T>(prev[6], prev[7], prev[8], a, m, flat, G);
                 T hl[4], vl[4];
                 lower4(G, im.f_hh, hl);
                 lower4(G, im.f_vv, vl);
@@ -2055,7 +2052,7 @@ __global__ void __launch_bounds__(128, BL_PRE64_MIN_CTAS) fp64_samples_kernel(co
             load_record<double>(pool + it.k * RecStride<double>::v, cur);
             const T xs[3] = {cur[0], cur[1], cur[2]};
             KSGeom<T> G;
-            ks_geom<T>(xs[0], xs[1], xs[2], a, m, flat, false, G);
+            ks_geom<T>(xs[0], xs[1], xs[2], a, m, flat, G);
             Plasma<T> P;
             if (plasma_at<T, kSlow>(im, xs, cur[13], G, P, true)) {
                 const T kl[4] = {kt, cur[3], cur[4], cur[5]};
@@ -2255,7 +2252,7 @@ __device__ __forceinline__ void transport_fp64_body(
     using T = double;
     const int64_t re = wave_end(bs, ray_end);
     const int64_t n_rays = re > ray_begin ? re - ray_begin : 0;
-    const int64_t total_rays = perm ? ordered_total<kTransportGroup>(n_rays) : n_rays;
+    const int64_t total_rays = ordered_total<kTransportGroup>(n_rays);
     int64_t wray = 0, ray = 0, opix = 0;
     bool active = false, started = false;
     int q = 0, pi = 0, pj = 0;
@@ -2270,8 +2267,8 @@ __device__ __forceinline__ void transport_fp64_body(
         if (need) {
             if ((int64_t)got >= total_rays) exhausted = true;
             else {
-                // the sample pass's work order (longest first) where there is one
-                wray = perm ? ordered_ray<kTransportGroup>(perm, got, n_rays) : (int64_t)got;
+                // the sample pass's work order (longest first)
+                wray = ordered_ray<kTransportGroup>(perm, got, n_rays);
                 ray = ray_begin + wray;
             }
         }
@@ -2291,9 +2288,9 @@ __device__ __forceinline__ void transport_fp64_body(
                 }
                 continue;
             }
-            // from the farthest plasma sample where the sample pass found it (the records
-            // beyond it leave N = 0 untouched); with none, straight to the read-out
-            idx = side.first ? side.first[wray] : hd.nrec - 1;
+            // from the farthest plasma sample (the records beyond it leave N = 0 untouched); with
+            // none, straight to the read-out
+            idx = side.first[wray];
             kt = hd.kt;
             a = ic<T>(im, kcSpin);
             m = ic<T>(im, kcMass);
@@ -2328,7 +2325,7 @@ __device__ __forceinline__ void transport_fp64_body(
             if (finishing) {
                 // read out in the camera basis at the camera-side node of the last record
                 KSGeom<T> G;
-                ks_geom<T>(__ldg(pr + 6), __ldg(pr + 7), __ldg(pr + 8), a, m, flat, false, G);
+                ks_geom<T>(__ldg(pr + 6), __ldg(pr + 7), __ldg(pr + 8), a, m, flat, G);
                 T hl[4], vl[4];
                 lower4(G, im.hh, hl);
                 lower4(G, im.vv, vl);

@@ -109,23 +109,18 @@ constexpr double kPi = 3.14159265358979323846;
 // Kerr metric in Cartesian Kerr-Schild form (Sec. 2, Eq. cks_aux):
 //   g_ab = eta_ab + f l_a l_b,  g^ab = eta^ab - f l^a l^b,  l_a = (1, lx, ly, lz),
 //   f = 2 M r^3 / (r^4 + a^2 z^2),  2 r^2 = R^2 - a^2 + ((R^2 - a^2)^2 + 4 a^2 z^2)^{1/2}.
-// Derivatives are hand-expanded: with D = ((R^2 - a^2)^2 + 4 a^2 z^2)^{1/2},
-//   dr/dx = r x / D, dr/dy = r y / D, dr/dz = z (r^2 + a^2) / (r D).
 // ---------------------------------------------------------------------------------------
 template <class T>
 struct KSGeom {
     T r, f;
     T l[4];         // covariant l_a, l[0] = 1
-    T df[3];        // d_c f
-    T dl[3][3];     // d_c l_b (b spatial)
 };
 
 template <class T>
-__device__ __forceinline__ void ks_geom(T x, T y, T z, T a, T m, bool flat, bool derivs,
-                                        KSGeom<T>& G) {
+__device__ __forceinline__ void ks_geom(T x, T y, T z, T a, T m, bool flat, KSGeom<T>& G) {
     // Special functions kept to two reciprocal square roots and one reciprocal:
     // D = D2 rsqrt(D2), r = r2 rsqrt(r2), and 1/P, 1/s4 from 1/(P s4).
-    constexpr T c1 = T(1), c2 = T(2), c3 = T(3), c4 = T(4), cHalf = T(0.5), c0 = T(0);
+    constexpr T c1 = T(1), c2 = T(2), c4 = T(4), cHalf = T(0.5), c0 = T(0);
     const T rr2 = x * x + y * y + z * z;
     const T q = rr2 - a * a;
     const T D2 = q * q + c4 * a * a * z * z;
@@ -146,19 +141,9 @@ __device__ __forceinline__ void ks_geom(T x, T y, T z, T a, T m, bool flat, bool
     G.l[1] = (r * x + a * y) * iP;
     G.l[2] = (r * y - a * x) * iP;
     G.l[3] = z * ir;
-    if (!derivs) return;
-    const T dr[3] = {r * x * iD, r * y * iD, z * P * ir * iD};
-    for (int c = 0; c < 3; ++c) {
-        const T extra = (c == 2) ? c2 * a * a * z : c0;
-        G.df[c] = flat ? c0 : f * (c3 * dr[c] * ir - (c4 * r2 * r * dr[c] + extra) * is4);
-        const T two_r_dr_iP = c2 * r * dr[c] * iP;
-        G.dl[c][0] = (dr[c] * x + (c == 0 ? r : c0) + (c == 1 ? a : c0)) * iP - G.l[1] * two_r_dr_iP;
-        G.dl[c][1] = (dr[c] * y + (c == 1 ? r : c0) - (c == 0 ? a : c0)) * iP - G.l[2] * two_r_dr_iP;
-        G.dl[c][2] = ((c == 2 ? c1 : c0) - G.l[3] * dr[c]) * ir;
-    }
 }
 
-// ks_geom in FP32 without derivatives, its roundings written out, for the FP32 sample pass: rays
+// ks_geom in FP32, its roundings written out, for the FP32 sample pass: rays
 // that graze the horizon amplify a last-bit difference of a sample's plasma state a thousandfold, and
 // the bf16 rounding of the learned form's model inputs one to 2^-9, so both are formed from the same
 // bits whatever kernel the call is inlined into. The two forms round the numerator of l_y in
@@ -182,13 +167,6 @@ __device__ __forceinline__ void ks_geom_pinned(float x, float y, float z, float 
     G.l[1] = __fmul_rn(__fmaf_rn(a, y, __fmul_rn(r, x)), iP);
     G.l[2] = __fmul_rn(kModel ? __fmaf_rn(r, y, -__fmul_rn(a, x)) : __fmaf_rn(-a, x, __fmul_rn(r, y)), iP);
     G.l[3] = __fmul_rn(z, ir);
-}
-
-// r of a CKS point (Eq. cks_aux:r).
-template <class T>
-__device__ __forceinline__ T ks_r(T x, T y, T z, T a) {
-    const T q = x * x + y * y + z * z - a * a;
-    return sqrt(T(0.5) * (q + sqrt(q * q + T(4) * a * a * z * z)));
 }
 
 // Lower / raise with g = eta + f l l (contravariant l^a = (-1, lx, ly, lz)).
