@@ -96,7 +96,8 @@ __device__ __forceinline__ double mul3(double a, double b, double c) {
 //   V = (A - 2 r L_xy) / (r^2 + a^2) - k_z z / r^2,
 // and d_c f = F1 d_c r - [c = z] 2 a^2 z f / (r^4 + a^2 z^2), F1 = f (3 / r - 4 r^3 / (r^4 + a^2 z^2)).
 // The same quantities as the nine-derivative form, in about 40 fewer operations.
-// Exact scalings are folded away: d_c f is carried halved (F1), so that 1/2 L need not be formed.
+// Exact scalings are folded away: d_c f is carried halved (F1, the halving in its bracket: f itself
+// is zero in flat space and, r^6 overflowing, beyond r = 2e51), so that 1/2 L need not be formed.
 // The order of operations and the roundings are part of the method: rays that graze the photon
 // orbit amplify them, and every kernel integrates with the same ones (bl_geodf.cuh in
 // double-float).
@@ -138,8 +139,7 @@ __device__ __forceinline__ double geodesic_rhs64(const double y[8], const Rhs64&
     const double Sx = fma_dot2(fma_dot2(r, kx, -a, ky), iP, drx, V);
     const double Sy = fma_dot2(fma_dot2(a, kx, r, ky), iP, dry, V);
     const double Sz = __fma_rn(drz, V, w);
-    const double fh = C.flat ? 0.0 : scale_exp(f, -1);
-    const double F1 = __dmul_rn(fh, fma_dot2(3.0, ir, -__dmul_rn(scale_exp(r2, 2), r), is4));
+    const double F1 = __dmul_rn(f, fma_dot2(1.5, ir, -__dmul_rn(scale_exp(r2, 1), r), is4));
     const double dfx = __dmul_rn(F1, drx), dfy = __dmul_rn(F1, dry);
     const double dfz = __fma_rn(F1, drz, -mul3(aaz, f, is4));
     dy[5] = __dmul_rn(L, fma_dot2(dfx, L, f, Sx));
