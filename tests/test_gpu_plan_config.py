@@ -93,3 +93,25 @@ def test_fixed_step_plan_reports_its_own_kernel(torus):
     assert 1 <= rk.config()["geo_ctas_per_sm"] < dp.config()["geo_ctas_per_sm"]
     dp.close()
     rk.close()
+
+
+@pytest.mark.parametrize("precision", [native.BL_PREC_FP64, native.BL_PREC_MIXED])
+@pytest.mark.parametrize("integrator,n", [(native.BL_INT_RK4, 37), (native.BL_INT_RK2, 37),
+                                          (native.BL_INT_RK4, 300)])
+@pytest.mark.parametrize("ctas", [1, 2])
+def test_fixed_step_launch_shapes_give_the_same_bits(torus, precision, integrator, n, ctas):
+    """The kernel's own rule (9 rays an SM: one CTA of an SM stays; 592: two) against a set number."""
+    gp, prim = torus
+    cam = S.Camera(theta=math.radians(80.0), n=n)
+    met = S.Metric(spin=0.9, precision=precision, integrator=integrator, f_step=0.05)
+    dt = torch.float64 if precision == native.BL_PREC_FP64 else torch.float32
+    a, b = (images.alloc_outputs(n, dt, end_state=True, samples=True) for _ in range(2))
+    images.trace_images([cam], [met], [gp], [prim], [FREQ], outs=[a])
+    plan = native.Plan([cam], [met], [gp], [prim], [FREQ], [b],
+                       config={"geo_ctas_per_sm": ctas, "tr_ctas_per_sm": ctas})
+    assert plan.config()["geo_ctas_per_sm"] == ctas
+    plan.run()
+    plan.check()
+    plan.close()
+    for k in a:
+        assert torch.equal(a[k], b[k]), k
