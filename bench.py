@@ -68,9 +68,10 @@ FLOP64_EMIT_PER_RECORD = 108
 # Arithmetic per transfer sample of the method (see the module docstring): FP32 flops and
 # special-function instructions of the single-kernel FP32 transfer per sample with the
 # stencil field test on (a sample whose lookup stencil carries no magnetic field stops after
-# the lookup), from the ncu capture of the one-image 256^2 case on plane-layout grids (a =
+# the lookup), from an ncu capture of the one-image 256^2 case on plane-layout grids (a =
 # 0.94, i = 60 deg; 18,372,183 samples): 2 x 4.397e9 FFMA + 2.661e9 FMUL + 0.703e9 FADD
-# thread instructions, 2.43e8 MUFU.
+# thread instructions, 2.43e8 MUFU. (The kernel has since had some roundings written out and
+# executes 660.)
 FLOP_PER_SAMPLE = 662
 SFU_PER_SAMPLE = 13.2
 # The CUDA kernel headers (their code hash is printed with the results), and the ones the
@@ -87,20 +88,20 @@ TRAFFIC_HEADERS = ("bl_kernels.cuh", "bl_math.cuh", "bl_df64.cuh", "bl_internal.
 # fp64_instr: thread-level DFMA + DMUL + DADD instructions per unit from the same capture,
 # which gives the FP64 pipe's issue rate beside the algorithmic roofline.
 DRAM_PER_UNIT = {
-    # FP64 form, 7,845,751 attempts, the kernel of large waves at 15 CTAs an SM: 0.793 GB read +
-    # 5.434 GB written (the FP64 records and the stage derivatives, held in local memory)
-    "geodesic_fp64": {"src": "ad6fe3ed8e2f591c", "bytes": 793.7, "unit": "attempt",
+    # FP64 form, 7,845,751 attempts, the kernel of large waves at 15 CTAs an SM: 0.783 GB read +
+    # 5.461 GB written (the FP64 records and the stage derivatives, held in local memory)
+    "geodesic_fp64": {"src": "06a4bb7d91f68e31", "bytes": 795.9, "unit": "attempt",
                       "fp64_instr": 975.4},
-    # FP64 form, 18,372,204 samples, the transfer's launches: fp64_samples_kernel 4.179 + 3.872
+    # FP64 form, 18,372,204 samples, the transfer's launches: fp64_samples_kernel 4.182 + 3.878
     # GB (records, the stencils' field values, grid gathers, 193 B of results a plasma sample,
-    # spills) and transport_fp64_kernel 1.258 + 0.660 GB (records, those results, spills)
-    "transfer_fp64": {"src": "ad6fe3ed8e2f591c", "bytes": 542.6, "unit": "sample",
-                      "fp64_instr": 284.5},
-    # fast form, 7,845,744 attempts: 0.023 GB read + 1.134 GB written
-    "geodesic_df64": {"src": "ad6fe3ed8e2f591c", "bytes": 147.5, "unit": "attempt"},
-    # fast form on cell-layout grids, 18,372,183 samples: field mask 0.167 + 0.003 GB, samples
-    # 1.309 + 0.318, transport 0.640 + 0.003
-    "transfer_fp32": {"src": "ad6fe3ed8e2f591c", "bytes": 132.9, "unit": "sample"},
+    # spills) and transport_fp64_kernel 1.238 + 0.629 GB (records, those results, spills)
+    "transfer_fp64": {"src": "06a4bb7d91f68e31", "bytes": 540.3, "unit": "sample",
+                      "fp64_instr": 285.7},
+    # fast form, 7,845,744 attempts: 0.022 GB read + 1.134 GB written
+    "geodesic_df64": {"src": "06a4bb7d91f68e31", "bytes": 147.3, "unit": "attempt"},
+    # fast form on cell-layout grids, 18,372,183 samples: field mask 0.166 + 0.003 GB, samples
+    # 1.309 + 0.318, transport 0.640 + 0.004
+    "transfer_fp32": {"src": "06a4bb7d91f68e31", "bytes": 132.8, "unit": "sample"},
 }
 
 

@@ -2309,8 +2309,9 @@ int blacklight_trace_host_batch(int32_t n_images, const bl_camera_t* cams,
         if (r2 != 0) rc = r2;
     }
     // The scratch goes back to the memory pool after the wait, as in trace_impl: a wait after the
-    // free gives it back to the driver at once, and the next call maps it again (two 256^2 images:
-    // 22.0 ms a call with the wait last, 12.8 so)
+    // free gives it back to the driver at once, and the next call maps it again. Two 256^2 images:
+    // 10.1 ms a call back to back, 14.0 where the caller synchronises between two calls, which gives
+    // it back all the same (blacklight_set_memory_retention: 10.1 either way)
     cudaFreeAsync(dev, st);
     cudaError_t se = waited ? cudaSuccess : cudaStreamSynchronize(st);
     if (rc == 0 && se != cudaSuccess) rc = cuda_fail(se, "cudaStreamSynchronize");

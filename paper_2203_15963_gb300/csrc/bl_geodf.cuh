@@ -1,8 +1,8 @@
 // Double-float Dormand-Prince geodesics (the fast form, and the work-ordered queue's prediction).
 // Included by bl_kernels.cuh.
 //
-// What bounds it: instruction issue and fetch (two thirds of the issue slots with 12 resident
-// warps an SM; the FP32 pipe itself is under half used). sm_103a's packed FP32 instructions
+// What bounds it: instruction issue and dependent latency (57 % of the issue slots on one 256^2
+// image with at most 12 resident warps an SM, which its 152 registers allow). sm_103a's packed FP32 instructions
 // (fma/add/mul.f32x2) do two IEEE operations in one issue slot, so everything that is done alike
 // for two components is packed: (x, y), (k_x, k_y) and (z, k_z) in the stage, error and midpoint
 // sums, (x, y)-like pairs in the right-hand side. Each half of a packed operation is the scalar

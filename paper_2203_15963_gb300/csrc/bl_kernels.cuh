@@ -368,10 +368,12 @@ __global__ void cost_descs_kernel(const ImageDesc* __restrict__ src, ImageDesc* 
 }
 
 // The transfers' ray orders sort groups of G consecutive wave rays by their largest work: the
-// FP64 transport pass groups of a warp's 32 (neighbouring pixels of the geodesic queue, so a
-// warp keeps rays of similar paths through the plasma: 245.7 -> 240.5 ms against single rays
-// on the nine-image step), the FP32 transfer single rays (10.9 ms against 13.2 with groups:
-// its per-sample chain costs the same with or without plasma, and single rays balance better).
+// passes after a sample pass groups of a warp's 32 (neighbouring pixels of the geodesic queue, so
+// a warp keeps rays of similar paths through the plasma: FP64 transport 245.7 -> 240.5 ms against
+// single rays on the nine-image step, when both were slower), the single kernels of the
+// auxiliary images single rays (measured on the FP32 single kernel without them, 10.9 ms against
+// 13.2 with groups: its per-sample chain costs the same with or without plasma, and single rays
+// balance better).
 constexpr int kTransportGroup = 32;
 constexpr int kFusedGroup = 1;
 
@@ -753,9 +755,10 @@ __global__ void __launch_bounds__(128, BL_GEO_MIN_CTAS) geodesic_df_kernel(
 // further warp slows the ones there: a launch of few rays ends with its longest rays, which then
 // run at the pace of the crowd. So up to kSparse64Rays rays an SM a single CTA an SM works
 // through the queue (FP64, one 256^2 image: 22.2 ms against 28.5 at 3 CTAs and 33.9 at 16; mixed
-// 17.9 against 27.7), and up to kTwo64Rays two (mixed, two 201^2 images, 531 rays an SM: 22.7 ms
-// against 23.6 with one and 26.8 with three; two 256^2, 862: 27.2 / 33.3 / 32.0, FP64 35.5 / 41.7 /
-// 38.9; from 1192 to 2400 rays an SM two and three are within 4 % of each other either way). The
+// 17.9 against 27.7), and up to kTwo64Rays two (mixed, two 201^2 images, 531 rays an SM: 27.1 ms
+// against 33.5 with one and 29.9 with three; two 256^2, 862, with their prediction: 29.8 / 35.8 /
+// 33.1, FP64 38.5 / 44.8 / 40.1; from 1192 to 2400 rays an SM two and three are within 4 % of each
+// other either way). The
 // CTAs beyond those of an SM decide that for themselves, as a device block list's length is not
 // known to the host.
 #ifndef BL_GEO64_MIN_CTAS
@@ -1698,7 +1701,7 @@ __device__ __forceinline__ void transfer_body(const ImageDesc* __restrict__ imgs
 // (learned coefficients: from the model's outputs), the operations of the single kernel
 // (transfer_body) in its order. The row of the sample is asked for when the sample's record
 // arrives and read after the transport step. Bound by the latency of its serial chain of matrix
-// steps (nine 256^2 images 3.26 ms with 4 CTAs an SM; 3: 3.7, 5: 3.3, 6: 3.7).
+// steps (nine 256^2 images 3.2 ms with 4 CTAs an SM; 3: 3.7, 5: 3.3, 6: 3.7).
 template <bool kUnpol, bool kMlp>
 __device__ __forceinline__ void transport32_body(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
@@ -1865,11 +1868,12 @@ __global__ void __launch_bounds__(128, (kF & kFAux) ? 0 : BL_TR32_MIN_CTAS) tran
     }
     transfer_body<T, R, kF>(imgs, n_images, ray_begin, ray_end, hdr, pool, chunks, ctr, bs, side);
 }
-// Register cap and CTA size of the FP64 transfer kernel. Its FP64 arithmetic runs at 1/64 of
-// the FP32 rate with long dependent latencies, so resident warps matter more than spills to
-// L1: measured on the 9 x 256^2 step, 96 registers (20 warps an SM) 459 ms, 80: 441 ms, 72:
-// 429 ms, 64 (32 warps an SM): 405 ms, 56: 395 ms, 48 (42 warps an SM): 385 ms, 40: 373 ms,
-// 32 (64 warps, the SM's limit): 349 ms.
+// Register cap and CTA size of the FP64 single kernel, which now serves polarized images with
+// auxiliary images alone. The cap dates from when every FP64 transfer ran in it and its transport
+// matrix took twice the operations (nine 256^2 images without auxiliary images: 96 registers 459
+// ms, 64: 405, 48: 385, 32: 349). With auxiliary images and the closed matrix, the transfer of
+// three 256^2 images takes 119 ms at 32 registers, 115 at 40, 102 at 48, 86 at 64 and 84 at 96, of
+// one 49 to 62, 63, 61, 58 and 43; CTAs of 128 threads measure as 64 do.
 #ifndef BL_TR64_MAXNREG
 #define BL_TR64_MAXNREG 32
 #endif
@@ -2363,7 +2367,8 @@ __device__ __forceinline__ void transport_fp64_body(
 // CTAs of 128 threads an SM without spills up to kDeep64Rays rays an SM (three 256^2 images,
 // both transfer passes: 34.3 ms against 48.9), of which all but the first one or two of an SM leave
 // when the wave has few rays (one 256^2 image: 14.3 ms against 22.0 with all and 24.0 in the dense
-// shape; a 32^2 image 5.4 against 7.0; two 201^2 images 16.4 with two, 17.3 with one, 19.9). Nine images: 105 ms dense, 109 in the other shape.
+// shape; a 32^2 image 5.4 against 7.0; two 201^2 images 16.4 with two, 19.5 with one, 18.4 with
+// three). Nine images: 103 ms dense, 109 in the other shape.
 __global__ void __maxnreg__(BL_TRANSPORT64_MAXNREG) transport_fp64_kernel(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
         const RayHdr* __restrict__ hdr, const double* __restrict__ pool,
@@ -2386,7 +2391,7 @@ __global__ void __launch_bounds__(128, kTransport64WideCtas) transport64_wide_ke
 // intensity steps and, with auxiliary images, their accumulation, from the first pass's values; no
 // transport, so a record without plasma costs its flag. Few operations a sample in a serial chain:
 // latency-bound, so 4 CTAs of 128 threads an SM. 160^2 with
-// auxiliary images, both passes: 3.3 ms (1.3 samples, 2.0 here) against the single kernel's 15.3.
+// auxiliary images, both passes: 2.2 ms (1.3 samples, 0.9 here) against the single kernel's 15.3.
 template <bool kAux>
 __global__ void __launch_bounds__(128, 4) unpolarized64_kernel(
         const ImageDesc* __restrict__ imgs, int n_images, int64_t ray_begin, int64_t ray_end,
@@ -2457,9 +2462,10 @@ __global__ void __launch_bounds__(128, 4) unpolarized64_kernel(
 // the value before it. Each ray's farthest plasma sample and its number of plasma samples
 // (atomics, one a ray and batch; tfirst -1 and tnpl 0 beforehand) start and order the second pass.
 // Bound by instruction issue and the latency of the record and stencil reads: nine 256^2 images
-// 3.7 ms in 72 registers and 7 CTAs an SM (8 CTAs 3.8, 6: 3.9, 5: 4.4, 4: 5.0), the learned form at 1024^2 6.7 in
-// 64 and 8 CTAs (7: 7.0, 5: 7.2, 4: 9.0). Both passes: nine images 11.3 -> 7.0 ms, slow light at
-// 512^2 6.6 -> 3.4, learned without the model 20.1 -> 13.2.
+// 4.0 ms in 72 registers and 7 CTAs an SM (of 3.7 then: 8 CTAs 3.8, 6: 3.9, 5: 4.4, 4: 5.0), the
+// learned form at 1024^2 6.7 in 64 and 8 CTAs (7: 7.0, 5: 7.2, 4: 9.0). Both passes and the mask:
+// nine images 11.3 -> 7.4 ms, slow light at 512^2 6.6 -> 3.7, learned without the model 20.1 ->
+// 13.4.
 // ---------------------------------------------------------------------------------------
 struct Sample32Item {
     float* rec;
